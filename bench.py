@@ -65,12 +65,11 @@ FLOPS_BOND_NL = {1: 36.0, 2: 44.0}
 # ... and its per-step part when (xi, |xi|) come from the per-slot table and pass 1 leaves (e, 1/|Y|)
 # for pass 2 (rsqrt counted as one flop).
 FLOPS_BOND_NL_TABLED = {1: 29.0, 2: 19.0}
-# ... and its pair form, per directed bond: pass 1a forms the geometry, root, divide and failure test
-# once per bond, both entries' theta terms and the direction Y/|Y| (26 flop per pair without the
-# theta sum, + 2 x 2 for the two terms, + 3 for the direction: 16.5 per directed bond), 1b adds the
-# terms (1), pass 2 forms the coefficient from the tables and the force along the stored direction
-# (12).
-FLOPS_BOND_NL_PAIRS = {"k_pass1a_nlp": 16.5, "k_pass1b_nlp": 1.0, "k_pass2_nlp": 12.0}
+# ... and its pair form, per directed bond: pass 1a forms the displacement, Y and |Y|^2 - |xi|^2 (14 flop
+# per pair), the two series of the extension (24), and the direction, the theta term and the force
+# coefficient's term (8): 23 per directed bond; 1b adds the terms (1); pass 2 adds the dilatation part
+# to the stored coefficient and sums the force along the stored direction (9).
+FLOPS_BOND_NL_PAIRS = {"k_pass1a_nlp": 23.0, "k_pass1b_nlp": 1.0, "k_pass2_nlp": 9.0}
 # Algorithmic bytes per directed bond and per particle of each step kernel (the model above, 3D,
 # no body force): the pair form's pass 1 is split between its two kernels (1a: index, status read and
 # write, x and u; 1b: 1/m, theta and the row pointer), pass 2 is one kernel.

@@ -66,7 +66,8 @@ void free_build(pd_ctx* c) {
   c->bE = nullptr;
   c->bt = nullptr;
   c->bY = nullptr;
-  c->bX = nullptr;
+  c->bC = nullptr;
+  c->bX = c->bX2 = nullptr;
   c->lam = nullptr;
   c->gnew = c->gold = nullptr;
   c->adr_part = nullptr;

@@ -112,8 +112,12 @@ struct StepArgs {
   uint8_t* dirty;          // FP64 pair path: per slice, bS needs recomputing
   double2* bE;             // tabled nonlinear path: per slot (e, 1 / |Y|), written by pass 1 (bA = (xi, |xi|))
   double* bt;              // tabled nonlinear pair form: per slot V_j |xi| e, written by pass 1a
-  double4* bY;             // tabled nonlinear pair form: per slot (Y/|Y|, e), written by pass 1a
-  const double2* bX;       // tabled nonlinear pair form: per slot (|xi| V_j, V_j), built once
+  double4* bY;             // tabled nonlinear pair form: per slot (Y/|Y|, G (1/m_i + 1/m_j) V_j e), written by pass 1a
+  // tabled nonlinear pair form, built once: per slot (1/|xi|^2, 1/|xi|, s0 (2 + s0) |xi|^2,
+  // G (1/m_i + 1/m_j) V_j |xi|), |xi| V_j and |xi|^2 V_j
+  const double4* bC;
+  const double* bX;
+  const double* bX2;
   int expire;              // testing (PD_OPT_EXPIRE_WAITS): staged kernels skip their first copy
   double uscale;           // mixed path: the FP32 shadow holds u * uscale (1, or 1/Q for nonlinear bonds)
   int adr;                 // PD_SOLVER_ADR: pass 2 stores g = f + b in gnew instead of updating
@@ -211,8 +215,10 @@ struct pd_ctx {
   bool bs_stale = true;           // bS no longer matches the status bits (recomputed before a step)
   double2* bE = nullptr;          // nonlinear FP64: per-slot (e, 1/|Y|) of the current step
   double* bt = nullptr;           // nonlinear FP64 pair form: per-slot theta term V_j |xi| e
-  double4* bY = nullptr;          // nonlinear FP64 pair form: per-slot (Y/|Y|, e)
-  double2* bX = nullptr;          // nonlinear FP64 pair form: per-slot (|xi| V_j, V_j)
+  double4* bY = nullptr;          // nonlinear FP64 pair form: per-slot (Y/|Y|, force coefficient's e term)
+  double4* bC = nullptr;          // nonlinear FP64 pair form: per-slot constants of pass 1a (see StepArgs)
+  double* bX = nullptr;           // nonlinear FP64 pair form: per-slot |xi| V_j
+  double* bX2 = nullptr;          // nonlinear FP64 pair form: per-slot |xi|^2 V_j
   int bond_cache = 1;             // use the table in the FP64 path
   int pairs = 1;                  // FP64 tabled path: evaluate each bond once per pair (needs pairs_ok)
   int stage = 1;                  // mixed path: TMA-staged index streams (split 1)

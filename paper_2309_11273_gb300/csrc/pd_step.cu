@@ -560,38 +560,70 @@ __device__ __forceinline__ double flip_sign(double x) {
   return __longlong_as_double(__double_as_longlong(x) ^ (long long)0x8000000000000000ull);
 }
 
+// The nonlinear extension from t = (|Y|^2 - |xi|^2) / |xi|^2:  e / |xi| = sqrt(1 + t) - 1 and
+// |xi| / |Y| = 1 / sqrt(1 + t).  For |t| <= 2^-8 (stretches up to 0.2 %; a bond of the brittle bodies
+// breaks below that) both are their binomial series to degree 6, (sqrt(1 + t) - 1) / t and 1 / sqrt(1 + t)
+// cut below 2^-58 of their values: 12 FMAs, where the reciprocal square root and the division cost about
+// 25 FP64 instructions, which bound pass 1a.  A bond beyond that range takes the root and the division;
+// the choice is the bond's own, so its numbers do not depend on the warp it lands in.
+__device__ __forceinline__ bool nl_small(double t) {
+  return ((unsigned)__double2hiint(t) & 0x7fffffffu) < 0x3f700000u;  // |t| < 2^-8, false for a NaN
+}
+__device__ __forceinline__ void nl_series(double t, double& ext, double& inv) {
+  double a = fma(t, 33.0 / 2048.0, -21.0 / 1024.0);
+  double b = fma(t, 231.0 / 1024.0, -63.0 / 256.0);
+  a = fma(t, a, 7.0 / 256.0);
+  b = fma(t, b, 35.0 / 128.0);
+  a = fma(t, a, -5.0 / 128.0);
+  b = fma(t, b, -5.0 / 16.0);
+  a = fma(t, a, 1.0 / 16.0);
+  b = fma(t, b, 3.0 / 8.0);
+  a = fma(t, a, -1.0 / 8.0);
+  b = fma(t, b, -0.5);
+  a = fma(t, a, 0.5);
+  inv = fma(t, b, 1.0);
+  ext = t * a;
+}
+
 // Pair form of the tabled nonlinear pass 1.  Y and u_j - u_i change sign between the two entries of a
 // bond and |Y|^2 - |xi|^2 does not, so the failure test, e and 1/|Y| are the same numbers at both
 // ends: pass 1a forms them once, at the owned entry, clears both bits of a broken bond, and writes
-// (M = Y/|Y|, e) and the theta terms V_j |xi| e and V_i |xi| e of both entries (M changes sign);
-// pass 1b sums theta, and pass 2 takes the bond's direction and extension from the table instead of
-// recomputing Y from the displacements.  The root and the divide, most of the FP64 work of the
-// single pass, run once per bond.
-// UV: every body has one particle volume, so both entries' dilatation terms (V_j |xi| e and V_i |xi| e)
-// are the same product, formed once (bitwise the same values).
+// (M = Y/|Y|, its part G (1/m_i + 1/m_j) V_j e of the force coefficient of Eq 1.14) and the theta terms
+// V_j |xi| e of both entries (M changes sign); pass 1b sums theta, and pass 2 takes the bond's direction
+// and coefficient from the table instead of recomputing Y from the displacements.
+// Bound by the FP64 pipe (2 FMAs per clock and SM): 32 FP64 instructions per pair, with every factor
+// that does not depend on the displacement tabled (bC, bX2: 80 bytes read and 80 written per pair, 0.4
+// of the pipe's time at the HBM rate) and the failure threshold compared on the integer pipe.  Each lane
+// walks its own owned entries (own0 up to its family size): a common slot for the warp would run over
+// the union of the lanes' ranges, 1.16 times as many on a 101 x 50 x 49 block and 1.4 times on 60 x 30 x 25.
+// UV: every body has one particle volume, so both entries' terms are the same products, formed once.
 template <int DIM, int SPLIT, bool UV>
 __global__ void __launch_bounds__(512) k_pass1a_nlp(StepArgs a, const double4* __restrict__ disp) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (!t.active) return;  // whole warps; no block-wide barrier below
   const int b = a.body ? a.body[t.i] : 0;
-  const double s0nl = a.bp[b].s0nl;
   const bool can_break = a.bp[b].breaks != 0;
   const int own = a.own0[t.i], cnt = a.cnt[t.i];
-  const int k_lo = __reduce_min_sync(kFull, (unsigned)own);
-  const int k_hi = __reduce_max_sync(kFull, (unsigned)cnt);
+  const int nown = __reduce_max_sync(kFull, (unsigned)(cnt - own));
   const double4 ui = disp[t.i];
   uint32_t* bw = a.bits + (t.base >> 5);
   const int32_t* __restrict__ cl = a.col + t.base + t.lane;
   const int32_t* __restrict__ tw = a.twin + t.base + t.lane;
   const double4* __restrict__ ta = a.bA + t.base + t.lane;
-  for (int k = k_lo + t.sub; k < k_hi; k += SPLIT) {
-    const bool mine = k >= own && k < cnt;
+  const double4* __restrict__ tc = a.bC + t.base + t.lane;
+  const double* __restrict__ tx = a.bX2 + t.base + t.lane;
+  for (int m = t.sub; m < nown; m += SPLIT) {
+    const int k = own + m;
+    const bool mine = k < cnt;
     const int64_t e = t.base + t.lane + ((int64_t)k << 5);
-    double p = 0.0, yl2 = 0.0, xl = 0.0, vj = 0.0, yx = 0.0, yy = 0.0, yz = 0.0;
+    double p = 0.0, yx = 0.0, yy = 0.0, yz = 0.0, xv = 0.0;
+    double4 c = make_double4(0.0, 0.0, 0.0, 0.0);
     int32_t te = 0;
     if (mine) {
       const int32_t j = cl[(int64_t)k << 5];
       const double4 g = ta[(int64_t)k << 5];
+      c = tc[(int64_t)k << 5];
+      xv = tx[(int64_t)k << 5];
       const double4 uj = disp[j];
       te = tw[(int64_t)k << 5];
       const double hx = uj.x - ui.x, hy = uj.y - ui.y, hz = DIM == 3 ? uj.z - ui.z : 0.0;
@@ -600,30 +632,31 @@ __global__ void __launch_bounds__(512) k_pass1a_nlp(StepArgs a, const double4* _
       yz = g.z + hz;
       p = hx * (g.x + yx) + hy * (g.y + yy);
       if (DIM == 3) p = fma(hz, g.z + yz, p);
-      yl2 = yx * yx + yy * yy;
-      if (DIM == 3) yl2 = fma(yz, yz, yl2);
-      xl = g.w;
-      vj = uj.w;
     }
-    bool intact = mine && ((bw[k] >> t.lane) & 1u);  // this warp's owned bits change only here
-    if (a.check) {
-      const bool brk = intact && can_break && p >= s0nl * (xl * xl);
-      const unsigned m = __ballot_sync(kFull, brk);
-      if (m) {
-        if (t.lane == 0) atomicAnd(&bw[k], ~m);
-        if (brk) atomicAnd(a.bits + (te >> 5), ~(1u << (te & 31)));
-        intact = intact && !brk;
-      }
+    bool intact = mine && ((bw[k] >> t.lane) & 1u);  // an owned bit changes only here
+    if (a.check && intact && can_break && pd_ge_threshold(p, c.z)) {  // p >= s0 (2 + s0) |xi|^2
+      atomicAnd(&bw[k], ~(1u << t.lane));
+      atomicAnd(a.bits + (te >> 5), ~(1u << (te & 31)));
+      intact = false;
     }
     if (intact) {
-      const double ry = rsqrt(yl2);
-      const double ev = p / fma(yl2, ry, xl);
+      const double tt = p * c.x;  // (|Y|^2 - |xi|^2) / |xi|^2
+      double z, ry;               // e / |xi| and 1 / |Y|
+      if (nl_small(tt)) {
+        nl_series(tt, z, ry);
+        ry *= c.y;
+      } else {
+        double yl2 = yx * yx + yy * yy;
+        if (DIM == 3) yl2 = fma(yz, yz, yl2);
+        ry = rsqrt(yl2);
+        z = tt / fma(yl2 * ry, c.y, 1.0);
+      }
       const double mx = ry * yx, my = ry * yy, mz = ry * yz;  // M = Y / |Y| (Eq 1.13), -M at j
+      const double ev = c.w * z, tij = xv * z;                // Eq 1.14's and Eq 1.6's terms of entry (i, j)
       a.bY[e] = make_double4(mx, my, mz, ev);
-      a.bY[te] = make_double4(flip_sign(mx), flip_sign(my), flip_sign(mz), ev);
-      const double tij = (vj * xl) * ev;  // Eq 1.6 term of entry (i, j): w |xi| e V_j
+      a.bY[te] = make_double4(flip_sign(mx), flip_sign(my), flip_sign(mz), UV ? ev : a.bC[te].w * z);
       a.bt[e] = tij;
-      a.bt[te] = UV ? tij : (ui.w * xl) * ev;  // and of entry (j, i): w |xi| e V_i
+      a.bt[te] = UV ? tij : a.bX2[te] * z;  // and of entry (j, i)
     }
   }
 }
@@ -651,8 +684,9 @@ __global__ void __launch_bounds__(512) k_pass1b_nlp(StepArgs a, int write_theta)
 }
 
 // Pass 2 of the nonlinear pair form: Eq 1.14 for both ends along M (Eq 1.13),
-// f_i = sum_j [(K - G/3)(theta_i/m_i + theta_j/m_j) |xi| V_j + G (1/m_i + 1/m_j) e V_j] M, with
-// (M, e) from pass 1a and (|xi| V_j, V_j) from a per-slot table built once.
+// f_i = sum_j [(K - G/3)(theta_i/m_i + theta_j/m_j) |xi| V_j + G (1/m_i + 1/m_j) e V_j] M, with M and
+// the second term from pass 1a and |xi| V_j from a per-slot table built once: 5 FP64 instructions and 44
+// bytes per directed bond, whose times on their units nearly meet.
 template <int DIM, int SPLIT>
 __global__ void __launch_bounds__(512) k_pass2_nlp(StepArgs a, const double4* __restrict__ disp,
                                                     double4* __restrict__ disp_out) {
@@ -661,11 +695,11 @@ __global__ void __launch_bounds__(512) k_pass2_nlp(StepArgs a, const double4* __
   int b = 0;
   if (t.active) {
     b = a.body ? a.body[t.i] : 0;
-    const double2 ti = a.thm[t.i];
+    const double ti = a.thm[t.i].x;
     const uint32_t* __restrict__ bw = a.bits + (t.base >> 5);
     const int32_t* __restrict__ cl = a.col + t.base + t.lane;
     const double4* __restrict__ ty = a.bY + t.base + t.lane;
-    const double2* __restrict__ tx = a.bX + t.base + t.lane;
+    const double* __restrict__ tx = a.bX + t.base + t.lane;
     constexpr int U = 4;
     int32_t jn[U];
     uint32_t wn[U];
@@ -673,19 +707,19 @@ __global__ void __launch_bounds__(512) k_pass2_nlp(StepArgs a, const double4* __
     for (int k0 = t.sub; k0 < t.W; k0 += U * SPLIT) {
       uint32_t wd[U];
       double4 y[U];
-      double2 x[U], tj[U];
+      double x[U], tj[U];
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int k = min(k0 + u * SPLIT, t.W - 1);
         wd[u] = wn[u];
         y[u] = ty[(int64_t)k << 5];
         x[u] = tx[(int64_t)k << 5];
-        tj[u] = a.thm[jn[u]];
+        tj[u] = a.thm[jn[u]].x;
       }
       load_slots<U, SPLIT>(t, cl, bw, k0 + U * SPLIT, jn, wn);
 #pragma unroll
       for (int u = 0; u < U; ++u) {
-        double c = fma(ti.x + tj[u].x, x[u].x, (ti.y + tj[u].y) * (y[u].w * x[u].y));
+        double c = fma(ti + tj[u], x[u], y[u].w);
         c = ((wd[u] >> t.lane) & 1u) ? c : 0.0;  // broken and unused slots
         f[0] = fma(c, y[u].x, f[0]);
         f[1] = fma(c, y[u].y, f[1]);
@@ -700,19 +734,29 @@ __global__ void __launch_bounds__(512) k_pass2_nlp(StepArgs a, const double4* __
   }
 }
 
-// (|xi| V_j, V_j) per slot for k_pass2_nlp, |xi| as in k_bond_tables_nl.
+// Per-slot tables of the nonlinear pair form, |xi| and |xi|^2 as in k_bond_tables_nl and the threshold
+// with the rounding of the single pass (s0 (2 + s0) times |xi| |xi|): bC = (1 / |xi|^2, 1 / |xi|,
+// s0 (2 + s0) |xi|^2, G (1/m_i + 1/m_j) V_j |xi|), bX = |xi| V_j, bX2 = |xi|^2 V_j.
 template <int DIM>
-__global__ void k_bond_tables_nlp(StepArgs a, double2* __restrict__ bX) {
+__global__ void k_bond_tables_nlp(StepArgs a, double4* __restrict__ bC, double* __restrict__ bX,
+                                  double* __restrict__ bX2) {
   const SliceIdx t = slice_index<1>(a.n_pad, a.slice_ptr);
   if (!t.active) return;
+  const BodyDev& bp = a.bp[a.body ? a.body[t.i] : 0];
+  const double s0nl = bp.s0nl, G = bp.G, mi = a.mu[t.i];
   const double4 pi = a.pos[t.i];
   const double4 zero = make_double4(0.0, 0.0, 0.0, 0.0);
   for (int k = 0; k < t.W; ++k) {
     const int64_t e = t.base + t.lane + ((int64_t)k << 5);
-    const double4 pj = a.pos[a.col[e]];
+    const int32_t j = a.col[e];
+    const double4 pj = a.pos[j];
     double ex, ey, ez, d, q;
     bond_f64<DIM>(pi, pj, zero, zero, ex, ey, ez, d, q);
-    bX[e] = make_double2(sqrt(q) * pj.w, pj.w);
+    const double xl = sqrt(q);
+    const bool bond = q > 0.0;
+    bC[e] = make_double4(bond ? 1.0 / q : 0.0, bond ? 1.0 / xl : 0.0, s0nl * (xl * xl), G * (mi + a.mu[j]) * pj.w * xl);
+    bX[e] = xl * pj.w;
+    bX2[e] = q * pj.w;
   }
 }
 
@@ -2843,7 +2887,9 @@ StepArgs make_args(pd_ctx* c) {
   a.own0 = (c->bond_cache && c->pairs && c->pairs_ok && pairs_ready) ? c->own0 : nullptr;
   a.bt = c->bt;
   a.bY = c->bY;
+  a.bC = c->bC;
   a.bX = c->bX;
+  a.bX2 = c->bX2;
   a.twin = c->twin;
   a.dirty = c->dirty;
   a.bE = c->bond_cache ? c->bE : nullptr;
@@ -3161,12 +3207,14 @@ pd_status ensure_bond_cache(pd_ctx* c) {
       PD_CUDA(cudaMemsetAsync(c->bt, 0, sizeof(double) * ne, c->stream));
       if ((st = alloc(c, &c->bY, ne)) != PD_OK) return st;
       PD_CUDA(cudaMemsetAsync(c->bY, 0, sizeof(double4) * ne, c->stream));
+      if ((st = alloc(c, &c->bC, ne)) != PD_OK) return st;
+      if ((st = alloc(c, &c->bX2, ne)) != PD_OK) return st;
       if ((st = alloc(c, &c->bX, ne)) != PD_OK) return st;
       StepArgs ax = make_args(c);
       if (c->dim == 3)
-        k_bond_tables_nlp<3><<<grid, tb, 0, c->stream>>>(ax, c->bX);
+        k_bond_tables_nlp<3><<<grid, tb, 0, c->stream>>>(ax, c->bC, c->bX, c->bX2);
       else
-        k_bond_tables_nlp<2><<<grid, tb, 0, c->stream>>>(ax, c->bX);
+        k_bond_tables_nlp<2><<<grid, tb, 0, c->stream>>>(ax, c->bC, c->bX, c->bX2);
       PD_CUDA(cudaGetLastError());
     }
     StepArgs a = make_args(c);
