@@ -565,11 +565,13 @@ pd_status pd_set_option(pd_ctx* c, int32_t option, int64_t value) {
       if (value < 32 || value > 512 || value % 32) return fail(PD_ERR_ARG, "block must be a multiple of 32 in [32, 512]");
       if ((value / 32) % c->split) return fail(PD_ERR_ARG, "block warps must be a multiple of split");
       c->block = (int)value;
+      c->auto_map = false;
       break;
     case PD_OPT_SPLIT:
       if (value != 1 && value != 2 && value != 4) return fail(PD_ERR_ARG, "split must be 1, 2 or 4");
       if ((c->block / 32) % value) return fail(PD_ERR_ARG, "block warps must be a multiple of split");
       c->split = (int)value;
+      c->auto_map = false;
       break;
     case PD_OPT_BOND_CACHE:
       c->bond_cache = value != 0;
@@ -926,6 +928,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     const int cur0 = c->cur;
     const int64_t steps0 = c->steps;
     const bool skip0 = c->skip_next_check, pend0 = c->check_pending;
+    const bool auto0 = c->auto_map;
     const int prof0 = c->profile, chunk0 = c->graph_chunk, block0 = c->block, split0 = c->split;
     cudaStream_t s = c->stream;
     PD_CUDA(cudaMemcpyAsync(su, c->disp[cur0], sizeof(double4) * np, cudaMemcpyDeviceToDevice, s));
@@ -953,6 +956,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     };
     c->profile = 0;
     c->graph_chunk = 0;
+    c->auto_map = false;
     double best_ms = 1e300;
     const int blocks[] = {64, 128, 256, 512};
     const int splits[] = {1, 2, 4};
@@ -1014,6 +1018,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     c->block = block0;
     c->split = split0;
     c->lat_stage = stage0;
+    c->auto_map = auto0;
     if (st != PD_OK) return st;
     if (st2 != PD_OK) return st2;
     best_lat = best_ring;
@@ -1026,6 +1031,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
   }
   c->block = best_block;
   c->split = best_split;
+  c->auto_map = false;
   if (best_lat >= 0) c->lat_stage = best_lat;
   if (best_pairs >= 0) {
     if ((best_pairs != 0) != (c->pairs != 0)) c->bs_stale = true;  // as a PD_OPT_PAIRS switch

@@ -262,6 +262,7 @@ struct pd_ctx {
   int validate = 0;
   int block = 256;
   int split = 1;
+  bool auto_map = true;  // no mapping was chosen (PD_OPT_BLOCK, PD_OPT_SPLIT, pd_autotune): each kernel takes its own
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   pd::KernelTimes times;
   int64_t device_bytes = 0;
