@@ -73,6 +73,8 @@ void free_build(pd_ctx* c) {
   c->adr_part = nullptr;
   c->adr_st = nullptr;
   c->adr_first = nullptr;
+  c->bar = nullptr;
+  c->bar_base = 0;
   c->adr_restart = true;
   c->diag_theta = nullptr;
   c->diag_part = nullptr;
@@ -885,7 +887,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
   for (char* p = key; *p; ++p)
     if (*p == '\n' || *p == '|') *p = ' ';
   const char* cache = std::getenv("PD_AUTOTUNE_CACHE");
-  int best_block = -1, best_split = -1, best_pairs = -1, best_lat = -1;
+  int best_block = -1, best_split = -1, best_pairs = -1, best_lat = -1, best_auto = 0;
   if (cache) {
     if (FILE* f = std::fopen(cache, "r")) {
       char line[700];
@@ -893,12 +895,13 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
         char* bar = std::strchr(line, '|');
         if (!bar) continue;
         *bar = 0;
-        int b = 0, s = 0, pr = -1, rg = -1;
-        if (std::strcmp(line, key) == 0 && std::sscanf(bar + 1, "%d %d %d %d", &b, &s, &pr, &rg) >= 2) {
+        int b = 0, s = 0, pr = -1, rg = -1, am = 0;
+        if (std::strcmp(line, key) == 0 && std::sscanf(bar + 1, "%d %d %d %d %d", &b, &s, &pr, &rg, &am) >= 2) {
           best_block = b;
           best_split = s;
           best_pairs = pr;
           best_lat = rg;
+          best_auto = am;
         }
       }
       std::fclose(f);
@@ -956,7 +959,6 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     };
     c->profile = 0;
     c->graph_chunk = 0;
-    c->auto_map = false;
     double best_ms = 1e300;
     const int blocks[] = {64, 128, 256, 512};
     const int splits[] = {1, 2, 4};
@@ -969,40 +971,52 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     const int stage0 = c->lat_stage;
-    const int nrings = c->lattice ? 4 : 1;
     int best_ring = stage0;
-    for (int bl : blocks) {
+    struct Candidate {
+      int block, split, pairs, ring;
+      bool automatic;
+    };
+    std::vector<Candidate> cands;
+    c->auto_map = true;
+    c->pairs = pairs0;
+    // the automatic choice, where it is more than launch shapes: the resident step kernel
+    if (resident_plan(c).split) cands.push_back({block0, split0, pairs0, stage0, true});
+    for (int bl : blocks)
       for (int sp : splits) {
         if ((bl / 32) % sp) continue;
         if (c->lattice && sp != 1) continue;  // the lattice kernels run one warp per slice
-        for (int po = 0; po < (try_pairs ? 2 : 1) * nrings; ++po) {
-          c->block = bl;
-          c->split = sp;
-          c->pairs = try_pairs ? pair_opts[po] : pairs0;
-          if (c->lattice) c->lat_stage = po;  // the staging ring of the lattice kernels
-          if ((st = restore()) != PD_OK) break;
-          run_steps(c, 1);  // warm-up
-          cudaEventRecord(e0, s);
-          st = run_steps(c, trial_steps);
-          cudaEventRecord(e1, s);
-          if (st != PD_OK) break;
-          if (cudaEventSynchronize(e1) != cudaSuccess) {
-            st = cuda_fail(cudaGetLastError(), "autotune trial");
-            break;
-          }
-          float ms = 0.0f;
-          cudaEventElapsedTime(&ms, e0, e1);
-          if (ms < best_ms) {
-            best_ms = ms;
-            best_block = bl;
-            best_split = sp;
-            best_pairs = c->pairs;
-            best_ring = c->lat_stage;
-          }
-        }
-        if (st != PD_OK) break;
+        if (c->lattice)
+          for (int ring = 0; ring < 4; ++ring) cands.push_back({bl, sp, pairs0, ring, false});
+        else
+          for (int po = 0; po < (try_pairs ? 2 : 1); ++po)
+            cands.push_back({bl, sp, try_pairs ? pair_opts[po] : pairs0, stage0, false});
       }
+    for (const Candidate& cd : cands) {
+      c->auto_map = cd.automatic;
+      c->block = cd.block;
+      c->split = cd.split;
+      c->pairs = cd.pairs;
+      c->lat_stage = cd.ring;  // the staging ring of the lattice kernels
+      if ((st = restore()) != PD_OK) break;
+      run_steps(c, 1);  // warm-up
+      cudaEventRecord(e0, s);
+      st = run_steps(c, trial_steps);
+      cudaEventRecord(e1, s);
       if (st != PD_OK) break;
+      if (cudaEventSynchronize(e1) != cudaSuccess) {
+        st = cuda_fail(cudaGetLastError(), "autotune trial");
+        break;
+      }
+      float ms = 0.0f;
+      cudaEventElapsedTime(&ms, e0, e1);
+      if (ms < best_ms) {
+        best_ms = ms;
+        best_block = cd.block;
+        best_split = cd.split;
+        best_pairs = cd.pairs;
+        best_ring = cd.ring;
+        best_auto = cd.automatic ? 1 : 0;
+      }
     }
     c->pairs = pairs0;
     cudaEventDestroy(e0);
@@ -1024,14 +1038,14 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     best_lat = best_ring;
     if (cache && best_block > 0) {
       if (FILE* f = std::fopen(cache, "a")) {
-        std::fprintf(f, "%s|%d %d %d %d\n", key, best_block, best_split, best_pairs, best_ring);
+        std::fprintf(f, "%s|%d %d %d %d %d\n", key, best_block, best_split, best_pairs, best_ring, best_auto);
         std::fclose(f);
       }
     }
   }
   c->block = best_block;
   c->split = best_split;
-  c->auto_map = false;
+  c->auto_map = best_auto != 0;
   if (best_lat >= 0) c->lat_stage = best_lat;
   if (best_pairs >= 0) {
     if ((best_pairs != 0) != (c->pairs != 0)) c->bs_stale = true;  // as a PD_OPT_PAIRS switch

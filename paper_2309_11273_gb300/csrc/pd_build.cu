@@ -778,6 +778,11 @@ pd_status create(pd_ctx** out, int32_t nbodies, const pd_params* prm, const int6
     c->own_stream = true;
   }
 
+  int coop = 0, sms = 0;
+  if (cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, c->device) == cudaSuccess && coop &&
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device) == cudaSuccess)
+    c->sms = sms;
+
   // Internal order inside each body (bodies stay contiguous in their given order):
   //   PD_ORDER_MORTON: Morton curve of the coordinates;
   //   PD_ORDER_BRICKS: bricks of 32 x 4 x 4 (3D) / 32 x 8 (2D) points of the body's typical spacing

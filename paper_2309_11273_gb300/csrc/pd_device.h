@@ -1,0 +1,179 @@
+// Device helpers shared by the step kernels (pd_step.cu) and the resident step kernel (pd_resident.cu).
+#pragma once
+
+#include <type_traits>
+
+#include "pd_internal.h"
+#include "pd_order.h"
+
+namespace pd {
+namespace {
+
+constexpr unsigned kFull = 0xffffffffu;
+
+struct SliceIdx {
+  int64_t i;
+  int64_t base;
+  int W;
+  int lane;
+  int sub;
+  bool active;
+};
+
+template <int SPLIT>
+__device__ __forceinline__ SliceIdx slice_index(int64_t n_pad, const int64_t* __restrict__ slice_ptr) {
+  SliceIdx r;
+  const int64_t gwarp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  r.lane = threadIdx.x & 31;
+  r.sub = (int)(gwarp % SPLIT);
+  const int64_t s = gwarp / SPLIT;
+  r.i = s * 32 + r.lane;
+  r.active = r.i < n_pad;  // n_pad is a multiple of 32: uniform over the warp
+  r.base = 0;
+  r.W = 0;
+  if (r.active) {
+    r.base = slice_ptr[s];
+    r.W = (int)((slice_ptr[s + 1] - r.base) >> 5);
+  }
+  return r;
+}
+
+// Partial sums of the SPLIT warps sharing a slice, combined by the first warp (fixed order).
+template <int SPLIT, int NC, class T>
+__device__ __forceinline__ void split_reduce(T (&v)[NC]) {
+  if (SPLIT == 1) return;
+  extern __shared__ unsigned char smem_raw[];
+  T* red = reinterpret_cast<T*>(smem_raw);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) red[c * blockDim.x + threadIdx.x] = v[c];
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w % SPLIT == 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      T s = red[c * blockDim.x + w * 32 + lane];
+#pragma unroll
+      for (int q = 1; q < SPLIT; ++q) s += red[c * blockDim.x + (w + q) * 32 + lane];
+      v[c] = s;
+    }
+  }
+}
+
+// The sums of the tabled FP64 kernels run in four parts, slot k in part k mod 4, combined as (0 + 2) +
+// (1 + 3) whatever the number of warps that share a slice: a warp holds 4 / SPLIT of them, so the result
+// is bitwise the same for every split (and four independent chains of FP64 additions are shorter).
+template <int SPLIT, int NC>
+__device__ __forceinline__ void parts_sum(const double (&p)[NC][4 / SPLIT], double (&v)[NC]) {
+#pragma unroll
+  for (int c = 0; c < NC; ++c) {
+    if constexpr (SPLIT == 1) v[c] = (p[c][0] + p[c][2]) + (p[c][1] + p[c][3]);
+    else if constexpr (SPLIT == 2) v[c] = p[c][0] + p[c][1];
+    else v[c] = p[c][0];
+  }
+}
+// ... and across the warps of the slice (their parts combined by the first warp).
+template <int SPLIT, int NC>
+__device__ __forceinline__ void parts_across(double (&v)[NC]) {
+  if (SPLIT == 1) return;
+  extern __shared__ unsigned char smem_raw[];
+  double* red = reinterpret_cast<double*>(smem_raw);
+#pragma unroll
+  for (int c = 0; c < NC; ++c) red[c * blockDim.x + threadIdx.x] = v[c];
+  __syncthreads();
+  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (w % SPLIT == 0) {
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+      const double* r = red + c * blockDim.x + w * 32 + lane;
+      v[c] = SPLIT == 2 ? r[0] + r[32] : (r[0] + r[64]) + (r[32] + r[96]);
+    }
+  }
+}
+
+// bS_i from the status bits and bB, in slot order (so bS is a function of the bits alone).  The
+// words are read through L2: other warps of the block may have just written them.
+__device__ __forceinline__ void bond_sum_row(const StepArgs& a, const SliceIdx& t) {
+  const uint32_t* bw = a.bits + (t.base >> 5);
+  const double4* tb = a.bB + t.base + t.lane;
+  double sx = 0.0, sy = 0.0, sz = 0.0;
+  for (int k = 0; k < t.W; ++k) {
+    if ((__ldcg(bw + k) >> t.lane) & 1u) {
+      const double4 g = tb[(int64_t)k << 5];
+      sx += g.x;
+      sy += g.y;
+      sz += g.z;
+    }
+  }
+  a.bS[t.i] = make_double4(sx, sy, sz, 0.0);
+}
+
+// Relaxation solver: a slice's sums of u (k u) and u u over its free particles' components, k =
+// -(g - g_prev) / (lambda v), in lane 0 of the warp.
+__device__ __forceinline__ double2 adr_terms(bool free, const double4& u, const double4& v, const double4& g,
+                                             const double4& gp, double lam) {
+  double num = 0.0, den = 0.0;
+  if (free) {
+    const double uu[3] = {u.x, u.y, u.z}, vv[3] = {v.x, v.y, v.z}, gg[3] = {g.x, g.y, g.z}, go[3] = {gp.x, gp.y, gp.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double kk = vv[k] != 0.0 ? -(gg[k] - go[k]) / (lam * vv[k]) : 0.0;
+      num += uu[k] * kk * uu[k];
+      den += uu[k] * uu[k];
+    }
+  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    num += __shfl_down_sync(kFull, num, o);
+    den += __shfl_down_sync(kFull, den, o);
+  }
+  return make_double2(num, den);
+}
+
+// v^{n+1/2} of one component: ((2 - c) v^{n-1/2} + 2 g / lambda) / (2 + c), from rest on a start g / (2 lambda),
+// with the stored reciprocals 1 / lambda and 1 / (2 + c) (the contraction written out: both kernels that
+// relax round alike).
+__device__ __forceinline__ double adr_velocity(double v, double g, double inv_lam, double c, double inv_2c, bool start) {
+  return start ? g * (0.5 * inv_lam) : fma(2.0 - c, v, g * (2.0 * inv_lam)) * inv_2c;
+}
+
+// The damping c = 2 sqrt(u.k.u / u.u) (0 unless both are positive) and 1 / (2 + c) from the slices' sums,
+// for every thread of the block: 1024 strided sums, combined by warps of them, in the same order whatever
+// the block's size.
+__device__ __forceinline__ double2 adr_damping(const double2* part, int64_t nslices) {
+  __shared__ double wn[32], wd[32];
+  __shared__ double2 c_s;
+  for (int v = threadIdx.x; v < 1024; v += blockDim.x) {  // whole warps
+    double num = 0.0, den = 0.0;
+    for (int64_t k = v; k < nslices; k += 1024) {
+      num += part[k].x;
+      den += part[k].y;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_down_sync(kFull, num, o);
+      den += __shfl_down_sync(kFull, den, o);
+    }
+    if ((v & 31) == 0) {
+      wn[v >> 5] = num;
+      wd[v >> 5] = den;
+    }
+  }
+  __syncthreads();
+  if (threadIdx.x < 32) {
+    double num = wn[threadIdx.x], den = wd[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      num += __shfl_down_sync(kFull, num, o);
+      den += __shfl_down_sync(kFull, den, o);
+    }
+    if (threadIdx.x == 0) {
+      const double c = (den > 0.0 && num > 0.0) ? 2.0 * sqrt(num / den) : 0.0;
+      c_s = make_double2(c, 1.0 / (2.0 + c));
+    }
+  }
+  __syncthreads();
+  return c_s;
+}
+
+}  // namespace
+}  // namespace pd

@@ -228,7 +228,7 @@ struct pd_ctx {
   double2* lam = nullptr;         // ADR fictitious density (lambda_i, 1 / lambda_i)
   double4* gnew = nullptr;        // ADR g^n (force density incl. body force)
   double4* gold = nullptr;        // ADR g^{n-1}
-  double2* adr_part = nullptr;    // ADR per-block partial sums (u.k.u, u.u)
+  double2* adr_part = nullptr;    // ADR per-slice partial sums (u.k.u, u.u)
   double4* adr_st = nullptr;      // ADR (c^n, start flag, 1 / (2 + c^n)) of the current iteration
   int* adr_first = nullptr;       // ADR: 1 = the next iteration starts from rest
   double* diag_theta = nullptr;   // pd_get_stats: theta at the current state
@@ -257,6 +257,9 @@ struct pd_ctx {
   double rate = 0.0;                      // prescribed rotation rate
   double bc_point[3] = {0, 0, 0}, bc_dir[3] = {0, 0, 0};
   // options
+  int sms = 0;                  // SMs of the device; 0: no cooperative launch (the resident step kernel is off)
+  unsigned* bar = nullptr;      // resident step kernel: grid barrier (arrivals, abort)
+  unsigned bar_base = 0;        // ... arrivals enqueued so far
   int graph_chunk = 100;
   int profile = 0;
   int validate = 0;
@@ -312,6 +315,16 @@ pd_status max_abs_u(pd_ctx* c, double* out, int* nonfinite);
 pd_status check_device_error(pd_ctx* c);
 pd_status run_steps(pd_ctx* c, int64_t nsteps);
 pd_status read_profile(pd_ctx* c);
+// The resident step kernel (pd_resident.cu): all steps of a call in one cooperative launch, for bodies
+// that fit the chip in one wave.
+struct ResidentPlan {
+  int split = 0;  // warps per slice; 0: the pass kernels take the steps
+  int block = 0;
+  unsigned grid = 0;
+  bool pair = false;  // pass 1 in its pair form
+};
+ResidentPlan resident_plan(const pd_ctx* c);
+pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done);
 }  // namespace pd
 
 #define PD_CUDA(call)                                        \

@@ -1,0 +1,411 @@
+// The resident step kernel: bodies that fit the chip in one wave take all the steps of a pd_step call in
+// one cooperative launch.
+//
+// On a body of up to about a hundred thousand particles a step of the pass kernels is shorter than what
+// surrounds it: three launches (six with the relaxation solver), each with its ramp up and its last warps,
+// and per launch the chain index -> gather -> sum of a slice's row.  Here one block per SM holds its
+// slices for the whole call; the displacements and velocities of its particles stay in registers, and the
+// passes are separated by a grid barrier (about 1.5 us) instead of a launch.  The arithmetic is that of
+// k_pass1a_f64p / k_pass1b_f64p / k_pass2_f64t (pair form) or k_pass1_f64t / k_pass2_f64t, with the same
+// order of every sum (parts_sum), so the results are bitwise those of the pass kernels.
+//
+// The barrier is an arrival counter in the context's memory that only grows; every wait is bounded (1 s of
+// the GPU's global timer), and when one expires the block sets the context's error word and an abort word
+// that ends every other wait, and all blocks return: the next pd_sync / pd_get_* reports PD_ERR_TIMEOUT.
+#include <algorithm>
+
+#include "pd_internal.h"
+#include "pd_device.h"
+
+namespace pd {
+namespace {
+
+struct ResidentArgs {
+  double4* disp;       // u^n
+  double4* disp_out;   // the other displacement buffer
+  int nsteps;
+  int check0;          // the failure check at the head of the first step
+  int64_t step0;       // index of the first step
+  unsigned* bar;       // [0] arrivals, [1] abort
+  unsigned bar_base;   // arrivals before this launch
+  int uv;              // every body has one particle volume
+  // relaxation solver
+  double4* gold;
+  const double2* lam;
+  double2* part;       // per slice (u.k.u, u.u)
+  int* first;
+};
+
+constexpr unsigned kPollLimit = 1u << 26;
+constexpr unsigned long long kBarrierNs = 1000000000ull;
+
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ unsigned long long timer_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// All blocks of the grid: what any of them wrote before is visible to all of them after.  The fence
+// after the wait drops this SM's cached lines, so plain loads see the other SMs' stores.  False when the
+// wait expired or another block gave up.
+__device__ __forceinline__ bool grid_barrier(const StepArgs& a, const ResidentArgs& r, unsigned& target) {
+  __shared__ int ok_s;
+  target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int ok = 1;
+    __threadfence();
+    // testing (PD_OPT_EXPIRE_WAITS): block 0 never arrives
+    if (!(a.expire && blockIdx.x == 0)) asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(r.bar) : "memory");
+    if ((int)(ld_relaxed(r.bar) - target) < 0) {
+      const unsigned long long t0 = timer_ns();
+      for (unsigned it = 1; (int)(ld_relaxed(r.bar) - target) < 0; ++it) {
+        if ((it & 63u) == 0u &&
+            (ld_relaxed(r.bar + 1) != 0u || timer_ns() - t0 > kBarrierNs || it > kPollLimit)) {
+          ok = 0;
+          atomicExch(r.bar + 1, 1u);
+          atomicExch(&a.counters[4], 1ull);
+          break;
+        }
+      }
+    }
+    __threadfence();
+    ok_s = ok;
+  }
+  __syncthreads();
+  return ok_s != 0;
+}
+
+// PAIR: pass 1 in its pair form (fewer FP64 instructions, one barrier more).  MAXT: largest block; its
+// registers bound the slots in flight U.
+template <int DIM, int SPLIT, bool PAIR, bool ADR, int MAXT>
+__global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r) {
+  constexpr int P = 4 / SPLIT;
+  constexpr int U = MAXT > 512 ? 2 : 4;
+  constexpr int H = P > U ? P / U : 1;
+  if (ld_relaxed(r.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
+  unsigned target = r.bar_base;
+  const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
+  const bool lead = t.active && t.sub == 0;
+  const int64_t i = t.active ? t.i : 0, s = i >> 5;
+  const int b = t.active && a.body ? a.body[i] : 0;
+  const BodyDev& bp = a.bp[b];
+  const bool can_break = bp.breaks != 0;
+  const int own = t.active ? a.own0[i] : 0, cnt = t.active ? a.cnt[i] : 0;
+  const int nown = __reduce_max_sync(kFull, (unsigned)(cnt - own));
+  uint32_t* bw = a.bits + (t.base >> 5);
+  const int32_t* cl = a.col + t.base + t.lane;
+  const int32_t* tw = a.twin + t.base + t.lane;
+  const double4* ta = a.bA + t.base + t.lane;
+  const double4* tb = a.bB + t.base + t.lane;
+  double* td = a.bd + t.base + t.lane;
+  double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u, gold = u;
+  double2 lam = make_double2(0.0, 0.0);
+  double th = 0.0;
+  bool start = false;
+  const uint8_t fl = lead && a.flag ? a.flag[i] : (uint8_t)0;
+  const double4 bb = lead && a.bacc ? a.bacc[i] : make_double4(0.0, 0.0, 0.0, 0.0);
+  if (lead) {
+    u = r.disp[i];
+    v = a.vel[i];
+    if (ADR) {
+      gold = r.gold[i];
+      lam = r.lam[i];
+      start = *r.first != 0;
+    }
+    if (a.dirty[s]) {  // bonds broken by a check between calls
+      bond_sum_row(a, t);
+      __syncwarp();
+      if (t.lane == 0) a.dirty[s] = 0;
+    }
+  }
+  const double vi = t.active ? a.pos[i].w : 0.0;
+  for (int step = 0; step < r.nsteps; ++step) {
+    const double4* disp = (step & 1) ? r.disp_out : r.disp;
+    double4* disp_out = (step & 1) ? r.disp : r.disp_out;
+    const bool check = (step > 0 || r.check0) && can_break;
+    double sum[2] = {0.0, 0.0}, part1[1][P] = {};
+    // ---- pass 1
+    if (PAIR) {
+      if (t.active) {
+        const double4 ui = disp[i];
+        for (int m0 = t.sub; m0 < nown; m0 += U * SPLIT) {
+          int32_t j[U], te[U];
+          double4 g[U], uj[U];
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            const int k = min(own + m0 + q * SPLIT, max(cnt - 1, 0));
+            j[q] = cl[(int64_t)k << 5];
+            g[q] = ta[(int64_t)k << 5];
+            te[q] = tw[(int64_t)k << 5];
+          }
+#pragma unroll
+          for (int q = 0; q < U; ++q) uj[q] = disp[j[q]];
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            const int k = own + m0 + q * SPLIT;
+            if (k >= cnt) continue;
+            double d = g[q].x * (uj[q].x - ui.x) + g[q].y * (uj[q].y - ui.y);
+            if (DIM == 3) d = fma(g[q].z, uj[q].z - ui.z, d);
+            td[(int64_t)k << 5] = d;
+            a.bd[te[q]] = d;
+            if (check && ((bw[k] >> t.lane) & 1u) && pd_ge_threshold(d, g[q].w)) {  // d >= s0 |xi|^2
+              atomicAnd(&bw[k], ~(1u << t.lane));
+              atomicAnd(a.bits + (te[q] >> 5), ~(1u << (te[q] & 31)));
+              a.dirty[s] = 1;
+              a.dirty[j[q] >> 5] = 1;
+            }
+          }
+        }
+      }
+      if (!grid_barrier(a, r, target)) return;
+      if (t.active) {
+        for (int k0 = t.sub; k0 < t.W; k0 += 4) {  // slots k0, k0 + SPLIT, ...: the sum's parts
+#pragma unroll
+          for (int q = 0; q < P; ++q) {
+            const int k = k0 + q * SPLIT;
+            const double vj = r.uv ? vi : disp[cl[(int64_t)k << 5]].w;
+            if ((bw[k] >> t.lane) & 1u) part1[0][q] = fma(vj, td[(int64_t)k << 5], part1[0][q]);
+          }
+        }
+      }
+    } else if (t.active) {
+      const double4 ui = disp[i];
+      for (int kb = t.sub; kb < t.W; kb += H * U * SPLIT) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int k0 = kb + h * U * SPLIT;
+          uint32_t wd[U];
+          double4 g[U], uj[U];
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            const int k = min(k0 + q * SPLIT, t.W - 1);
+            wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
+            g[q] = ta[(int64_t)k << 5];
+            uj[q] = disp[cl[(int64_t)k << 5]];
+          }
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            double d = g[q].x * (uj[q].x - ui.x) + g[q].y * (uj[q].y - ui.y);
+            if (DIM == 3) d = fma(g[q].z, uj[q].z - ui.z, d);
+            const int k = k0 + q * SPLIT;
+            if (k < t.W) td[(int64_t)k << 5] = d;
+            bool intact = (wd[q] >> t.lane) & 1u;
+            const unsigned m = __ballot_sync(kFull, check && intact && pd_ge_threshold(d, g[q].w));
+            if (m) {
+              if ((m >> t.lane) & 1u) intact = false;
+              if (t.lane == 0) bw[k] = wd[q] & ~m;
+              sum[1] = 1.0;
+            }
+            part1[0][(h * U + q) % P] = fma(intact ? uj[q].w : 0.0, d, part1[0][(h * U + q) % P]);
+          }
+        }
+      }
+      __syncwarp();
+    }
+    double th1[1];
+    parts_sum<SPLIT, 1>(part1, th1);
+    sum[0] = th1[0];
+    parts_across<SPLIT, 2>(sum);
+    if (lead) {
+      th = a.aA[i] * sum[0];
+      const double mu = a.mu[i];
+      a.thm[i] = make_double2(bp.Kp * (th * mu), bp.G * mu);
+      if (PAIR ? a.dirty[s] != 0 : sum[1] != 0.0) {  // uniform over the warp
+        bond_sum_row(a, t);
+        __syncwarp();
+        if (PAIR && t.lane == 0) a.dirty[s] = 0;
+      }
+    }
+    if (!grid_barrier(a, r, target)) return;
+    // ---- pass 2
+    double f[3], part[3][P] = {};
+    if (t.active) {
+      for (int kb = t.sub; kb < t.W; kb += H * U * SPLIT) {
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+          const int k0 = kb + h * U * SPLIT;
+          uint32_t wd[U];
+          double4 g[U];
+          double d[U], tj[U];
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            const int k = min(k0 + q * SPLIT, t.W - 1);
+            wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
+            g[q] = tb[(int64_t)k << 5];
+            d[q] = td[(int64_t)k << 5];
+            tj[q] = a.thm[cl[(int64_t)k << 5]].x;
+          }
+#pragma unroll
+          for (int q = 0; q < U; ++q) {
+            double c = fma(g[q].w, d[q], tj[q]);
+            c = ((wd[q] >> t.lane) & 1u) ? c : 0.0;
+            const int n = (h * U + q) % P;
+            part[0][n] = fma(c, g[q].x, part[0][n]);
+            part[1][n] = fma(c, g[q].y, part[1][n]);
+            if (DIM == 3) part[2][n] = fma(c, g[q].z, part[2][n]);
+          }
+        }
+      }
+    }
+    parts_sum<SPLIT, 3>(part, f);
+    parts_across<SPLIT, 3>(f);
+    if (lead) {
+      const double ti = a.thm[i].x;
+      const double4 S = a.bS[i];
+      f[0] = fma(ti, S.x, f[0]);
+      f[1] = fma(ti, S.y, f[1]);
+      f[2] = fma(ti, S.z, f[2]);
+    }
+    double2 c = make_double2(0.0, 0.0);
+    if (ADR) {  // g = f + b, and this slice's part of the Rayleigh quotient
+      if (lead) {
+        f[0] += bb.x;
+        f[1] += bb.y;
+        f[2] += bb.z;
+        const double2 sums = adr_terms(fl == 0 && lam.x > 0.0, u, v, make_double4(f[0], f[1], f[2], 0.0), gold, lam.x);
+        if (t.lane == 0) r.part[s] = sums;
+      }
+      if (!grid_barrier(a, r, target)) return;
+      c = adr_damping(r.part, a.n_pad >> 5);
+    }
+    // ---- update (as update() and k_adr_update)
+    if (lead) {
+      if (fl == 0) {
+        if (ADR) {
+          if (lam.x > 0.0) {
+            v.x = adr_velocity(v.x, f[0], lam.y, c.x, c.y, start);
+            v.y = adr_velocity(v.y, f[1], lam.y, c.x, c.y, start);
+            v.z = adr_velocity(v.z, f[2], lam.y, c.x, c.y, start);
+            u.x = u.x + v.x;
+            u.y = u.y + v.y;
+            u.z = u.z + v.z;
+          } else {
+            v = make_double4(0.0, 0.0, 0.0, 0.0);
+          }
+        } else {
+          v.x = v.x + bp.dt * ((f[0] + bb.x) * bp.inv_rho);
+          v.y = v.y + bp.dt * ((f[1] + bb.y) * bp.inv_rho);
+          v.z = v.z + bp.dt * ((f[2] + bb.z) * bp.inv_rho);
+          u.x = u.x + bp.dt * v.x;
+          u.y = u.y + bp.dt * v.y;
+          u.z = u.z + bp.dt * v.z;
+        }
+      } else if (fl == 1) {
+        u = make_double4(0.0, 0.0, 0.0, u.w);
+        v = make_double4(0.0, 0.0, 0.0, 0.0);
+      } else {
+        const double t1 = (double)(r.step0 + step + 1) * bp.dt;
+        const double4 g = a.gvec[i];
+        const double rt = bp.rate * t1;
+        u = make_double4(rt * g.x, rt * g.y, rt * g.z, u.w);
+        v = make_double4(bp.rate * g.x, bp.rate * g.y, bp.rate * g.z, 0.0);
+      }
+      disp_out[i] = u;  // .w carries V_i unchanged
+      if (ADR) gold = make_double4(f[0], f[1], f[2], 0.0);
+      start = false;
+    }
+    if (step + 1 < r.nsteps && !grid_barrier(a, r, target)) return;
+  }
+  if (lead) {
+    a.vel[i] = v;
+    a.theta[i] = th;
+    if (ADR) r.gold[i] = gold;
+    if (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z)) atomicExch(&a.counters[5], 1ull);
+  }
+  if (blockIdx.x == 0 && threadIdx.x == 0) {
+    *a.d_step = r.step0 + r.nsteps - 1;
+    if (ADR) *r.first = 0;  // every block read it before its first barrier
+  }
+}
+
+template <int DIM, int SPLIT, bool PAIR, int MAXT>
+cudaError_t launch(pd_ctx* c, StepArgs a, ResidentArgs r, unsigned grid, int block) {
+  void* args[] = {&a, &r};
+  const size_t sm = SPLIT > 1 ? (size_t)block * 3 * sizeof(double) : 0;
+  const void* k = a.adr ? (const void*)k_resident<DIM, SPLIT, PAIR, true, MAXT>
+                        : (const void*)k_resident<DIM, SPLIT, PAIR, false, MAXT>;
+  return cudaLaunchCooperativeKernel(k, dim3(grid), dim3((unsigned)block), args, sm, c->stream);
+}
+
+template <int DIM, int SPLIT>
+cudaError_t launch_form(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, unsigned grid, int block, bool pair) {
+  if (block > 512) return launch<DIM, SPLIT, true, 768>(c, a, r, grid, block);
+  return pair ? launch<DIM, SPLIT, true, 512>(c, a, r, grid, block) : launch<DIM, SPLIT, false, 512>(c, a, r, grid, block);
+}
+
+template <int DIM>
+cudaError_t launch_split(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, unsigned grid, int block, int split,
+                         bool pair) {
+  if (split == 4) return launch_form<DIM, 4>(c, a, r, grid, block, pair);
+  if (split == 2) return launch_form<DIM, 2>(c, a, r, grid, block, pair);
+  return launch_form<DIM, 1>(c, a, r, grid, block, pair);
+}
+
+}  // namespace
+
+ResidentPlan resident_plan(const pd_ctx* c) {
+  ResidentPlan p;
+  if (!c->auto_map || c->precision != PD_FP64 || c->kin != PD_LINEARIZED || !c->bond_cache || !c->pairs || !c->pairs_ok ||
+      c->profile || c->sms <= 0)
+    return p;
+  // Warps per slice: the largest split that still leaves each SM at most 8 warps (short rows), else the
+  // largest that fits; up to 24 warps (768 threads of 80 registers) per SM.
+  const int64_t ns = c->nslices, sms = c->sms;
+  int split = 0;
+  if (ns * 4 <= sms * 16) split = 4;
+  else if (ns * 2 <= sms * 20) split = 2;
+  else if (ns <= sms * 24) split = 1;
+  if (!split) return p;
+  int64_t warps = (ns * split + sms - 1) / sms;  // per block, one block per SM
+  warps = (warps + split - 1) / split * split;
+  p.split = split;
+  p.block = (int)warps * 32;
+  p.grid = (unsigned)((ns * split + warps - 1) / warps);
+  p.pair = c->nbonds > 600000;
+  return p;
+}
+
+pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done) {
+  *done = false;
+  if (!c->bar) {
+    pd_status st = alloc(c, &c->bar, 2);
+    if (st != PD_OK) return st;
+    PD_CUDA(cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
+    c->bar_base = 0;
+  }
+  ResidentArgs r{};
+  r.disp = c->disp[c->cur];
+  r.disp_out = c->disp[c->cur ^ 1];
+  r.nsteps = (int)nsteps;
+  r.check0 = check0 ? 1 : 0;
+  r.step0 = c->steps;
+  r.bar = c->bar;
+  r.bar_base = c->bar_base;
+  r.uv = c->vol_uniform ? 1 : 0;
+  r.gold = c->gold;
+  r.lam = c->lam;
+  r.part = c->adr_part;
+  r.first = c->adr_first;
+  const cudaError_t e = c->dim == 3 ? launch_split<3>(c, a, r, p.grid, p.block, p.split, p.pair)
+                                    : launch_split<2>(c, a, r, p.grid, p.block, p.split, p.pair);
+  if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
+    cudaGetLastError();
+    c->sms = 0;  // this device (or this share of it) cannot hold the grid: the pass kernels take the steps
+    return PD_OK;
+  }
+  if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel");
+  const bool pair = p.pair || p.block > 512;
+  const unsigned per_step = 2u + (pair ? 1u : 0u) + (a.adr ? 1u : 0u);
+  c->bar_base += p.grid * (per_step * (unsigned)nsteps - 1u);
+  if (nsteps & 1) c->cur ^= 1;
+  *done = true;
+  return PD_OK;
+}
+
+}  // namespace pd

@@ -24,61 +24,11 @@
 #include <vector>
 
 #include "pd_internal.h"
-#include "pd_order.h"
+#include "pd_device.h"
 #include "pd_lattice.h"
 
 namespace pd {
 namespace {
-
-constexpr unsigned kFull = 0xffffffffu;
-
-struct SliceIdx {
-  int64_t i;
-  int64_t base;
-  int W;
-  int lane;
-  int sub;
-  bool active;
-};
-
-template <int SPLIT>
-__device__ __forceinline__ SliceIdx slice_index(int64_t n_pad, const int64_t* __restrict__ slice_ptr) {
-  SliceIdx r;
-  const int64_t gwarp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-  r.lane = threadIdx.x & 31;
-  r.sub = (int)(gwarp % SPLIT);
-  const int64_t s = gwarp / SPLIT;
-  r.i = s * 32 + r.lane;
-  r.active = r.i < n_pad;  // n_pad is a multiple of 32: uniform over the warp
-  r.base = 0;
-  r.W = 0;
-  if (r.active) {
-    r.base = slice_ptr[s];
-    r.W = (int)((slice_ptr[s + 1] - r.base) >> 5);
-  }
-  return r;
-}
-
-// Partial sums of the SPLIT warps sharing a slice, combined by the first warp (fixed order).
-template <int SPLIT, int NC, class T>
-__device__ __forceinline__ void split_reduce(T (&v)[NC]) {
-  if (SPLIT == 1) return;
-  extern __shared__ unsigned char smem_raw[];
-  T* red = reinterpret_cast<T*>(smem_raw);
-#pragma unroll
-  for (int c = 0; c < NC; ++c) red[c * blockDim.x + threadIdx.x] = v[c];
-  __syncthreads();
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  if (w % SPLIT == 0) {
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      T s = red[c * blockDim.x + w * 32 + lane];
-#pragma unroll
-      for (int q = 1; q < SPLIT; ++q) s += red[c * blockDim.x + (w + q) * 32 + lane];
-      v[c] = s;
-    }
-  }
-}
 
 // xi = x_j - x_i, du = u_j - u_i, d = xi . du, q = xi . xi in FP64.  Shared by the FP64 path and by
 // the FP64 re-decision of the mixed path, so both decide a bond with identical arithmetic.
@@ -177,7 +127,7 @@ __device__ __forceinline__ void load_slots(const SliceIdx& t, const int32_t* __r
 }
 
 // ------------------------------------------------------------------------------------ FP64 path
-constexpr int kU64 = 2;
+constexpr int kU64 = 2;  // (the recompute and single-pass nonlinear kernels)
 constexpr int kU32 = 4;
 
 // Plain FP64 kernels: the reference geometry of each bond is recomputed from the coordinates.
@@ -791,23 +741,6 @@ __global__ void k_bond_tables_nl(StepArgs a, double4* __restrict__ bA) {
 // xi.du (negative values and -0 sort below every positive double), and it runs on the integer pipe
 // instead of the FP64 one.
 
-// bS_i from the status bits and bB, in slot order (so bS is a function of the bits alone).  The
-// words are read through L2: other warps of the block may have just written them.
-__device__ __forceinline__ void bond_sum_row(const StepArgs& a, const SliceIdx& t) {
-  const uint32_t* bw = a.bits + (t.base >> 5);
-  const double4* tb = a.bB + t.base + t.lane;
-  double sx = 0.0, sy = 0.0, sz = 0.0;
-  for (int k = 0; k < t.W; ++k) {
-    if ((__ldcg(bw + k) >> t.lane) & 1u) {
-      const double4 g = tb[(int64_t)k << 5];
-      sx += g.x;
-      sy += g.y;
-      sz += g.z;
-    }
-  }
-  a.bS[t.i] = make_double4(sx, sy, sz, 0.0);
-}
-
 __global__ void k_bond_sums(StepArgs a) {
   const SliceIdx t = slice_index<1>(a.n_pad, a.slice_ptr);
   if (t.active) bond_sum_row(a, t);
@@ -821,6 +754,8 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (write_theta && blockIdx.x == 0 && threadIdx.x == 0) *a.d_step += 1;
   double acc[2] = {0.0, 0.0};  // theta sum, and 1 if a bond of this warp's slots broke (warp-uniform)
+  constexpr int U = kU64, P = 4 / SPLIT, H = P > U ? P / U : 1;  // H half batches of U slots: the sum's parts
+  double part[1][P] = {};
   int b = 0;
   if (t.active) {
     b = a.body ? a.body[t.i] : 0;
@@ -830,11 +765,13 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
     const int32_t* __restrict__ cl = a.col + t.base + t.lane;
     const double4* __restrict__ ta = a.bA + t.base + t.lane;
     double* __restrict__ td = a.bd + t.base + t.lane;
-    constexpr int U = kU64;
     int32_t jn[U];
     uint32_t wn[U];
     load_slots<U, SPLIT>(t, cl, bw, t.sub, jn, wn);
-    for (int k0 = t.sub; k0 < t.W; k0 += U * SPLIT) {
+    for (int kb = t.sub; kb < t.W; kb += H * U * SPLIT) {
+#pragma unroll
+     for (int h = 0; h < H; ++h) {
+      const int k0 = kb + h * U * SPLIT;
       uint32_t wd[U];
       double4 g[U], uj[U];
 #pragma unroll
@@ -862,12 +799,16 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
             acc[1] = 1.0;
           }
         }
-        if (THETA) acc[0] = fma(intact ? uj[u].w : 0.0, d, acc[0]);
+        if (THETA) part[0][(h * U + u) % P] = fma(intact ? uj[u].w : 0.0, d, part[0][(h * U + u) % P]);
       }
+     }
     }
   }
   if (SPLIT == 1) __syncwarp();  // lane 0's status words, for the bS recomputation below
-  split_reduce<SPLIT, 2>(acc);   // (SPLIT > 1: its block barrier orders the other warps' words)
+  double th1[1];
+  parts_sum<SPLIT, 1>(part, th1);
+  acc[0] = th1[0];
+  parts_across<SPLIT, 2>(acc);  // (SPLIT > 1: its block barrier orders the other warps' words)
   if (t.active && t.sub == 0) {
     if (THETA && write_theta) {
       const double th = a.aA[t.i] * acc[0];
@@ -952,7 +893,7 @@ template <int DIM, int SPLIT, bool UV>
 __global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* __restrict__ disp, int write_theta) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (write_theta && blockIdx.x == 0 && threadIdx.x == 0) *a.d_step += 1;
-  double acc[1] = {0.0};
+  double acc[1], part[1][4 / SPLIT] = {};
   int b = 0;
   if (t.active) {
     b = a.body ? a.body[t.i] : 0;
@@ -997,10 +938,11 @@ __global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* 
       for (int u = 0; u < U; ++u) dn[u] = td[(int64_t)min(k0 + (U + u) * SPLIT, t.W - 1) << 5];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if ((wd[u] >> t.lane) & 1u) acc[0] = fma(v[u], d[u], acc[0]);
+        if ((wd[u] >> t.lane) & 1u) part[0][u % (4 / SPLIT)] = fma(v[u], d[u], part[0][u % (4 / SPLIT)]);
     }
   }
-  split_reduce<SPLIT, 1>(acc);
+  parts_sum<SPLIT, 1>(part, acc);
+  parts_across<SPLIT, 1>(acc);
   if (t.active && t.sub == 0) {
     if (write_theta) {
       const double th = a.aA[t.i] * acc[0];
@@ -1200,7 +1142,7 @@ template <int DIM, int SPLIT>
 __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* __restrict__ disp,
                                                      double4* __restrict__ disp_out) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
-  double f[3] = {0.0, 0.0, 0.0};
+  double f[3], part[3][4 / SPLIT] = {};
   int b = 0;
   if (t.active) {
     b = a.body ? a.body[t.i] : 0;
@@ -1208,37 +1150,44 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
     const int32_t* __restrict__ cl = a.col + t.base + t.lane;
     const double4* __restrict__ tb = a.bB + t.base + t.lane;
     const double* __restrict__ td = a.bd + t.base + t.lane;
-    constexpr int U = 4;
+    // two slots in flight per warp and half batch: with four the parts of the sums need 77 registers
+    constexpr int U = 2, P = 4 / SPLIT, H = P > U ? P / U : 1;
     int32_t jn[U];
     uint32_t wn[U];
     load_slots<U, SPLIT>(t, cl, bw, t.sub, jn, wn);
-    for (int k0 = t.sub; k0 < t.W; k0 += U * SPLIT) {
-      uint32_t wd[U];
-      double4 g[U];
-      double d[U], tj[U];
+    for (int k0 = t.sub; k0 < t.W; k0 += H * U * SPLIT) {
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int k = min(k0 + u * SPLIT, t.W - 1);
-        wd[u] = wn[u];
-        g[u] = tb[(int64_t)k << 5];
-        d[u] = td[(int64_t)k << 5];
-        tj[u] = a.thm[jn[u]].x;
-      }
-      load_slots<U, SPLIT>(t, cl, bw, k0 + U * SPLIT, jn, wn);
+      for (int h = 0; h < H; ++h) {
+        const int kh = k0 + h * U * SPLIT;
+        uint32_t wd[U];
+        double4 g[U];
+        double d[U], tj[U];
 #pragma unroll
-      for (int u = 0; u < U; ++u) {
-        // Eq 2.2 with V_j folded into the tabled xi, G (1/m_i + 1/m_j) / |xi|^2 tabled and the
-        // i-end term (K - G/3) theta_i / m_i applied to bS_i below:
-        // [(K - G/3) theta_j / m_j + G (1/m_i + 1/m_j) e / |xi|] (V_j xi)
-        double c = fma(g[u].w, d[u], tj[u]);
-        c = ((wd[u] >> t.lane) & 1u) ? c : 0.0;
-        f[0] = fma(c, g[u].x, f[0]);
-        f[1] = fma(c, g[u].y, f[1]);
-        if (DIM == 3) f[2] = fma(c, g[u].z, f[2]);
+        for (int u = 0; u < U; ++u) {
+          const int k = min(kh + u * SPLIT, t.W - 1);
+          wd[u] = wn[u];
+          g[u] = tb[(int64_t)k << 5];
+          d[u] = td[(int64_t)k << 5];
+          tj[u] = a.thm[jn[u]].x;
+        }
+        load_slots<U, SPLIT>(t, cl, bw, kh + U * SPLIT, jn, wn);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          // Eq 2.2 with V_j folded into the tabled xi, G (1/m_i + 1/m_j) / |xi|^2 tabled and the
+          // i-end term (K - G/3) theta_i / m_i applied to bS_i below:
+          // [(K - G/3) theta_j / m_j + G (1/m_i + 1/m_j) e / |xi|] (V_j xi)
+          double c = fma(g[u].w, d[u], tj[u]);
+          c = ((wd[u] >> t.lane) & 1u) ? c : 0.0;
+          const int n = (h * U + u) % P;
+          part[0][n] = fma(c, g[u].x, part[0][n]);
+          part[1][n] = fma(c, g[u].y, part[1][n]);
+          if (DIM == 3) part[2][n] = fma(c, g[u].z, part[2][n]);
+        }
       }
     }
   }
-  split_reduce<SPLIT, 3>(f);
+  parts_sum<SPLIT, 3>(part, f);
+  parts_across<SPLIT, 3>(f);
   if (t.active && t.sub == 0) {
     const double ti = a.thm[t.i].x;
     const double4 S = a.bS[t.i];
@@ -2473,62 +2422,23 @@ __global__ void k_adr_lambda(StepArgs a, const double* __restrict__ alpha, doubl
 
 constexpr int kAdrBlock = 256;
 
-// Per block: sum over its free particles' components of u (k u) and u u, k = -(g - g_prev) / (lambda v).
+// Per slice: sum over its free particles' components of u (k u) and u u, k = -(g - g_prev) / (lambda v).
 __global__ void __launch_bounds__(kAdrBlock) k_adr_sums(StepArgs a, const double4* __restrict__ disp,
                                                          const double4* __restrict__ gold,
                                                          const double2* __restrict__ lam,
                                                          double2* __restrict__ part) {
-  __shared__ double sn[kAdrBlock], sd[kAdrBlock];
   const int64_t i = blockIdx.x * (int64_t)kAdrBlock + threadIdx.x;
-  double num = 0.0, den = 0.0;
-  if (i < a.n_pad && (!a.flag || a.flag[i] == 0) && lam[i].x > 0.0) {
-    const double4 u = disp[i], v = a.vel[i], g = a.gnew[i], go = gold[i];
-    const double li = lam[i].x;
-    const double uu[3] = {u.x, u.y, u.z}, vv[3] = {v.x, v.y, v.z}, gg[3] = {g.x, g.y, g.z},
-                 gp[3] = {go.x, go.y, go.z};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const double kk = vv[k] != 0.0 ? -(gg[k] - gp[k]) / (li * vv[k]) : 0.0;
-      num += uu[k] * kk * uu[k];
-      den += uu[k] * uu[k];
-    }
-  }
-  sn[threadIdx.x] = num;
-  sd[threadIdx.x] = den;
-  __syncthreads();
-  for (int w = kAdrBlock / 2; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sn[threadIdx.x] += sn[threadIdx.x + w];
-      sd[threadIdx.x] += sd[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
-  if (threadIdx.x == 0) part[blockIdx.x] = make_double2(sn[0], sd[0]);
+  if (i >= a.n_pad) return;  // whole warps: n_pad is a multiple of 32
+  const double2 s = adr_terms((!a.flag || a.flag[i] == 0) && lam[i].x > 0.0, disp[i], a.vel[i], a.gnew[i], gold[i], lam[i].x);
+  if ((threadIdx.x & 31) == 0) part[i >> 5] = s;
 }
 
-// One block: c = 2 sqrt(num / den) (0 unless both are positive), the start flag of this iteration and
-// 1 / (2 + c).
-__global__ void __launch_bounds__(1024) k_adr_coef(const double2* __restrict__ part, int nblk, int* first,
+// One block: the damping and the start flag of this iteration.
+__global__ void __launch_bounds__(1024) k_adr_coef(const double2* __restrict__ part, int64_t nslices, int* first,
                                                    double4* st) {
-  __shared__ double sn[1024], sd[1024];
-  double num = 0.0, den = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += 1024) {
-    num += part[b].x;
-    den += part[b].y;
-  }
-  sn[threadIdx.x] = num;
-  sd[threadIdx.x] = den;
-  __syncthreads();
-  for (int w = 512; w > 0; w >>= 1) {
-    if (threadIdx.x < w) {
-      sn[threadIdx.x] += sn[threadIdx.x + w];
-      sd[threadIdx.x] += sd[threadIdx.x + w];
-    }
-    __syncthreads();
-  }
+  const double2 c = adr_damping(part, nslices);
   if (threadIdx.x == 0) {
-    const double c = (sd[0] > 0.0 && sn[0] > 0.0) ? 2.0 * sqrt(sn[0] / sd[0]) : 0.0;
-    *st = make_double4(c, (double)*first, 1.0 / (2.0 + c), 0.0);
+    *st = make_double4(c.x, (double)*first, c.y, 0.0);
     *first = 0;
   }
 }
@@ -2553,15 +2463,10 @@ __global__ void __launch_bounds__(kAdrBlock) k_adr_update(StepArgs a, const doub
     const double2 li = lam[i];  // (lambda, 1 / lambda)
     if (li.x > 0.0) {
       const double4 s = *st;
-      if (s.y != 0.0) {
-        const double h = 0.5 * li.y;
-        v = make_double4(g.x * h, g.y * h, g.z * h, 0.0);
-      } else {
-        const double cm = 2.0 - s.x, r2 = 2.0 * li.y;
-        v.x = (cm * v.x + g.x * r2) * s.z;
-        v.y = (cm * v.y + g.y * r2) * s.z;
-        v.z = (cm * v.z + g.z * r2) * s.z;
-      }
+      const bool start = s.y != 0.0;
+      v.x = adr_velocity(v.x, g.x, li.y, s.x, s.z, start);
+      v.y = adr_velocity(v.y, g.y, li.y, s.x, s.z, start);
+      v.z = adr_velocity(v.z, g.z, li.y, s.x, s.z, start);
       u.x = u.x + v.x;
       u.y = u.y + v.y;
       u.z = u.z + v.z;
@@ -2921,6 +2826,7 @@ cudaEvent_t take_event(pd_ctx* c) {
 // kSplit1a warps per slice in the pair forms' pass 1a, which sums nothing, so that its results do not
 // depend on the split (nonlinear: 1.405 -> 1.34 ms).
 constexpr int kAutoBlock64 = 64;
+constexpr int kAutoSplit64 = 2;  // linearized, tabled: any split gives the same sums
 constexpr int kSplit1aL = 2, kBlock1aL = 64;    // linearized
 constexpr int kSplit1aNL = 4, kBlock1aNL = 128;  // nonlinear
 
@@ -3158,7 +3064,7 @@ namespace {
 template <int DIM>
 void dispatch_pass(pd_ctx* c, const StepArgs& a, int pass, int write_theta) {
   const int block = c->auto_map && c->precision == PD_FP64 ? kAutoBlock64 : c->block;
-  const int split = c->split;
+  const int split = c->auto_map && c->precision == PD_FP64 && c->kin == PD_LINEARIZED && a.bA ? kAutoSplit64 : c->split;
   const int64_t threads = c->nslices * 32 * (int64_t)split;
   const unsigned grid = (unsigned)((threads + block - 1) / block);
   if (c->precision == PD_MIXED && c->lattice) {
@@ -3283,11 +3189,10 @@ pd_status ensure_adr(pd_ctx* c) {
   pd_status st;
   if (!c->lam) {
     const int64_t np = c->n_pad;
-    const size_t nblk = (size_t)((np + kAdrBlock - 1) / kAdrBlock);
     if ((st = alloc(c, &c->lam, np)) != PD_OK) return st;
     if ((st = alloc(c, &c->gnew, np)) != PD_OK) return st;
     if ((st = alloc(c, &c->gold, np)) != PD_OK) return st;
-    if ((st = alloc(c, &c->adr_part, nblk)) != PD_OK) return st;
+    if ((st = alloc(c, &c->adr_part, (size_t)c->nslices)) != PD_OK) return st;
     if ((st = alloc(c, &c->adr_st, 1)) != PD_OK) return st;
     if ((st = alloc(c, &c->adr_first, 1)) != PD_OK) return st;
     PD_CUDA(cudaMemsetAsync(c->gnew, 0, sizeof(double4) * np, c->stream));
@@ -3381,7 +3286,7 @@ pd_status launch_step(pd_ctx* c, bool check) {
   if (a.adr) {
     const unsigned nblk = (unsigned)((c->n_pad + kAdrBlock - 1) / kAdrBlock);
     k_adr_sums<<<nblk, kAdrBlock, 0, c->stream>>>(a, c->disp[c->cur], c->gold, c->lam, c->adr_part);
-    k_adr_coef<<<1, 1024, 0, c->stream>>>(c->adr_part, (int)nblk, c->adr_first, c->adr_st);
+    k_adr_coef<<<1, 1024, 0, c->stream>>>(c->adr_part, c->nslices, c->adr_first, c->adr_st);
     k_adr_update<<<nblk, kAdrBlock, 0, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1], c->gold, c->lam,
                                                     c->adr_st,
                                                     c->precision == PD_MIXED ? c->u32[c->cur ^ 1] : nullptr,
@@ -3560,8 +3465,12 @@ pd_status check_device_error(pd_ctx* c) {
   PD_CUDA(cudaStreamSynchronize(c->stream));
   if (flag) {
     PD_CUDA(cudaMemsetAsync(c->counters + 4, 0, sizeof(flag), c->stream));
-    return fail(PD_ERR_TIMEOUT, "a staged neighbour-index copy did not complete within the wait limit; "
-                                "the step's results were not written");
+    if (c->bar) {  // the resident step kernel's barrier starts over
+      PD_CUDA(cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
+      c->bar_base = 0;
+    }
+    return fail(PD_ERR_TIMEOUT, "a staged neighbour-index copy or a grid barrier did not complete within the wait "
+                                "limit; the step's results were not written");
   }
   if (nonfinite) {
     PD_CUDA(cudaMemsetAsync(c->counters + 5, 0, sizeof(nonfinite), c->stream));
@@ -3586,6 +3495,9 @@ pd_status max_abs_u(pd_ctx* c, double* out, int* nonfinite) {
   return PD_OK;
 }
 
+// Steps per launch of the resident step kernel (tens of milliseconds at most).
+constexpr int64_t kResidentSteps = 1000;
+
 // nsteps time steps: the first step after a state change skips the failure check at its head (the
 // paper checks after each update, never before the first force evaluation); then CUDA-graph
 // chunks of graph_chunk steps, then single steps.
@@ -3605,9 +3517,28 @@ pd_status run_steps(pd_ctx* c, int64_t nsteps) {
   if (st != PD_OK) return st;
   if (c->precision == PD_FP64 && !c->bond_cache) c->bs_stale = true;  // untabled kernels break bonds
   if ((st = ensure_adr(c)) != PD_OK) return st;
+  int64_t left = nsteps;
+  const ResidentPlan plan = resident_plan(c);
+  if (plan.split) {
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    PD_CUDA(cudaStreamIsCapturing(c->stream, &cap));
+    bool done = cap == cudaStreamCaptureStatusNone;  // a caller's capture takes the pass kernels
+    while (left > 0 && done) {
+      const int64_t n = std::min<int64_t>(left, kResidentSteps);
+      st = run_resident(c, make_args(c), plan, n, !c->skip_next_check, &done);
+      if (st != PD_OK) return st;
+      if (!done) break;
+      c->skip_next_check = false;
+      left -= n;
+      c->steps += n;
+    }
+    if (left == 0) {
+      c->check_pending = true;
+      return PD_OK;  // the kernel has marked a non-finite state
+    }
+  }
   st = launch_set_step(c, c->steps - 1);
   if (st != PD_OK) return st;
-  int64_t left = nsteps;
   if (c->skip_next_check) {
     st = launch_step(c, false);
     if (st != PD_OK) return st;

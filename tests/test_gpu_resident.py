@@ -1,0 +1,113 @@
+"""The resident step kernel (bodies that fit the chip in one wave) against the pass kernels, which a
+chosen launch mapping selects: bitwise the same states, damage and bond status at the edges of its sizes
+and forms, with breaking, reads between steps, constraints, uneven volumes and batches; its bounded
+barrier wait (GPU only)."""
+import numpy as np
+import pytest
+
+from paper_2309_11273_gb300 import BatchSimulation, PDError, Simulation
+from paper_2309_11273_gb300 import _binding as B
+from paper_2309_11273_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _pass_kernels(sim):
+    sim.set_option(B.PD_OPT_BLOCK, 128)
+    return sim
+
+
+def _run(sim, chunks):
+    out = []
+    for k in chunks:
+        sim.step(k)
+        out += list(sim.state())
+    out += [sim.damage(), sim.neighbors()[2]]
+    sim.close()
+    return out
+
+
+def _same(make, chunks):
+    for x, y in zip(_run(make(), chunks), _run(_pass_kernels(make()), chunks)):
+        assert np.array_equal(x, y)
+
+
+def _plate(nx, ny, ratio=3.015):
+    w = W.cracked_plate(nx=nx, ny=ny, ratio=ratio, crack_cells=nx // 2 + 0.125)
+    w.u0 = np.random.default_rng(3).normal(0.0, 2e-9, (2, w.n))
+    w.u0[1] += 4e-4 * (w.y - 0.5 * w.y.max())  # near the critical stretch: bonds break from the first steps
+    return w
+
+
+# particles: one slice, a ragged one, each side of four and of two warps per slice, the largest resident
+# bodies (768-thread blocks) and the first beyond them
+@pytest.mark.parametrize("nx,ny", [(5, 4), (11, 8), (40, 40), (139, 140), (180, 110), (221, 220), (250, 256), (341, 340),
+                                   (350, 340)])
+def test_plates_are_bitwise_the_pass_kernels(nx, ny):
+    _same(lambda: Simulation(_plate(nx, ny)), [1, 2, 30, 17])
+
+
+@pytest.mark.parametrize("shape", [(9, 7, 5), (24, 12, 10), (40, 25, 20), (61, 30, 25), (80, 40, 36)])
+def test_blocks_are_bitwise_the_pass_kernels(shape):
+    def make():
+        w = W.notched_block(*shape, nsteps=300, seed=5, amp=2e-8)
+        return Simulation(w)
+    _same(make, [1, 25, 24])
+
+
+def test_uneven_volumes_and_impact():
+    def cloud():
+        rng = np.random.default_rng(11)
+        x, y, z = W.grid_3d(30, 20, 18, 1e-3)
+        x, y, z = (a + rng.uniform(-2e-4, 2e-4, a.size) for a in (x, y, z))
+        w = W.Workload("cloud", W.MODEL_3D, dx=1e-3, delta=3.015e-3, dt=2e-7, nsteps=50, x=x, y=y, z=z,
+                       vol=1e-9 * rng.uniform(0.5, 1.5, x.size), Gc=50.0, u0=rng.normal(0.0, 3e-7, (3, x.size)), **W.CONCRETE)
+        return Simulation(w)
+    _same(cloud, [3, 40])
+    _same(lambda: Simulation(W.kalthoff(nx=120, ny=61, notch_cells=30.125, gap_cells=30)), [50, 51])
+
+
+def test_batches_and_relaxation():
+    _same(lambda: BatchSimulation(W.plate_batch(nplates=9, side_hi=90)), [60, 40])
+
+    def static():
+        x, y, z = W.grid_3d(30, 12, 10, 1e-3)
+        flag = np.where(x < 3e-3, 1, 0).astype(np.uint8)
+        b = np.zeros((3, x.size))
+        b[2] = -2e6
+        w = W.Workload("static", W.MODEL_3D, dx=1e-3, delta=3.015e-3, dt=1.0, nsteps=0, x=x, y=y, z=z,
+                       vol=np.full(x.size, 1e-9), flag=flag, b=b, **W.CONCRETE)
+        sim = Simulation(w, s0=0.0)
+        sim.set_option(B.PD_OPT_SOLVER, B.PD_SOLVER_ADR)
+        return sim
+    _same(static, [1, 40, 59])
+
+
+def test_switching_between_the_kernels_keeps_the_run():
+    ref = Simulation(_plate(90, 60))
+    ref.step(120)
+    sim = Simulation(_plate(90, 60))
+    sim.step(40)
+    _pass_kernels(sim).step(40)
+    assert B.pd_autotune(sim.h, 2)[0] > 0
+    sim.step(40)
+    for x, y in zip(list(sim.state()) + [sim.damage()], list(ref.state()) + [ref.damage()]):
+        assert np.array_equal(x, y)
+
+
+def test_expired_barrier_reports_timeout_and_the_context_recovers():
+    w = _plate(60, 40)
+    sim = Simulation(w)
+    sim.set_option(B.PD_OPT_EXPIRE_WAITS, 1)  # block 0 never arrives: every wait runs out
+    sim.step(3)
+    with pytest.raises(PDError) as e:
+        sim.sync()
+    assert e.value.status == B.PD_ERR_TIMEOUT
+    sim.set_option(B.PD_OPT_EXPIRE_WAITS, 0)
+    B.pd_build_neighbors(sim.h, w.cracks)
+    B.pd_set_bc(sim.h, 2, w.n, None, w.b)
+    sim.set_state(w.u0)
+    sim.step(50)
+    ref = Simulation(w)
+    ref.step(50)
+    assert np.array_equal(sim.state()[0], ref.state()[0])
