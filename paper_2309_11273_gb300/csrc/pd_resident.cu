@@ -81,12 +81,17 @@ __device__ __forceinline__ bool grid_barrier(const StepArgs& a, const ResidentAr
   return ok_s != 0;
 }
 
-// PAIR: pass 1 in its pair form (fewer FP64 instructions, one barrier more).  MAXT: largest block; its
-// registers bound the slots in flight U.
+// PAIR: pass 1 in its pair form (fewer FP64 instructions, one barrier more).  MAXT: the largest block.  Up to
+// 512 threads (128 registers) four slots are in flight per warp and the state stays in registers; up to
+// 768 (80 registers) two, and the state is read again at the update.  Without the pair form, on the
+// smallest bodies, the neighbour indices are loaded a batch ahead, and a pass's first ones before the
+// barrier in front of it, so that a batch waits for one round trip to L2 instead of two (40 x 40 plate 9.7
+// -> 9.1 us per step); the pair form spills with it (400 x 160 plate 39.8 -> 41.3 us).
 template <int DIM, int SPLIT, bool PAIR, bool ADR, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r) {
   constexpr int P = 4 / SPLIT;
-  constexpr int U = MAXT > 512 ? 2 : 4;
+  constexpr bool kKeep = MAXT <= 512;  // the particles' state in registers
+  constexpr int U = kKeep ? 4 : 2;
   constexpr int H = P > U ? P / U : 1;
   if (ld_relaxed(r.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
   unsigned target = r.bar_base;
@@ -104,27 +109,40 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   const double4* ta = a.bA + t.base + t.lane;
   const double4* tb = a.bB + t.base + t.lane;
   double* td = a.bd + t.base + t.lane;
-  double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u, gold = u;
-  double2 lam = make_double2(0.0, 0.0);
-  double th = 0.0;
-  bool start = false;
   const uint8_t fl = lead && a.flag ? a.flag[i] : (uint8_t)0;
-  const double4 bb = lead && a.bacc ? a.bacc[i] : make_double4(0.0, 0.0, 0.0, 0.0);
-  if (lead) {
-    u = r.disp[i];
+  double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u, gold = u, bb = u;
+  double2 lam = make_double2(0.0, 0.0);
+  auto load_state = [&](const double4* disp) {  // of the slice's first warp
+    if (!lead) return;
+    u = disp[i];
     v = a.vel[i];
+    if (a.bacc) bb = a.bacc[i];
     if (ADR) {
       gold = r.gold[i];
       lam = r.lam[i];
-      start = *r.first != 0;
     }
-    if (a.dirty[s]) {  // bonds broken by a check between calls
-      bond_sum_row(a, t);
-      __syncwarp();
-      if (t.lane == 0) a.dirty[s] = 0;
-    }
+  };
+  auto store_state = [&]() {
+    if (!lead) return;
+    a.vel[i] = v;
+    if (ADR) r.gold[i] = gold;
+  };
+  const bool start0 = ADR && *r.first != 0;
+  if (kKeep) load_state(r.disp);
+  if (lead && a.dirty[s]) {  // bonds broken by a check between calls
+    bond_sum_row(a, t);
+    __syncwarp();
+    if (t.lane == 0) a.dirty[s] = 0;
   }
   const double vi = t.active ? a.pos[i].w : 0.0;
+  // the neighbours of a batch of slots (past the row: its last one), loaded in place or ahead
+  int32_t jn[U];
+  auto slots = [&](int k0, bool ahead) {
+    if (ahead == PAIR || !t.active || k0 >= t.W) return;
+#pragma unroll
+    for (int q = 0; q < U; ++q) jn[q] = cl[(int64_t)min(k0 + q * SPLIT, t.W - 1) << 5];
+  };
+  slots(t.sub, true);
   for (int step = 0; step < r.nsteps; ++step) {
     const double4* disp = (step & 1) ? r.disp_out : r.disp;
     double4* disp_out = (step & 1) ? r.disp : r.disp_out;
@@ -139,13 +157,12 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
           double4 g[U], uj[U];
 #pragma unroll
           for (int q = 0; q < U; ++q) {
-            const int k = min(own + m0 + q * SPLIT, max(cnt - 1, 0));
-            j[q] = cl[(int64_t)k << 5];
-            g[q] = ta[(int64_t)k << 5];
-            te[q] = tw[(int64_t)k << 5];
+            const int64_t k = (int64_t)min(own + m0 + q * SPLIT, max(cnt - 1, 0)) << 5;
+            j[q] = cl[k];
+            te[q] = tw[k];
+            g[q] = ta[k];
+            uj[q] = disp[j[q]];
           }
-#pragma unroll
-          for (int q = 0; q < U; ++q) uj[q] = disp[j[q]];
 #pragma unroll
           for (int q = 0; q < U; ++q) {
             const int k = own + m0 + q * SPLIT;
@@ -174,48 +191,54 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
           }
         }
       }
-    } else if (t.active) {
-      const double4 ui = disp[i];
-      for (int kb = t.sub; kb < t.W; kb += H * U * SPLIT) {
+    } else {
+      if (t.active) {
+        const double4 ui = disp[i];
+        for (int kb = t.sub; kb < t.W; kb += H * U * SPLIT) {
 #pragma unroll
-        for (int h = 0; h < H; ++h) {
-          const int k0 = kb + h * U * SPLIT;
-          uint32_t wd[U];
-          double4 g[U], uj[U];
+          for (int h = 0; h < H; ++h) {
+            const int k0 = kb + h * U * SPLIT;
+            uint32_t wd[U];
+            double4 g[U], uj[U];
 #pragma unroll
-          for (int q = 0; q < U; ++q) {
-            const int k = min(k0 + q * SPLIT, t.W - 1);
-            wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
-            g[q] = ta[(int64_t)k << 5];
-            uj[q] = disp[cl[(int64_t)k << 5]];
-          }
-#pragma unroll
-          for (int q = 0; q < U; ++q) {
-            double d = g[q].x * (uj[q].x - ui.x) + g[q].y * (uj[q].y - ui.y);
-            if (DIM == 3) d = fma(g[q].z, uj[q].z - ui.z, d);
-            const int k = k0 + q * SPLIT;
-            if (k < t.W) td[(int64_t)k << 5] = d;
-            bool intact = (wd[q] >> t.lane) & 1u;
-            const unsigned m = __ballot_sync(kFull, check && intact && pd_ge_threshold(d, g[q].w));
-            if (m) {
-              if ((m >> t.lane) & 1u) intact = false;
-              if (t.lane == 0) bw[k] = wd[q] & ~m;
-              sum[1] = 1.0;
+            for (int q = 0; q < U; ++q) {
+              const int k = min(k0 + q * SPLIT, t.W - 1);
+              wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
+              g[q] = ta[(int64_t)k << 5];
+              uj[q] = disp[jn[q]];
             }
-            part1[0][(h * U + q) % P] = fma(intact ? uj[q].w : 0.0, d, part1[0][(h * U + q) % P]);
+            slots(k0 + U * SPLIT, true);
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+              double d = g[q].x * (uj[q].x - ui.x) + g[q].y * (uj[q].y - ui.y);
+              if (DIM == 3) d = fma(g[q].z, uj[q].z - ui.z, d);
+              const int k = k0 + q * SPLIT;
+              if (k < t.W) td[(int64_t)k << 5] = d;
+              bool intact = (wd[q] >> t.lane) & 1u;
+              const unsigned m = __ballot_sync(kFull, check && intact && pd_ge_threshold(d, g[q].w));
+              if (m) {
+                if ((m >> t.lane) & 1u) intact = false;
+                if (t.lane == 0) bw[k] = wd[q] & ~m;
+                sum[1] = 1.0;
+              }
+              part1[0][(h * U + q) % P] = fma(intact ? uj[q].w : 0.0, d, part1[0][(h * U + q) % P]);
+            }
           }
         }
       }
+      slots(t.sub, true);
       __syncwarp();
     }
     double th1[1];
     parts_sum<SPLIT, 1>(part1, th1);
     sum[0] = th1[0];
     parts_across<SPLIT, 2>(sum);
+    double ti = 0.0;
     if (lead) {
-      th = a.aA[i] * sum[0];
-      const double mu = a.mu[i];
-      a.thm[i] = make_double2(bp.Kp * (th * mu), bp.G * mu);
+      const double th = a.aA[i] * sum[0], mu = a.mu[i];
+      ti = bp.Kp * (th * mu);
+      a.thm[i] = make_double2(ti, bp.G * mu);
+      if (step + 1 == r.nsteps) a.theta[i] = th;
       if (PAIR ? a.dirty[s] != 0 : sum[1] != 0.0) {  // uniform over the warp
         bond_sum_row(a, t);
         __syncwarp();
@@ -233,14 +256,16 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
           uint32_t wd[U];
           double4 g[U];
           double d[U], tj[U];
+          slots(k0, false);
 #pragma unroll
           for (int q = 0; q < U; ++q) {
             const int k = min(k0 + q * SPLIT, t.W - 1);
             wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
             g[q] = tb[(int64_t)k << 5];
             d[q] = td[(int64_t)k << 5];
-            tj[q] = a.thm[cl[(int64_t)k << 5]].x;
+            tj[q] = a.thm[jn[q]].x;
           }
+          slots(k0 + U * SPLIT, true);
 #pragma unroll
           for (int q = 0; q < U; ++q) {
             double c = fma(g[q].w, d[q], tj[q]);
@@ -253,10 +278,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
         }
       }
     }
+    if (!kKeep) load_state(disp);
     parts_sum<SPLIT, 3>(part, f);
     parts_across<SPLIT, 3>(f);
     if (lead) {
-      const double ti = a.thm[i].x;
       const double4 S = a.bS[i];
       f[0] = fma(ti, S.x, f[0]);
       f[1] = fma(ti, S.y, f[1]);
@@ -279,6 +304,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
       if (fl == 0) {
         if (ADR) {
           if (lam.x > 0.0) {
+            const bool start = start0 && step == 0;
             v.x = adr_velocity(v.x, f[0], lam.y, c.x, c.y, start);
             v.y = adr_velocity(v.y, f[1], lam.y, c.x, c.y, start);
             v.z = adr_velocity(v.z, f[2], lam.y, c.x, c.y, start);
@@ -308,16 +334,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
       }
       disp_out[i] = u;  // .w carries V_i unchanged
       if (ADR) gold = make_double4(f[0], f[1], f[2], 0.0);
-      start = false;
     }
-    if (step + 1 < r.nsteps && !grid_barrier(a, r, target)) return;
+    const bool last = step + 1 == r.nsteps;
+    if (!kKeep || last) store_state();
+    if (last) break;
+    slots(t.sub, true);
+    if (!grid_barrier(a, r, target)) return;
   }
-  if (lead) {
-    a.vel[i] = v;
-    a.theta[i] = th;
-    if (ADR) r.gold[i] = gold;
-    if (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z)) atomicExch(&a.counters[5], 1ull);
-  }
+  if (lead && (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z))) atomicExch(&a.counters[5], 1ull);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *a.d_step = r.step0 + r.nsteps - 1;
     if (ADR) *r.first = 0;  // every block read it before its first barrier
@@ -354,15 +378,16 @@ ResidentPlan resident_plan(const pd_ctx* c) {
   if (!c->auto_map || c->precision != PD_FP64 || c->kin != PD_LINEARIZED || !c->bond_cache || !c->pairs || !c->pairs_ok ||
       c->profile || c->sms <= 0)
     return p;
-  // Warps per slice: the largest split that still leaves each SM at most 8 warps (short rows), else the
-  // largest that fits; up to 24 warps (768 threads of 80 registers) per SM.
+  // Warps per slice: four while that leaves an SM at most 16 warps (128 registers each), two up to 20, one up
+  // to 24 (80 registers); beyond, the pass kernels with their own balance over waves are the faster ones.
   const int64_t ns = c->nslices, sms = c->sms;
   int split = 0;
   if (ns * 4 <= sms * 16) split = 4;
   else if (ns * 2 <= sms * 20) split = 2;
   else if (ns <= sms * 24) split = 1;
   if (!split) return p;
-  int64_t warps = (ns * split + sms - 1) / sms;  // per block, one block per SM
+  // One block per SM; a slice's warps share a block (parts_across).
+  int64_t warps = (ns * split + sms - 1) / sms;
   warps = (warps + split - 1) / split * split;
   p.split = split;
   p.block = (int)warps * 32;
