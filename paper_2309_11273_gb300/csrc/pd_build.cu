@@ -922,6 +922,7 @@ pd_status upload_body_params(pd_ctx* c) {
     d.G = G;
     d.inv_rho = 1.0 / p.rho;
     d.dt = p.dt;
+    d.dt_rho = p.dt * d.inv_rho;
     d.s0 = p.s0;
     d.s0nl = p.s0 * (2.0 + p.s0);
     d.breaks = p.s0 > 0.0 ? 1 : 0;

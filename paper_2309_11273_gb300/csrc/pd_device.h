@@ -90,15 +90,53 @@ __device__ __forceinline__ void parts_across(double (&v)[NC]) {
   }
 }
 
+// Eq 2.11 for a free particle with the force density f and the body force b (nullptr: none): v += (dt / rho)
+// (f + b), u += dt v, two or three FMAs per component (an FP64 instruction occupies its pipe for 64 cycles
+// per warp); the z components stay as they are in 2D.
+template <int DIM>
+__device__ __forceinline__ void explicit_move(const BodyDev& bp, const double f[3], const double4* b, double4& u,
+                                              double4& v) {
+  v.x = fma(bp.dt_rho, f[0], v.x);
+  v.y = fma(bp.dt_rho, f[1], v.y);
+  if (DIM == 3) v.z = fma(bp.dt_rho, f[2], v.z);
+  if (b) {
+    v.x = fma(bp.dt_rho, b->x, v.x);
+    v.y = fma(bp.dt_rho, b->y, v.y);
+    if (DIM == 3) v.z = fma(bp.dt_rho, b->z, v.z);
+  }
+  u.x = fma(bp.dt, v.x, u.x);
+  u.y = fma(bp.dt, v.y, u.y);
+  if (DIM == 3) u.z = fma(bp.dt, v.z, u.z);
+}
+
+// Row e of a per-slot table of the linearized FP64 kernels.  In 2D the table holds no z: all pairs (x, y),
+// then all fourth words, 24 bytes per slot instead of 32 (a 400 x 160 plate's tables, index and extension
+// streams then stay in L2).
+template <int DIM>
+__device__ __forceinline__ double4 slot_row(const double4* __restrict__ table, int64_t ne, int64_t e) {
+  if (DIM == 3) return table[e];
+  const double2 xy = reinterpret_cast<const double2*>(table)[e];
+  return make_double4(xy.x, xy.y, 0.0, reinterpret_cast<const double*>(table)[2 * ne + e]);
+}
+template <int DIM>
+__device__ __forceinline__ void set_slot_row(double4* table, int64_t ne, int64_t e, const double4& v) {
+  if (DIM == 3) {
+    table[e] = v;
+  } else {
+    reinterpret_cast<double2*>(table)[e] = make_double2(v.x, v.y);
+    reinterpret_cast<double*>(table)[2 * ne + e] = v.w;
+  }
+}
+
 // bS_i from the status bits and bB, in slot order (so bS is a function of the bits alone).  The
 // words are read through L2: other warps of the block may have just written them.
+template <int DIM>
 __device__ __forceinline__ void bond_sum_row(const StepArgs& a, const SliceIdx& t) {
   const uint32_t* bw = a.bits + (t.base >> 5);
-  const double4* tb = a.bB + t.base + t.lane;
   double sx = 0.0, sy = 0.0, sz = 0.0;
   for (int k = 0; k < t.W; ++k) {
     if ((__ldcg(bw + k) >> t.lane) & 1u) {
-      const double4 g = tb[(int64_t)k << 5];
+      const double4 g = slot_row<DIM>(a.bB, a.ne, t.base + t.lane + ((int64_t)k << 5));
       sx += g.x;
       sy += g.y;
       sz += g.z;

@@ -20,6 +20,7 @@ struct BodyDev {
   double G;        // Eq 1.16
   double inv_rho;  // 1 / rho
   double dt;       // time step
+  double dt_rho;   // dt / rho: the velocity update's factor of the force density
   double s0;       // critical stretch (<= 0: no breaking)
   double s0nl;     // s0 (2 + s0): nonlinear break test |Y|^2 - |xi|^2 >= s0nl |xi|^2
   double rate;     // prescribed rotation rate
@@ -102,8 +103,9 @@ struct StepArgs {
   float band_c;            // safety factor of the band
   int validate;            // mixed: also decide every bond in FP64 and count mismatches
   int check;               // apply the failure criterion at the head of pass 1
-  const double4* bA;       // tabled FP64 path: per slot (xi, s0 |xi|^2), or nullptr
+  const double4* bA;       // tabled FP64 path: per slot (xi, s0 |xi|^2), or nullptr (2D linearized: slot_row)
   const double4* bB;       // tabled FP64 path: per slot (V_j xi, G (1/m_i + 1/m_j) / |xi|^2)
+  int64_t ne;              // slots of the tables
   double* bd;              // tabled FP64 path: per slot xi.(u_j - u_i), written by pass 1
   double4* bS;             // tabled FP64 path: per particle sum of V_j xi over the intact slots
   const int32_t* cnt;      // family size of each row

@@ -106,8 +106,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   uint32_t* bw = a.bits + (t.base >> 5);
   const int32_t* cl = a.col + t.base + t.lane;
   const int32_t* tw = a.twin + t.base + t.lane;
-  const double4* ta = a.bA + t.base + t.lane;
-  const double4* tb = a.bB + t.base + t.lane;
+  const int64_t e0 = t.base + t.lane;
   double* td = a.bd + t.base + t.lane;
   const uint8_t fl = lead && a.flag ? a.flag[i] : (uint8_t)0;
   double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u, gold = u, bb = u;
@@ -130,7 +129,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   const bool start0 = ADR && *r.first != 0;
   if (kKeep) load_state(r.disp);
   if (lead && a.dirty[s]) {  // bonds broken by a check between calls
-    bond_sum_row(a, t);
+    bond_sum_row<DIM>(a, t);
     __syncwarp();
     if (t.lane == 0) a.dirty[s] = 0;
   }
@@ -160,7 +159,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
             const int64_t k = (int64_t)min(own + m0 + q * SPLIT, max(cnt - 1, 0)) << 5;
             j[q] = cl[k];
             te[q] = tw[k];
-            g[q] = ta[k];
+            g[q] = slot_row<DIM>(a.bA, a.ne, e0 + k);
             uj[q] = disp[j[q]];
           }
 #pragma unroll
@@ -204,7 +203,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
             for (int q = 0; q < U; ++q) {
               const int k = min(k0 + q * SPLIT, t.W - 1);
               wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
-              g[q] = ta[(int64_t)k << 5];
+              g[q] = slot_row<DIM>(a.bA, a.ne, e0 + ((int64_t)k << 5));
               uj[q] = disp[jn[q]];
             }
             slots(k0 + U * SPLIT, true);
@@ -237,10 +236,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
     if (lead) {
       const double th = a.aA[i] * sum[0], mu = a.mu[i];
       ti = bp.Kp * (th * mu);
-      a.thm[i] = make_double2(ti, bp.G * mu);
+      a.thm[i].x = ti;
       if (step + 1 == r.nsteps) a.theta[i] = th;
       if (PAIR ? a.dirty[s] != 0 : sum[1] != 0.0) {  // uniform over the warp
-        bond_sum_row(a, t);
+        bond_sum_row<DIM>(a, t);
         __syncwarp();
         if (PAIR && t.lane == 0) a.dirty[s] = 0;
       }
@@ -261,7 +260,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
           for (int q = 0; q < U; ++q) {
             const int k = min(k0 + q * SPLIT, t.W - 1);
             wd[q] = k0 + q * SPLIT < t.W ? bw[k] : 0u;
-            g[q] = tb[(int64_t)k << 5];
+            g[q] = slot_row<DIM>(a.bB, a.ne, e0 + ((int64_t)k << 5));
             d[q] = td[(int64_t)k << 5];
             tj[q] = a.thm[jn[q]].x;
           }
@@ -285,7 +284,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
       const double4 S = a.bS[i];
       f[0] = fma(ti, S.x, f[0]);
       f[1] = fma(ti, S.y, f[1]);
-      f[2] = fma(ti, S.z, f[2]);
+      if (DIM == 3) f[2] = fma(ti, S.z, f[2]);
     }
     double2 c = make_double2(0.0, 0.0);
     if (ADR) {  // g = f + b, and this slice's part of the Rayleigh quotient
@@ -315,12 +314,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
             v = make_double4(0.0, 0.0, 0.0, 0.0);
           }
         } else {
-          v.x = v.x + bp.dt * ((f[0] + bb.x) * bp.inv_rho);
-          v.y = v.y + bp.dt * ((f[1] + bb.y) * bp.inv_rho);
-          v.z = v.z + bp.dt * ((f[2] + bb.z) * bp.inv_rho);
-          u.x = u.x + bp.dt * v.x;
-          u.y = u.y + bp.dt * v.y;
-          u.z = u.z + bp.dt * v.z;
+          explicit_move<DIM>(bp, f, a.bacc ? &bb : nullptr, u, v);
         }
       } else if (fl == 1) {
         u = make_double4(0.0, 0.0, 0.0, u.w);

@@ -75,6 +75,7 @@ __device__ __noinline__ bool fp64_breaks_nl(const StepArgs& a, int64_t i, int32_
 
 // Explicit update (Eq 2.11) with the diagonal mass rho V_i (Eqs 2.1, 2.12) and the boundary
 // conditions at t_{n+1}; f = F_i / V_i.
+template <int DIM>
 __device__ __forceinline__ void update(const StepArgs& a, int64_t i, int b, const double f[3],
                                        const double4* __restrict__ disp, double4* __restrict__ disp_out,
                                        double4& u) {
@@ -89,13 +90,7 @@ __device__ __forceinline__ void update(const StepArgs& a, int64_t i, int b, cons
   u = disp[i];
   double4 v = a.vel[i];
   if (fl == 0) {
-    const double4 bb = a.bacc ? a.bacc[i] : make_double4(0.0, 0.0, 0.0, 0.0);
-    v.x = v.x + bp.dt * ((f[0] + bb.x) * bp.inv_rho);
-    v.y = v.y + bp.dt * ((f[1] + bb.y) * bp.inv_rho);
-    v.z = v.z + bp.dt * ((f[2] + bb.z) * bp.inv_rho);
-    u.x = u.x + bp.dt * v.x;
-    u.y = u.y + bp.dt * v.y;
-    u.z = u.z + bp.dt * v.z;
+    explicit_move<DIM>(bp, f, a.bacc ? a.bacc + i : nullptr, u, v);
   } else if (fl == 1) {
     u = make_double4(0.0, 0.0, 0.0, u.w);
     v = make_double4(0.0, 0.0, 0.0, 0.0);
@@ -230,7 +225,7 @@ __global__ void __launch_bounds__(512) k_pass2_f64(StepArgs a, const double4* __
   split_reduce<SPLIT, 3>(f);
   if (t.active && t.sub == 0) {
     double4 u;
-    update(a, t.i, b, f, disp, disp_out, u);
+    update<DIM>(a, t.i, b, f, disp, disp_out, u);
   }
 }
 
@@ -379,7 +374,7 @@ __global__ void __launch_bounds__(512) k_pass2_nl(StepArgs a, const double4* __r
   split_reduce<SPLIT, 3>(f);
   if (t.active && t.sub == 0) {
     double4 u;
-    update(a, t.i, b, f, disp, disp_out, u);
+    update<DIM>(a, t.i, b, f, disp, disp_out, u);
   }
 }
 
@@ -501,7 +496,7 @@ __global__ void __launch_bounds__(512) k_pass2_nlt(StepArgs a, const double4* __
   split_reduce<SPLIT, 3>(f);
   if (t.active && t.sub == 0) {
     double4 u;
-    update(a, t.i, b, f, disp, disp_out, u);
+    update<DIM>(a, t.i, b, f, disp, disp_out, u);
   }
 }
 
@@ -680,7 +675,7 @@ __global__ void __launch_bounds__(512) k_pass2_nlp(StepArgs a, const double4* __
   split_reduce<SPLIT, 3>(f);
   if (t.active && t.sub == 0) {
     double4 u;
-    update(a, t.i, b, f, disp, disp_out, u);
+    update<DIM>(a, t.i, b, f, disp, disp_out, u);
   }
 }
 
@@ -741,9 +736,10 @@ __global__ void k_bond_tables_nl(StepArgs a, double4* __restrict__ bA) {
 // xi.du (negative values and -0 sort below every positive double), and it runs on the integer pipe
 // instead of the FP64 one.
 
+template <int DIM>
 __global__ void k_bond_sums(StepArgs a) {
   const SliceIdx t = slice_index<1>(a.n_pad, a.slice_ptr);
-  if (t.active) bond_sum_row(a, t);
+  if (t.active) bond_sum_row<DIM>(a, t);
 }
 
 // THETA = false: the failure check alone (applied to the current state before it is read), with no
@@ -763,7 +759,6 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
     const double4 ui = disp[t.i];
     uint32_t* __restrict__ bw = a.bits + (t.base >> 5);
     const int32_t* __restrict__ cl = a.col + t.base + t.lane;
-    const double4* __restrict__ ta = a.bA + t.base + t.lane;
     double* __restrict__ td = a.bd + t.base + t.lane;
     int32_t jn[U];
     uint32_t wn[U];
@@ -778,7 +773,7 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
       for (int u = 0; u < U; ++u) {
         const int k = min(k0 + u * SPLIT, t.W - 1);
         wd[u] = wn[u];
-        g[u] = ta[(int64_t)k << 5];
+        g[u] = slot_row<DIM>(a.bA, a.ne, t.base + t.lane + ((int64_t)k << 5));
         uj[u] = disp[jn[u]];
       }
       load_slots<U, SPLIT>(t, cl, bw, k0 + U * SPLIT, jn, wn);
@@ -814,9 +809,9 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
       const double th = a.aA[t.i] * acc[0];
       const double mu = a.mu[t.i];
       a.theta[t.i] = th;
-      a.thm[t.i] = make_double2(a.bp[b].Kp * (th * mu), a.bp[b].G * mu);
+      a.thm[t.i].x = a.bp[b].Kp * (th * mu);  // all that pass 2 reads
     }
-    if (acc[1] != 0.0) bond_sum_row(a, t);
+    if (acc[1] != 0.0) bond_sum_row<DIM>(a, t);
   }
 }
 
@@ -842,7 +837,7 @@ __global__ void __launch_bounds__(512) k_pass1a_f64p(StepArgs a, const double4* 
   uint32_t* bw = a.bits + (t.base >> 5);
   const int32_t* __restrict__ cl = a.col + t.base + t.lane;
   const int32_t* __restrict__ tw = a.twin + t.base + t.lane;
-  const double4* __restrict__ ta = a.bA + t.base + t.lane;
+  const int64_t e0 = t.base + t.lane;
   double* td = a.bd;
   // the owned-entry streams (index, table row, twin entry) of the next entry are loaded while the
   // current entry's displacement gather and arithmetic run; each lane walks its own owned entries (a
@@ -853,7 +848,7 @@ __global__ void __launch_bounds__(512) k_pass1a_f64p(StepArgs a, const double4* 
   if (mn) {
     const int64_t kn = (int64_t)(own + t.sub) << 5;
     jn = cl[kn];
-    gn = ta[kn];
+    gn = slot_row<DIM>(a.bA, a.ne, e0 + kn);
     ten = tw[kn];
   }
   for (int m = t.sub; m < nown; m += SPLIT) {
@@ -866,7 +861,7 @@ __global__ void __launch_bounds__(512) k_pass1a_f64p(StepArgs a, const double4* 
     if (mn) {
       const int64_t kn = (int64_t)(k + SPLIT) << 5;
       jn = cl[kn];
-      gn = ta[kn];
+      gn = slot_row<DIM>(a.bA, a.ne, e0 + kn);
       ten = tw[kn];
     }
     const int64_t e = t.base + t.lane + ((int64_t)k << 5);
@@ -948,10 +943,10 @@ __global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* 
       const double th = a.aA[t.i] * acc[0];
       const double mu = a.mu[t.i];
       a.theta[t.i] = th;
-      a.thm[t.i] = make_double2(a.bp[b].Kp * (th * mu), a.bp[b].G * mu);
+      a.thm[t.i].x = a.bp[b].Kp * (th * mu);  // all that pass 2 reads
     }
     if (a.dirty[t.i >> 5]) {  // uniform over the warp
-      bond_sum_row(a, t);
+      bond_sum_row<DIM>(a, t);
       __syncwarp();
       if (t.lane == 0) a.dirty[t.i >> 5] = 0;
     }
@@ -1050,7 +1045,7 @@ __global__ void __launch_bounds__(512) k_check_f64p(StepArgs a, const double4* _
   const float4 ui32 = SCREEN ? cu[t.i] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
   uint32_t* bw = a.bits + (t.base >> 5);
   const int32_t* __restrict__ cl = a.col + t.base + t.lane;
-  const double4* __restrict__ ta = a.bA + t.base + t.lane;
+  const int64_t e0 = t.base + t.lane;
   const float4* __restrict__ ts = SCREEN ? cA + t.base + t.lane : nullptr;
   // the next slot's index and table row are loaded while the current slot's gather runs
   int k = k_lo + t.sub;
@@ -1063,7 +1058,7 @@ __global__ void __launch_bounds__(512) k_check_f64p(StepArgs a, const double4* _
     if (SCREEN)
       sn = ts[(int64_t)k << 5];
     else
-      gn = ta[(int64_t)k << 5];
+      gn = slot_row<DIM>(a.bA, a.ne, e0 + ((int64_t)k << 5));
   }
   for (; k < k_hi; k += SPLIT) {
     const uint32_t wd = bw[k];  // this warp's owned bits change only here
@@ -1078,7 +1073,7 @@ __global__ void __launch_bounds__(512) k_check_f64p(StepArgs a, const double4* _
       if (SCREEN)
         sn = ts[(int64_t)kn << 5];
       else
-        gn = ta[(int64_t)kn << 5];
+        gn = slot_row<DIM>(a.bA, a.ne, e0 + ((int64_t)kn << 5));
     }
     bool brk = false;
     if (mine) {
@@ -1098,7 +1093,7 @@ __global__ void __launch_bounds__(512) k_check_f64p(StepArgs a, const double4* _
         exact = !(d + bound < sc.w);
       }
       if (exact) {
-        const double4 g = SCREEN ? ta[(int64_t)k << 5] : g0;
+        const double4 g = SCREEN ? slot_row<DIM>(a.bA, a.ne, e0 + ((int64_t)k << 5)) : g0;
         const double4 uj = disp[j];
         double d = g.x * (uj.x - ui.x) + g.y * (uj.y - ui.y);
         if (DIM == 3) d = fma(g.z, uj.z - ui.z, d);
@@ -1121,10 +1116,11 @@ __global__ void __launch_bounds__(512) k_check_f64p(StepArgs a, const double4* _
 }
 
 // FP32 tables of the screened check: per slot ξ rounded to nearest and s0|ξ|² rounded down.
-__global__ void k_check_tables(int64_t nentries, const double4* __restrict__ bA, float4* __restrict__ cA) {
+template <int DIM>
+__global__ void k_check_tables(int64_t nentries, int64_t ne, const double4* __restrict__ bA, float4* __restrict__ cA) {
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < nentries;
        e += (int64_t)gridDim.x * blockDim.x) {
-    const double4 g = bA[e];
+    const double4 g = slot_row<DIM>(bA, ne, e);
     cA[e] = make_float4(__double2float_rn(g.x), __double2float_rn(g.y), __double2float_rn(g.z),
                         __double2float_rd(g.w));
   }
@@ -1148,7 +1144,6 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
     b = a.body ? a.body[t.i] : 0;
     const uint32_t* __restrict__ bw = a.bits + (t.base >> 5);
     const int32_t* __restrict__ cl = a.col + t.base + t.lane;
-    const double4* __restrict__ tb = a.bB + t.base + t.lane;
     const double* __restrict__ td = a.bd + t.base + t.lane;
     // two slots in flight per warp and half batch: with four the parts of the sums need 77 registers
     constexpr int U = 2, P = 4 / SPLIT, H = P > U ? P / U : 1;
@@ -1166,7 +1161,7 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
         for (int u = 0; u < U; ++u) {
           const int k = min(kh + u * SPLIT, t.W - 1);
           wd[u] = wn[u];
-          g[u] = tb[(int64_t)k << 5];
+          g[u] = slot_row<DIM>(a.bB, a.ne, t.base + t.lane + ((int64_t)k << 5));
           d[u] = td[(int64_t)k << 5];
           tj[u] = a.thm[jn[u]].x;
         }
@@ -1193,9 +1188,9 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
     const double4 S = a.bS[t.i];
     f[0] = fma(ti, S.x, f[0]);
     f[1] = fma(ti, S.y, f[1]);
-    f[2] = fma(ti, S.z, f[2]);
+    if (DIM == 3) f[2] = fma(ti, S.z, f[2]);
     double4 u;
-    update(a, t.i, b, f, disp, disp_out, u);
+    update<DIM>(a, t.i, b, f, disp, disp_out, u);
   }
 }
 
@@ -1220,8 +1215,9 @@ __global__ void k_bond_tables(StepArgs a, double4* __restrict__ bA, double4* __r
     // the stored extension is w xi.du, the theta sum sum w V_j xi.du and the failure test, w > 0,
     // unchanged), w V_j xi and G (1/m_i + 1/m_j) / (w |xi|^2): the step kernels are the same.
     const double w = (wd > 0.0 && q > 0.0) ? wd / sqrt(q) : 1.0;
-    bA[e] = make_double4(w * ex, w * ey, w * ez, w * (s0 * q));
-    bB[e] = make_double4(w * pj.w * ex, w * pj.w * ey, w * pj.w * ez, q > 0.0 ? G * (mi + a.mu[j]) / (w * q) : 0.0);
+    set_slot_row<DIM>(bA, a.ne, e, make_double4(w * ex, w * ey, w * ez, w * (s0 * q)));
+    set_slot_row<DIM>(bB, a.ne, e, make_double4(w * pj.w * ex, w * pj.w * ey, w * pj.w * ez,
+                                                q > 0.0 ? G * (mi + a.mu[j]) / (w * q) : 0.0));
   }
 }
 
@@ -1408,7 +1404,7 @@ __global__ void __launch_bounds__(512) k_pass2_mixed(StepArgs a, const float4* _
   if (t.active && t.sub == 0) {
     const double fd[3] = {(double)f[0], (double)f[1], (double)f[2]};
     double4 u;
-    update(a, t.i, b, fd, disp, disp_out, u);
+    update<DIM>(a, t.i, b, fd, disp, disp_out, u);
     const double sc = a.uscale;
     u32_out[t.i] = make_float4((float)(u.x * sc), (float)(u.y * sc), (float)(u.z * sc), 0.0f);
   }
@@ -1765,7 +1761,7 @@ __global__ void __launch_bounds__(512) k_pass2_mixed_staged(StepArgs a, const fl
   if (ok) {
     const double fd[3] = {(double)f[0], (double)f[1], (double)f[2]};
     double4 u;
-    update(a, t.i, b, fd, disp, disp_out, u);
+    update<DIM>(a, t.i, b, fd, disp, disp_out, u);
     const double sc = a.uscale;
     u32_out[t.i] = make_float4((float)(u.x * sc), (float)(u.y * sc), (float)(u.z * sc), 0.0f);
   }
@@ -1844,7 +1840,7 @@ __device__ __forceinline__ void update_lat(const StepArgs& a, int64_t i, int b, 
   if (a.adr || fl != 0) {
     const double C = bp.lat_C;
     const double fd[3] = {C * (double)f[0], C * (double)f[1], C * (double)f[2]};
-    update(a, i, b, fd, disp, disp_out, u);
+    update<DIM>(a, i, b, fd, disp, disp_out, u);
     return;
   }
   u = disp[i];
@@ -2785,6 +2781,7 @@ StepArgs make_args(pd_ctx* c) {
   a.check = 1;
   a.bA = c->bond_cache ? c->bA : nullptr;
   a.bB = c->bond_cache ? c->bB : nullptr;
+  a.ne = std::max<int64_t>(c->nentries, 32);
   a.bd = c->bond_cache ? c->bd : nullptr;
   a.bS = c->bond_cache ? c->bS : nullptr;
   a.cnt = c->cnt;
@@ -3157,8 +3154,9 @@ pd_status ensure_bond_cache(pd_ctx* c) {
     return PD_OK;
   }
   if (!c->bA) {
-    if ((st = alloc(c, &c->bA, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bB, ne)) != PD_OK) return st;
+    const size_t nt = c->dim == 3 ? ne : (3 * ne + 3) / 4;  // 2D rows: 24 bytes (slot_row)
+    if ((st = alloc(c, &c->bA, nt)) != PD_OK) return st;
+    if ((st = alloc(c, &c->bB, nt)) != PD_OK) return st;
     if ((st = alloc(c, &c->bd, ne)) != PD_OK) return st;
     if ((st = alloc(c, &c->bS, (size_t)c->n_pad)) != PD_OK) return st;
     PD_CUDA(cudaMemsetAsync(c->bd, 0, sizeof(double) * ne, c->stream));  // padding slots stay 0
@@ -3175,7 +3173,8 @@ pd_status ensure_bond_cache(pd_ctx* c) {
     c->bs_stale = true;
   }
   if (c->bs_stale) {
-    k_bond_sums<<<grid, tb, 0, c->stream>>>(make_args(c));
+    if (c->dim == 3) k_bond_sums<3><<<grid, tb, 0, c->stream>>>(make_args(c));
+    else k_bond_sums<2><<<grid, tb, 0, c->stream>>>(make_args(c));
     PD_CUDA(cudaGetLastError());
     c->bs_stale = false;
   }
@@ -3351,7 +3350,9 @@ static void ensure_check_tables(pd_ctx* c) {
   }
   const int tb = 256;
   const unsigned grid = (unsigned)std::min<int64_t>((c->nentries + tb - 1) / tb, 152 * 64);
-  k_check_tables<<<grid, tb, 0, c->stream>>>(c->nentries, c->bA, cA);
+  const int64_t ne = make_args(c).ne;
+  if (c->dim == 3) k_check_tables<3><<<grid, tb, 0, c->stream>>>(c->nentries, ne, c->bA, cA);
+  else k_check_tables<2><<<grid, tb, 0, c->stream>>>(c->nentries, ne, c->bA, cA);
   if (cudaGetLastError() != cudaSuccess) return;
   c->cA32 = cA;
   c->cu32 = cu;
