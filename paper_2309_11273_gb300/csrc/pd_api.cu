@@ -591,6 +591,7 @@ pd_status pd_set_option(pd_ctx* c, int32_t option, int64_t value) {
       if (value < 0 || value > 3) return fail(PD_ERR_ARG, "PD_OPT_LAT_STAGE must be 0, 1, 2 or 3");
       if (c->lat_stage != (int)value) drop_graphs(c);
       c->lat_stage = (int)value;
+      c->auto_map = false;
       break;
     case PD_OPT_SHADOW_LO:
       c->shadow_lo_opt = value != 0;
@@ -980,7 +981,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     c->auto_map = true;
     c->pairs = pairs0;
     // the automatic choice, where it is more than launch shapes: the resident step kernel
-    if (resident_plan(c).split) cands.push_back({block0, split0, pairs0, stage0, true});
+    if (resident_plan(c).split || resident_lat_plan(c).split) cands.push_back({block0, split0, pairs0, stage0, true});
     for (int bl : blocks)
       for (int sp : splits) {
         if ((bl / 32) % sp) continue;

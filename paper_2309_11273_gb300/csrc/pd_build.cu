@@ -637,6 +637,8 @@ pd_status build_lattice(pd_ctx* c, BuildArgs& A, bool* done) {
   if (e != cudaSuccess) return cuda_fail(e, "lattice factors");
   // the common slice width (one family prefix for the whole context), 0 if the widths differ
   c->lat_wuni = (int)((sptr2[1] - sptr2[0]) >> 5);
+  c->lat_wmax = 0;
+  for (int64_t t = 0; t < c->nslices; ++t) c->lat_wmax = std::max(c->lat_wmax, (int)((sptr2[t + 1] - sptr2[t]) >> 5));
   for (int64_t t = 0; t < c->nslices; ++t)
     if ((int)((sptr2[t + 1] - sptr2[t]) >> 5) != c->lat_wuni) c->lat_wuni = 0;
   c->lattice = true;

@@ -213,5 +213,68 @@ __device__ __forceinline__ double2 adr_damping(const double2* part, int64_t nsli
   return c_s;
 }
 
+// xi = x_j - x_i, du = u_j - u_i, d = xi . du, q = xi . xi in FP64.  Shared by the FP64 path and by
+// the FP64 re-decision of the mixed path, so both decide a bond with identical arithmetic.
+template <int DIM>
+__device__ __forceinline__ void bond_f64(const double4& pi, const double4& pj, const double4& ui,
+                                         const double4& uj, double& ex, double& ey, double& ez,
+                                         double& d, double& q) {
+  ex = pj.x - pi.x;
+  ey = pj.y - pi.y;
+  const double dx = uj.x - ui.x, dy = uj.y - ui.y;
+  d = ex * dx + ey * dy;
+  q = ex * ex + ey * ey;
+  if (DIM == 3) {
+    ez = pj.z - pi.z;
+    const double dz = uj.z - ui.z;
+    d = fma(ez, dz, d);
+    q = fma(ez, ez, q);
+  } else {
+    ez = 0.0;
+  }
+}
+
+// FP64 decision of one bond.  Out of line for the general mixed kernels, which call it only for the
+// few bonds inside their rounding band; inlined into the lattice kernel's slow path (fewer registers
+// held across a call in its hot loop).
+template <int DIM>
+__device__ __forceinline__ bool fp64_breaks_inl(const StepArgs& a, int64_t i, int32_t j,
+                                                const double4* __restrict__ disp, double s0) {
+  double ex, ey, ez, d, q;
+  bond_f64<DIM>(a.pos[i], a.pos[j], disp[i], disp[j], ex, ey, ez, d, q);
+  return d >= s0 * q;
+}
+// Explicit update (Eq 2.11) with the diagonal mass rho V_i (Eqs 2.1, 2.12) and the boundary
+// conditions at t_{n+1}; f = F_i / V_i.
+template <int DIM>
+__device__ __forceinline__ void update(const StepArgs& a, int64_t i, int b, const double f[3],
+                                       const double4* __restrict__ disp, double4* __restrict__ disp_out,
+                                       double4& u) {
+  const BodyDev& bp = a.bp[b];
+  if (a.adr) {  // adaptive dynamic relaxation: k_adr_update moves the particles after the reduction
+    const double4 bb = a.bacc ? a.bacc[i] : make_double4(0.0, 0.0, 0.0, 0.0);
+    a.gnew[i] = make_double4(f[0] + bb.x, f[1] + bb.y, f[2] + bb.z, 0.0);
+    u = disp[i];
+    return;
+  }
+  const uint8_t fl = a.flag ? a.flag[i] : (uint8_t)0;
+  u = disp[i];
+  double4 v = a.vel[i];
+  if (fl == 0) {
+    explicit_move<DIM>(bp, f, a.bacc ? a.bacc + i : nullptr, u, v);
+  } else if (fl == 1) {
+    u = make_double4(0.0, 0.0, 0.0, u.w);
+    v = make_double4(0.0, 0.0, 0.0, 0.0);
+  } else {
+    const double t1 = (double)(*a.d_step + 1) * bp.dt;
+    const double4 g = a.gvec[i];
+    const double rt = bp.rate * t1;
+    u = make_double4(rt * g.x, rt * g.y, rt * g.z, u.w);
+    v = make_double4(bp.rate * g.x, bp.rate * g.y, bp.rate * g.z, 0.0);
+  }
+  disp_out[i] = u;  // .w carries V_i unchanged
+  a.vel[i] = v;
+}
+
 }  // namespace
 }  // namespace pd

@@ -243,6 +243,7 @@ struct pd_ctx {
   float4* lat_up = nullptr;       // lattice layout: per particle (u'_i, P_i) from pass 1
   uint8_t* lat_int = nullptr;     // lattice layout: per slice, every N_j = N_ref around it
   int lat_wuni = 0;               // lattice layout: the common slice width (0: widths differ)
+  int lat_wmax = 0;               // lattice layout: the largest slice width
   std::vector<double> lat_h;      // lattice layout: spacing per body
   std::vector<double> lat_nref;   // lattice layout: N_ref per body
   std::vector<int> lat_n1;        // lattice layout: largest |n|_1 of the body's family
@@ -327,6 +328,9 @@ struct ResidentPlan {
 };
 ResidentPlan resident_plan(const pd_ctx* c);
 pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done);
+pd_status upload_resident_tables(int device);  // its copy of the direction tables, at the build
+ResidentPlan resident_lat_plan(const pd_ctx* c);  // mixed form on the lattice layout (pd_resident_lat.cu)
+pd_status run_resident_lat(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done);
 }  // namespace pd
 
 #define PD_CUDA(call)                                        \

@@ -9,13 +9,11 @@
 // k_pass1a_f64p / k_pass1b_f64p / k_pass2_f64t (pair form) or k_pass1_f64t / k_pass2_f64t, with the same
 // order of every sum (parts_sum), so the results are bitwise those of the pass kernels.
 //
-// The barrier is an arrival counter in the context's memory that only grows; every wait is bounded (1 s of
-// the GPU's global timer), and when one expires the block sets the context's error word and an abort word
-// that ends every other wait, and all blocks return: the next pd_sync / pd_get_* reports PD_ERR_TIMEOUT.
 #include <algorithm>
 
 #include "pd_internal.h"
 #include "pd_device.h"
+#include "pd_grid.h"
 
 namespace pd {
 namespace {
@@ -26,8 +24,7 @@ struct ResidentArgs {
   int nsteps;
   int check0;          // the failure check at the head of the first step
   int64_t step0;       // index of the first step
-  unsigned* bar;       // [0] arrivals, [1] abort
-  unsigned bar_base;   // arrivals before this launch
+  GridBar grid;
   int uv;              // every body has one particle volume
   // relaxation solver
   double4* gold;
@@ -35,51 +32,6 @@ struct ResidentArgs {
   double2* part;       // per slice (u.k.u, u.u)
   int* first;
 };
-
-constexpr unsigned kPollLimit = 1u << 26;
-constexpr unsigned long long kBarrierNs = 1000000000ull;
-
-__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ unsigned long long timer_ns() {
-  unsigned long long t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-
-// All blocks of the grid: what any of them wrote before is visible to all of them after.  The fence
-// after the wait drops this SM's cached lines, so plain loads see the other SMs' stores.  False when the
-// wait expired or another block gave up.
-__device__ __forceinline__ bool grid_barrier(const StepArgs& a, const ResidentArgs& r, unsigned& target) {
-  __shared__ int ok_s;
-  target += gridDim.x;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    int ok = 1;
-    __threadfence();
-    // testing (PD_OPT_EXPIRE_WAITS): block 0 never arrives
-    if (!(a.expire && blockIdx.x == 0)) asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(r.bar) : "memory");
-    if ((int)(ld_relaxed(r.bar) - target) < 0) {
-      const unsigned long long t0 = timer_ns();
-      for (unsigned it = 1; (int)(ld_relaxed(r.bar) - target) < 0; ++it) {
-        if ((it & 63u) == 0u &&
-            (ld_relaxed(r.bar + 1) != 0u || timer_ns() - t0 > kBarrierNs || it > kPollLimit)) {
-          ok = 0;
-          atomicExch(r.bar + 1, 1u);
-          atomicExch(&a.counters[4], 1ull);
-          break;
-        }
-      }
-    }
-    __threadfence();
-    ok_s = ok;
-  }
-  __syncthreads();
-  return ok_s != 0;
-}
 
 // PAIR: pass 1 in its pair form (fewer FP64 instructions, one barrier more).  MAXT: the largest block.  Up to
 // 512 threads (128 registers) four slots are in flight per warp and the state stays in registers; up to
@@ -93,8 +45,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   constexpr bool kKeep = MAXT <= 512;  // the particles' state in registers
   constexpr int U = kKeep ? 4 : 2;
   constexpr int H = P > U ? P / U : 1;
-  if (ld_relaxed(r.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
-  unsigned target = r.bar_base;
+  if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
+  unsigned target = r.grid.base;
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   const bool lead = t.active && t.sub == 0;
   const int64_t i = t.active ? t.i : 0, s = i >> 5;
@@ -179,7 +131,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
           }
         }
       }
-      if (!grid_barrier(a, r, target)) return;
+      if (!grid_barrier(a, r.grid, target)) return;
       if (t.active) {
         for (int k0 = t.sub; k0 < t.W; k0 += 4) {  // slots k0, k0 + SPLIT, ...: the sum's parts
 #pragma unroll
@@ -244,7 +196,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
         if (PAIR && t.lane == 0) a.dirty[s] = 0;
       }
     }
-    if (!grid_barrier(a, r, target)) return;
+    if (!grid_barrier(a, r.grid, target)) return;
     // ---- pass 2
     double f[3], part[3][P] = {};
     if (t.active) {
@@ -295,7 +247,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
         const double2 sums = adr_terms(fl == 0 && lam.x > 0.0, u, v, make_double4(f[0], f[1], f[2], 0.0), gold, lam.x);
         if (t.lane == 0) r.part[s] = sums;
       }
-      if (!grid_barrier(a, r, target)) return;
+      if (!grid_barrier(a, r.grid, target)) return;
       c = adr_damping(r.part, a.n_pad >> 5);
     }
     // ---- update (as update() and k_adr_update)
@@ -333,7 +285,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
     if (!kKeep || last) store_state();
     if (last) break;
     slots(t.sub, true);
-    if (!grid_barrier(a, r, target)) return;
+    if (!grid_barrier(a, r.grid, target)) return;
   }
   if (lead && (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z))) atomicExch(&a.counters[5], 1ull);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -392,20 +344,14 @@ ResidentPlan resident_plan(const pd_ctx* c) {
 
 pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done) {
   *done = false;
-  if (!c->bar) {
-    pd_status st = alloc(c, &c->bar, 2);
-    if (st != PD_OK) return st;
-    PD_CUDA(cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
-    c->bar_base = 0;
-  }
+  if (pd_status st = ensure_grid_bar(c); st != PD_OK) return st;
   ResidentArgs r{};
   r.disp = c->disp[c->cur];
   r.disp_out = c->disp[c->cur ^ 1];
   r.nsteps = (int)nsteps;
   r.check0 = check0 ? 1 : 0;
   r.step0 = c->steps;
-  r.bar = c->bar;
-  r.bar_base = c->bar_base;
+  r.grid = GridBar{c->bar, c->bar_base};
   r.uv = c->vol_uniform ? 1 : 0;
   r.gold = c->gold;
   r.lam = c->lam;

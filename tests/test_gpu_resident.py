@@ -5,7 +5,7 @@ barrier wait (GPU only)."""
 import numpy as np
 import pytest
 
-from paper_2309_11273_gb300 import BatchSimulation, PDError, Simulation
+from paper_2309_11273_gb300 import PD_MIXED, PD_W_INV, BatchSimulation, PDError, Simulation
 from paper_2309_11273_gb300 import _binding as B
 from paper_2309_11273_gb300 import workloads as W
 
@@ -81,6 +81,33 @@ def test_batches_and_relaxation():
         sim.set_option(B.PD_OPT_SOLVER, B.PD_SOLVER_ADR)
         return sim
     _same(static, [1, 40, 59])
+
+
+# the mixed form on the lattice layout: one slice, ragged ones, rows in shared memory and through L2 (48- and
+# 124-slot rows on many slices), 512- and 768-thread blocks, the largest resident body and the first beyond
+@pytest.mark.parametrize("lo", [0, 1])
+@pytest.mark.parametrize("nx,ny,ratio", [(5, 5, 3.015), (11, 8, 3.015), (40, 40, 4.015), (279, 278, 3.015),
+                                         (290, 280, 3.015), (341, 340, 4.015), (350, 340, 3.015)])
+def test_mixed_plates_are_bitwise_the_pass_kernels(nx, ny, ratio, lo):
+    def make():
+        sim = Simulation(_plate(nx, ny, ratio), precision=PD_MIXED, shadow_lo=lo)
+        assert sim.get_option(B.PD_OPT_LATTICE) == 1
+        return sim
+    _same(make, [1, 2, 30, 17])
+
+
+@pytest.mark.parametrize("influence", [0, PD_W_INV])
+@pytest.mark.parametrize("shape", [(9, 7, 5), (33, 12, 10), (61, 30, 35), (64, 45, 40)])
+def test_mixed_blocks_are_bitwise_the_pass_kernels(shape, influence):
+    def make():
+        w = W.notched_block(*shape, nsteps=300, seed=5, amp=2e-8, dt=2.5e-7)
+        return Simulation(w, precision=PD_MIXED, influence=influence)
+    _same(make, [1, 25, 24])
+
+
+def test_mixed_impact_and_batch():
+    _same(lambda: Simulation(W.kalthoff(nx=120, ny=61, notch_cells=30.125, gap_cells=30), precision=PD_MIXED), [50, 51])
+    _same(lambda: BatchSimulation(W.plate_batch(nplates=9, side_hi=90), precision=PD_MIXED), [60, 40])
 
 
 def test_switching_between_the_kernels_keeps_the_run():
