@@ -29,31 +29,37 @@ __device__ __forceinline__ unsigned long long timer_ns() {
   return t;
 }
 
-// All blocks of the grid: what any of them wrote before is visible to all of them after.  The fence
-// after the wait drops this SM's cached lines, so plain loads see the other SMs' stores.  False when the
-// wait expired or another block gave up.
+__device__ __forceinline__ unsigned ld_acquire(const unsigned* p) {
+  unsigned v;
+  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+
+// All blocks of the grid: what any of them wrote before is visible to all of them after.  One thread of a
+// block arrives with release and polls with acquire order, between two block barriers, so that the block's
+// plain stores before and plain loads after are ordered too.  (A full fence on each side of the wait, and
+// the timer read at its start, cost a step of a one-slice body 7.4 us where this takes 6.5 us.)  False
+// when the wait expired or another block gave up.
 __device__ __forceinline__ bool grid_barrier(const StepArgs& a, const GridBar& r, unsigned& target) {
   __shared__ int ok_s;
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
     int ok = 1;
-    __threadfence();
     // testing (PD_OPT_EXPIRE_WAITS): block 0 never arrives
-    if (!(a.expire && blockIdx.x == 0)) asm volatile("red.relaxed.gpu.global.add.u32 [%0], 1;" ::"l"(r.bar) : "memory");
-    if ((int)(ld_relaxed(r.bar) - target) < 0) {
-      const unsigned long long t0 = timer_ns();
-      for (unsigned it = 1; (int)(ld_relaxed(r.bar) - target) < 0; ++it) {
-        if ((it & 63u) == 0u &&
-            (ld_relaxed(r.bar + 1) != 0u || timer_ns() - t0 > kBarrierNs || it > kPollLimit)) {
-          ok = 0;
-          atomicExch(r.bar + 1, 1u);
-          atomicExch(&a.counters[4], 1ull);
-          break;
-        }
+    if (!(a.expire && blockIdx.x == 0)) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(r.bar) : "memory");
+    unsigned long long t0 = 0ull;
+    for (unsigned it = 1; (int)(ld_acquire(r.bar) - target) < 0; ++it) {
+      if ((it & 255u) != 0u) continue;
+      const unsigned long long now = timer_ns();
+      if (t0 == 0ull) t0 = now;
+      if (ld_relaxed(r.bar + 1) != 0u || now - t0 > kBarrierNs || it > kPollLimit) {
+        ok = 0;
+        atomicExch(r.bar + 1, 1u);
+        atomicExch(&a.counters[4], 1ull);
+        break;
       }
     }
-    __threadfence();
     ok_s = ok;
   }
   __syncthreads();

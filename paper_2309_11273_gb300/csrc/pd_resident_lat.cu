@@ -34,7 +34,8 @@ constexpr int kLatRowSmem = 200 * 1024;  // shared memory for the rows of a bloc
 template <int DIM, bool WI, bool LO, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) {
   extern __shared__ __align__(128) unsigned char smem[];
-  constexpr int NB = MAXT <= 512 && !LO ? 2 : 1;
+  constexpr bool kKeep = MAXT <= 512;  // the FP64 state in registers
+  constexpr int NB = !LO ? 2 : 1;
   constexpr int U = 4;
   if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
   unsigned target = r.grid.base;
@@ -61,7 +62,7 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) 
   const float2 lf = t.active ? a.lat_f[i] : make_float2(0.0f, 0.0f);  // (N_ref / N_i, A / N_i)
   const bool interior = t.active && a.lat_int[i >> 5] != 0;           // uniform over the warp
   double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u;
-  if (t.active) {
+  if (kKeep && t.active) {
     u = r.disp[0][i];
     v = a.vel[i];
   }
@@ -231,6 +232,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) 
       if (interior) row(std::true_type{});
       else row(std::false_type{});
       // update (update_lat, update)
+      if (!kKeep) {
+        u = disp[i];
+        v = a.vel[i];
+      }
       if (fl == 0) {
         const double K = bp.lat_K, dt = bp.dt;
         v.x = fma(K, (double)f[0], v.x);
@@ -267,13 +272,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) 
       }
       (cur ? r.u32[0] : r.u32[1])[i] = hi;
       lat_raise_umax(umax_next, b, hi.w);
+      if (!kKeep || last) a.vel[i] = v;
     }
     if (!last && !grid_barrier(a, r.grid, target)) return;
   }
-  if (t.active) {
-    a.vel[i] = v;
-    if (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z)) atomicExch(&a.counters[5], 1ull);
-  }
+  if (t.active && (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z))) atomicExch(&a.counters[5], 1ull);
   if (blockIdx.x == 0 && threadIdx.x == 0) *a.d_step = r.step0 + r.nsteps - 1;
 }
 
