@@ -233,6 +233,16 @@ PD_LHD float lat_max_nan(float a, float b) {
   return (a != a || b != b) ? NAN : (a > b ? a : b);
 #endif
 }
+// The largest of three (one instruction), NaN if any is.
+PD_LHD float lat_max3_nan(float a, float b, float c) {
+#if defined(__CUDA_ARCH__)
+  float r;
+  asm("max.NaN.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
+#else
+  return lat_max_nan(lat_max_nan(a, b), c);
+#endif
+}
 
 // Full band: 0 intact, 1 broken (FP32 decision), 2 inside the band (decide in FP64).  A NaN g is
 // inside (both comparisons false).

@@ -118,8 +118,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) 
                                                    lat_delta_lo(Uj[h][q].z, Lj[h][q].z, Ui.z, Li.z))
                                : lat_dprime_pair<DIM>(dn, Uj[h][q], nUi);
             dm[q] = (wd[q] & lmask) ? d : 0.0f;
-            gmax = lat_max_nan(gmax, lat_g(dm[q], s0f, dn.w));
           }
+          gmax = lat_max3_nan(gmax, lat_g(lat_max_nan(dm[0], dm[1]), s0f, dA.w), lat_g(lat_max_nan(dm[2], dm[3]), s0f, dB.w));
           if (__any_sync(kFull, !(gmax + scr_i < 0.0f))) {
             // full band for the bonds the screen did not settle, FP64 inside it
             unsigned brk = 0u;
