@@ -33,8 +33,21 @@ struct ResidentArgs {
   int* first;
 };
 
+// A line of a static stream to L2, some batches before its load.
+__device__ __forceinline__ void to_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+template <int DIM>
+__device__ __forceinline__ void row_to_l2(const double4* table, int64_t ne, int64_t e) {
+  if (DIM == 3) {
+    to_l2(table + e);
+  } else {
+    to_l2(reinterpret_cast<const double2*>(table) + e);
+    to_l2(reinterpret_cast<const double*>(table) + 2 * ne + e);
+  }
+}
+
 // PAIR: pass 1 in its pair form (fewer FP64 instructions, one barrier more).  MAXT: the largest block.  Up to
-// 512 threads (128 registers) four slots are in flight per warp and the state stays in registers; up to
+// 512 threads (128 registers) four slots are in flight per warp (eight up to 256 threads without the pair
+// form) and the state stays in registers; up to
 // 768 (80 registers) two, and the state is read again at the update.  Without the pair form, on the
 // smallest bodies, the neighbour indices are loaded a batch ahead, and a pass's first ones before the
 // barrier in front of it, so that a batch waits for one round trip to L2 instead of two (40 x 40 plate 9.7
@@ -43,8 +56,12 @@ template <int DIM, int SPLIT, bool PAIR, bool ADR, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r) {
   constexpr int P = 4 / SPLIT;
   constexpr bool kKeep = MAXT <= 512;  // the particles' state in registers
-  constexpr int U = kKeep ? 4 : 2;
+  constexpr int U = MAXT <= 256 && !PAIR && !ADR ? 8 : (kKeep ? 4 : 2);
   constexpr int H = P > U ? P / U : 1;
+  // Batches of the static streams fetched to L2 ahead: in 3D they do not stay there from step to step, and each
+  // batch waited for its indices and then its rows from memory (relaxation of 45,000 particles 134.8 -> 124.4 us
+  // per step with 2, 129.9 with 4, 139.4 with 8, which push each other out).
+  constexpr int kAhead = PAIR && DIM == 3 ? 2 : 0;
   if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
   unsigned target = r.grid.base;
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
@@ -114,6 +131,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
             g[q] = slot_row<DIM>(a.bA, a.ne, e0 + k);
             uj[q] = disp[j[q]];
           }
+          if (kAhead > 0)
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+              const int64_t k = (int64_t)min(own + m0 + (q + kAhead * U) * SPLIT, max(cnt - 1, 0)) << 5;
+              to_l2(cl + k);
+              to_l2(tw + k);
+              row_to_l2<DIM>(a.bA, a.ne, e0 + k);
+            }
 #pragma unroll
           for (int q = 0; q < U; ++q) {
             const int k = own + m0 + q * SPLIT;
@@ -216,6 +241,14 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
             d[q] = td[(int64_t)k << 5];
             tj[q] = a.thm[jn[q]].x;
           }
+          if (kAhead > 0)
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+              const int64_t k = (int64_t)min(k0 + (q + kAhead * U) * SPLIT, t.W - 1) << 5;
+              to_l2(cl + k);
+              to_l2(td + k);
+              row_to_l2<DIM>(a.bB, a.ne, e0 + k);
+            }
           slots(k0 + U * SPLIT, true);
 #pragma unroll
           for (int q = 0; q < U; ++q) {
@@ -306,7 +339,8 @@ cudaError_t launch(pd_ctx* c, StepArgs a, ResidentArgs r, unsigned grid, int blo
 template <int DIM, int SPLIT>
 cudaError_t launch_form(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, unsigned grid, int block, bool pair) {
   if (block > 512) return launch<DIM, SPLIT, true, 768>(c, a, r, grid, block);
-  return pair ? launch<DIM, SPLIT, true, 512>(c, a, r, grid, block) : launch<DIM, SPLIT, false, 512>(c, a, r, grid, block);
+  if (pair) return launch<DIM, SPLIT, true, 512>(c, a, r, grid, block);
+  return block > 256 ? launch<DIM, SPLIT, false, 512>(c, a, r, grid, block) : launch<DIM, SPLIT, false, 256>(c, a, r, grid, block);
 }
 
 template <int DIM>
@@ -324,13 +358,15 @@ ResidentPlan resident_plan(const pd_ctx* c) {
   if (!c->auto_map || c->precision != PD_FP64 || c->kin != PD_LINEARIZED || !c->bond_cache || !c->pairs || !c->pairs_ok ||
       c->profile || c->sms <= 0)
     return p;
-  // Warps per slice: four while that leaves an SM at most 16 warps (128 registers each), two up to 20, one up
-  // to 24 (80 registers); beyond, the pass kernels with their own balance over waves are the faster ones.
+  // Warps per slice: four while that leaves an SM at most 16 warps (128 registers each), two up to 20, in 2D
+  // one up to 24 (80 registers).  Beyond, the pass kernels are the faster ones (us per step, resident against
+  // pass kernels: plates of 250^2 32 / 41, 340^2 59 / 70; blocks of 34^3 112 / 115, with one warp per slice
+  // 40^3 163 / 155).
   const int64_t ns = c->nslices, sms = c->sms;
   int split = 0;
   if (ns * 4 <= sms * 16) split = 4;
   else if (ns * 2 <= sms * 20) split = 2;
-  else if (ns <= sms * 24) split = 1;
+  else if (ns <= sms * 24 && c->dim == 2) split = 1;
   if (!split) return p;
   // One block per SM; a slice's warps share a block (parts_across).
   int64_t warps = (ns * split + sms - 1) / sms;

@@ -30,12 +30,14 @@ struct LatRun {
 
 constexpr int kLatRowSmem = 200 * 1024;  // shared memory for the rows of a block
 
-// MAXT: the largest block; up to 512 threads (128 registers) the gathers of two batches are in flight.
+// MAXT: the largest block.  A warp keeps the gathers of NB batches of four slots in flight: four up to 256
+// threads (255 registers), else two (one with the two-word shadow); the FP64 state stays in registers up to
+// 512 threads and is read again at the update beyond.
 template <int DIM, bool WI, bool LO, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) {
   extern __shared__ __align__(128) unsigned char smem[];
   constexpr bool kKeep = MAXT <= 512;  // the FP64 state in registers
-  constexpr int NB = !LO ? 2 : 1;
+  constexpr int NB = MAXT <= 256 ? 4 : (LO ? 1 : 2);
   constexpr int U = 4;
   if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
   unsigned target = r.grid.base;
@@ -293,8 +295,12 @@ cudaError_t launch(pd_ctx* c, StepArgs a, LatRun r, unsigned grid, int block) {
 template <int DIM, bool WI>
 cudaError_t launch_form(pd_ctx* c, const StepArgs& a, const LatRun& r, unsigned grid, int block) {
   if (c->shadow_lo)
-    return block > 512 ? launch<DIM, WI, true, 768>(c, a, r, grid, block) : launch<DIM, WI, true, 512>(c, a, r, grid, block);
-  return block > 512 ? launch<DIM, WI, false, 768>(c, a, r, grid, block) : launch<DIM, WI, false, 512>(c, a, r, grid, block);
+    return block > 512   ? launch<DIM, WI, true, 768>(c, a, r, grid, block)
+           : block > 256 ? launch<DIM, WI, true, 512>(c, a, r, grid, block)
+                         : launch<DIM, WI, true, 256>(c, a, r, grid, block);
+  return block > 512   ? launch<DIM, WI, false, 768>(c, a, r, grid, block)
+         : block > 256 ? launch<DIM, WI, false, 512>(c, a, r, grid, block)
+                       : launch<DIM, WI, false, 256>(c, a, r, grid, block);
 }
 
 }  // namespace

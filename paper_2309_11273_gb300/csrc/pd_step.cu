@@ -2636,7 +2636,12 @@ cudaEvent_t take_event(pd_ctx* c) {
 // kSplit1a warps per slice in the pair forms' pass 1a, which sums nothing, so that its results do not
 // depend on the split (nonlinear: 1.405 -> 1.34 ms).
 constexpr int kAutoBlock64 = 64;
-constexpr int kAutoSplit64 = 2;  // linearized, tabled: any split gives the same sums
+// Split of the linearized tabled kernels (any split gives the same sums): two warps per slice, and in 3D
+// four, in 128-thread blocks, where two would end in a partial second wave (48^3 particles 272 -> 243 us
+// per step; one wave at 40^3 155 against 163, many at 1M particles 1766 against 1777).
+inline int auto_split64(const pd_ctx* c) {
+  return c->dim == 3 && c->nslices * 2 > (int64_t)c->sms * 32 && c->nslices <= 16000 ? 4 : 2;
+}
 constexpr int kSplit1aL = 2, kBlock1aL = 64;    // linearized
 constexpr int kSplit1aNL = 4, kBlock1aNL = 128;  // nonlinear
 
@@ -2842,8 +2847,10 @@ namespace {
 
 template <int DIM>
 void dispatch_pass(pd_ctx* c, const StepArgs& a, int pass, int write_theta) {
-  const int block = !c->auto_map ? c->block : (c->precision == PD_FP64 ? kAutoBlock64 : (c->lattice ? kAutoBlockLat : c->block));
-  const int split = c->auto_map && c->precision == PD_FP64 && c->kin == PD_LINEARIZED && a.bA ? kAutoSplit64 : c->split;
+  const int split = c->auto_map && c->precision == PD_FP64 && c->kin == PD_LINEARIZED && a.bA ? auto_split64(c) : c->split;
+  int block = c->block;
+  if (c->auto_map && c->precision == PD_FP64) block = split == 4 ? 2 * kAutoBlock64 : kAutoBlock64;
+  else if (c->auto_map && c->lattice) block = kAutoBlockLat;
   const int64_t threads = c->nslices * 32 * (int64_t)split;
   const unsigned grid = (unsigned)((threads + block - 1) / block);
   if (c->precision == PD_MIXED && c->lattice) {
