@@ -1,5 +1,9 @@
 // extern "C" entry points of libosbpd (declared and documented in include/osbpd.h).
+#include <sys/mman.h>
+#include <unistd.h>
+
 #include <algorithm>
+#include <cerrno>
 #include <chrono>
 #include <cmath>
 #include <cstdio>
@@ -144,6 +148,23 @@ pd_status ensure_xfer(pd_ctx* c) {
     return cuda_fail(e, "cudaEventCreateWithFlags");
   }
   return PD_OK;
+}
+
+// Brings the pages of a large output array into memory while the GPU still works on what was enqueued before
+// (their contents do not change).  A fresh allocation of that size has none yet, and the copy into it would
+// fault them in one by one after the GPU has finished (3.5M particles: 7.6 ms of a read, 50 steps and a read
+// 54.1 -> 50.6 ms; 1.2M particles of batched plates 12.3 -> 10.4 ms).  Best effort: an error changes nothing.
+void populate(void* p, size_t bytes) {
+  constexpr size_t kLeast = (size_t)4 << 20;
+#ifndef MADV_POPULATE_WRITE
+#define MADV_POPULATE_WRITE 23
+#endif
+  if (!p || bytes < kLeast) return;
+  const uintptr_t page = (uintptr_t)sysconf(_SC_PAGESIZE);
+  const uintptr_t a = (uintptr_t)p & ~(page - 1), e = ((uintptr_t)p + bytes + page - 1) & ~(page - 1);
+  const int keep = errno;
+  madvise((void*)a, e - a, MADV_POPULATE_WRITE);
+  errno = keep;
 }
 
 pd_status check_ctx(pd_ctx* c, bool need_built) {
@@ -444,6 +465,12 @@ pd_status pd_get_damage(pd_ctx* c, double* phi) {
 pd_status pd_get_state(pd_ctx* c, double* u, double* v, double* theta) {
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
+  if (cudaStreamQuery(c->stream) == cudaErrorNotReady) {  // the GPU still steps
+    cudaGetLastError();
+    populate(u, sizeof(double) * c->dim * c->n);
+    populate(v, sizeof(double) * c->dim * c->n);
+    populate(theta, sizeof(double) * c->n);
+  }
   if ((st = check_device_error(c)) != PD_OK) return st;
   if ((st = ensure_xfer(c)) != PD_OK) return st;
   // u, v and theta do not depend on the bond status, so their copies run on the transfer stream,
