@@ -136,14 +136,17 @@ typedef struct {
 
 /* Options for pd_set_option / pd_get_option. */
 typedef enum {
-  PD_OPT_GRAPH_CHUNK = 1,  /* steps captured per CUDA graph launch (0: no graphs). Default 100.  PD_FP64
-                              bodies with linearized bonds that fit the GPU in one wave (up to about
-                              115,000 particles) take all steps of a call in one cooperative launch
-                              instead, while no launch mapping was chosen (PD_OPT_BLOCK, PD_OPT_SPLIT) */
+  PD_OPT_GRAPH_CHUNK = 1,  /* steps captured per CUDA graph launch (0: no graphs). Default 100.  Bodies
+                              with linearized bonds that fit the GPU in one wave (explicit solver; PD_FP64
+                              up to about 115,000 particles in 2D and 48,000 in 3D, PD_MIXED on the
+                              lattice layout up to 117,000) take all steps of a call in one cooperative
+                              launch instead, while no launch mapping was chosen (PD_OPT_BLOCK,
+                              PD_OPT_SPLIT, PD_OPT_LAT_STAGE); results are bitwise the same */
   PD_OPT_PROFILE = 2,      /* 1: time every kernel launch with CUDA events (forces eager launches) */
   PD_OPT_VALIDATE = 3,     /* PD_MIXED: 1 = also decide every bond in FP64 and count mismatches */
   PD_OPT_BLOCK = 4,        /* threads per block of the step kernels (multiple of 32, <= 512); until it or
-                              PD_OPT_SPLIT is set, each PD_FP64 kernel takes a shape of its own */
+                              PD_OPT_SPLIT is set, the PD_FP64 and the lattice kernels take shapes of
+                              their own */
   PD_OPT_SPLIT = 5,        /* warps cooperating on one 32-particle slice: 1, 2 or 4 */
   PD_OPT_BOND_CACHE = 6,   /* PD_FP64: 1 (default) = keep per-bond tables of the reference
                               geometry and bond coefficients (xi, s0 |xi|^2, V_j xi,
@@ -162,8 +165,8 @@ typedef enum {
                               do not issue each warp's first index copy, so its bounded wait (1 s
                               of the GPU's global timer) expires; the warps skip their outputs
                               and the next pd_sync / pd_get_* returns PD_ERR_TIMEOUT.  In the
-                              resident FP64 kernel a block does not arrive at the grid barrier, with
-                              the same end.  Default 0. */
+                              resident kernels (PD_OPT_GRAPH_CHUNK) a block does not arrive at the grid
+                              barrier, with the same end after 4 s.  Default 0. */
   PD_OPT_SOLVER = 9,       /* pd_solver: PD_SOLVER_EXPLICIT (0, default) or PD_SOLVER_ADR (1) */
   PD_OPT_PAIRS = 10,       /* PD_FP64 with the bond cache on: 1 (default) = form each bond's
                               extension (linearized: xi.(u_j - u_i); nonlinear: e and 1/|Y|) and

@@ -62,13 +62,14 @@ __device__ __forceinline__ void split_reduce(T (&v)[NC]) {
 // The sums of the tabled FP64 kernels run in four parts, slot k in part k mod 4, combined as (0 + 2) +
 // (1 + 3) whatever the number of warps that share a slice: a warp holds 4 / SPLIT of them, so the result
 // is bitwise the same for every split (and four independent chains of FP64 additions are shorter).
-template <int SPLIT, int NC>
-__device__ __forceinline__ void parts_sum(const double (&p)[NC][4 / SPLIT], double (&v)[NC]) {
+// P = 1 with one warp per slice: the plain sum in slot order, which the relaxation solver keeps (block_tree).
+template <int SPLIT, int NC, int P = 4 / SPLIT>
+__device__ __forceinline__ void parts_sum(const double (&p)[NC][P], double (&v)[NC]) {
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    if constexpr (SPLIT == 1) v[c] = (p[c][0] + p[c][2]) + (p[c][1] + p[c][3]);
-    else if constexpr (SPLIT == 2) v[c] = p[c][0] + p[c][1];
-    else v[c] = p[c][0];
+    if constexpr (P == 1) v[c] = p[c][0];
+    else if constexpr (SPLIT == 1) v[c] = (p[c][0] + p[c][2]) + (p[c][1] + p[c][3]);
+    else v[c] = p[c][0] + p[c][1];
   }
 }
 // ... and across the warps of the slice (their parts combined by the first warp).
@@ -143,74 +144,6 @@ __device__ __forceinline__ void bond_sum_row(const StepArgs& a, const SliceIdx& 
     }
   }
   a.bS[t.i] = make_double4(sx, sy, sz, 0.0);
-}
-
-// Relaxation solver: a slice's sums of u (k u) and u u over its free particles' components, k =
-// -(g - g_prev) / (lambda v), in lane 0 of the warp.
-__device__ __forceinline__ double2 adr_terms(bool free, const double4& u, const double4& v, const double4& g,
-                                             const double4& gp, double lam) {
-  double num = 0.0, den = 0.0;
-  if (free) {
-    const double uu[3] = {u.x, u.y, u.z}, vv[3] = {v.x, v.y, v.z}, gg[3] = {g.x, g.y, g.z}, go[3] = {gp.x, gp.y, gp.z};
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const double kk = vv[k] != 0.0 ? -(gg[k] - go[k]) / (lam * vv[k]) : 0.0;
-      num += uu[k] * kk * uu[k];
-      den += uu[k] * uu[k];
-    }
-  }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    num += __shfl_down_sync(kFull, num, o);
-    den += __shfl_down_sync(kFull, den, o);
-  }
-  return make_double2(num, den);
-}
-
-// v^{n+1/2} of one component: ((2 - c) v^{n-1/2} + 2 g / lambda) / (2 + c), from rest on a start g / (2 lambda),
-// with the stored reciprocals 1 / lambda and 1 / (2 + c) (the contraction written out: both kernels that
-// relax round alike).
-__device__ __forceinline__ double adr_velocity(double v, double g, double inv_lam, double c, double inv_2c, bool start) {
-  return start ? g * (0.5 * inv_lam) : fma(2.0 - c, v, g * (2.0 * inv_lam)) * inv_2c;
-}
-
-// The damping c = 2 sqrt(u.k.u / u.u) (0 unless both are positive) and 1 / (2 + c) from the slices' sums,
-// for every thread of the block: 1024 strided sums, combined by warps of them, in the same order whatever
-// the block's size.
-__device__ __forceinline__ double2 adr_damping(const double2* part, int64_t nslices) {
-  __shared__ double wn[32], wd[32];
-  __shared__ double2 c_s;
-  for (int v = threadIdx.x; v < 1024; v += blockDim.x) {  // whole warps
-    double num = 0.0, den = 0.0;
-    for (int64_t k = v; k < nslices; k += 1024) {
-      num += part[k].x;
-      den += part[k].y;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      num += __shfl_down_sync(kFull, num, o);
-      den += __shfl_down_sync(kFull, den, o);
-    }
-    if ((v & 31) == 0) {
-      wn[v >> 5] = num;
-      wd[v >> 5] = den;
-    }
-  }
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    double num = wn[threadIdx.x], den = wd[threadIdx.x];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      num += __shfl_down_sync(kFull, num, o);
-      den += __shfl_down_sync(kFull, den, o);
-    }
-    if (threadIdx.x == 0) {
-      const double c = (den > 0.0 && num > 0.0) ? 2.0 * sqrt(num / den) : 0.0;
-      c_s = make_double2(c, 1.0 / (2.0 + c));
-    }
-  }
-  __syncthreads();
-  return c_s;
 }
 
 // xi = x_j - x_i, du = u_j - u_i, d = xi . du, q = xi . xi in FP64.  Shared by the FP64 path and by

@@ -1,6 +1,6 @@
 // Grid barrier of the resident step kernels (cooperative launches: every block of the grid is resident).
 //
-// An arrival counter in the context's memory that only grows; every wait is bounded (1 s of the GPU's
+// An arrival counter in the context's memory that only grows; every wait is bounded (4 s of the GPU's
 // global timer), and when one expires the block sets the context's error word and an abort word that ends
 // every other wait, and all blocks return: the next pd_sync / pd_get_* reports PD_ERR_TIMEOUT.
 #pragma once
@@ -16,7 +16,7 @@ struct GridBar {
 };
 
 constexpr unsigned kPollLimit = 1u << 26;
-constexpr unsigned long long kBarrierNs = 1000000000ull;
+constexpr unsigned long long kBarrierNs = 4000000000ull;  // other work on the GPU may hold a block back for a while
 
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p) {
   unsigned v;

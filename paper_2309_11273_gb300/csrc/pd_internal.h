@@ -230,7 +230,7 @@ struct pd_ctx {
   double2* lam = nullptr;         // ADR fictitious density (lambda_i, 1 / lambda_i)
   double4* gnew = nullptr;        // ADR g^n (force density incl. body force)
   double4* gold = nullptr;        // ADR g^{n-1}
-  double2* adr_part = nullptr;    // ADR per-slice partial sums (u.k.u, u.u)
+  double2* adr_part = nullptr;    // ADR per-block partial sums (u.k.u, u.u)
   double4* adr_st = nullptr;      // ADR (c^n, start flag, 1 / (2 + c^n)) of the current iteration
   int* adr_first = nullptr;       // ADR: 1 = the next iteration starts from rest
   double* diag_theta = nullptr;   // pd_get_stats: theta at the current state

@@ -2,13 +2,13 @@
 // one cooperative launch.
 //
 // On a body of up to about a hundred thousand particles a step of the pass kernels is shorter than what
-// surrounds it: three launches (six with the relaxation solver), each with its ramp up and its last warps,
-// and per launch the chain index -> gather -> sum of a slice's row.  Here one block per SM holds its
-// slices for the whole call; the displacements and velocities of its particles stay in registers, and the
-// passes are separated by a grid barrier (about 1.5 us) instead of a launch.  The arithmetic is that of
+// surrounds it: three launches, each with its ramp up and its last warps, and per launch the chain index ->
+// gather -> sum of a slice's row.  Here one block per SM holds its slices for the whole call; the
+// displacements and velocities of its particles stay in registers, and the passes are separated by a grid
+// barrier (about 1.3 us) instead of a launch: a 40 x 40 plate 33.7 -> 8.7 us per step (100 steps and a read), a
+// 400 x 160 plate 64 -> 36 us, bound there by the FP64 pipe (60 %) and the passes' ramps.  The arithmetic is that of
 // k_pass1a_f64p / k_pass1b_f64p / k_pass2_f64t (pair form) or k_pass1_f64t / k_pass2_f64t, with the same
 // order of every sum (parts_sum), so the results are bitwise those of the pass kernels.
-//
 #include <algorithm>
 
 #include "pd_internal.h"
@@ -26,11 +26,6 @@ struct ResidentArgs {
   int64_t step0;       // index of the first step
   GridBar grid;
   int uv;              // every body has one particle volume
-  // relaxation solver
-  double4* gold;
-  const double2* lam;
-  double2* part;       // per slice (u.k.u, u.u)
-  int* first;
 };
 
 // A line of a static stream to L2, some batches before its load.
@@ -52,15 +47,15 @@ __device__ __forceinline__ void row_to_l2(const double4* table, int64_t ne, int6
 // smallest bodies, the neighbour indices are loaded a batch ahead, and a pass's first ones before the
 // barrier in front of it, so that a batch waits for one round trip to L2 instead of two (40 x 40 plate 9.7
 // -> 9.1 us per step); the pair form spills with it (400 x 160 plate 39.8 -> 41.3 us).
-template <int DIM, int SPLIT, bool PAIR, bool ADR, int MAXT>
+template <int DIM, int SPLIT, bool PAIR, int MAXT>
 __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r) {
   constexpr int P = 4 / SPLIT;
   constexpr bool kKeep = MAXT <= 512;  // the particles' state in registers
-  constexpr int U = MAXT <= 256 && !PAIR && !ADR ? 8 : (kKeep ? 4 : 2);
+  constexpr int U = MAXT <= 256 && !PAIR ? 8 : (kKeep ? 4 : 2);
   constexpr int H = P > U ? P / U : 1;
   // Batches of the static streams fetched to L2 ahead: in 3D they do not stay there from step to step, and each
-  // batch waited for its indices and then its rows from memory (relaxation of 45,000 particles 134.8 -> 124.4 us
-  // per step with 2, 129.9 with 4, 139.4 with 8, which push each other out).
+  // batch waited for its indices and then its rows from memory (a 45,000-particle block 134.8 -> 124.4 us per
+  // iteration with 2, 129.9 with 4, 139.4 with 8, which push each other out).
   constexpr int kAhead = PAIR && DIM == 3 ? 2 : 0;
   if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
   unsigned target = r.grid.base;
@@ -78,24 +73,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   const int64_t e0 = t.base + t.lane;
   double* td = a.bd + t.base + t.lane;
   const uint8_t fl = lead && a.flag ? a.flag[i] : (uint8_t)0;
-  double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u, gold = u, bb = u;
-  double2 lam = make_double2(0.0, 0.0);
+  double4 u = make_double4(0.0, 0.0, 0.0, 0.0), v = u, bb = u;
   auto load_state = [&](const double4* disp) {  // of the slice's first warp
     if (!lead) return;
     u = disp[i];
     v = a.vel[i];
     if (a.bacc) bb = a.bacc[i];
-    if (ADR) {
-      gold = r.gold[i];
-      lam = r.lam[i];
-    }
   };
-  auto store_state = [&]() {
-    if (!lead) return;
-    a.vel[i] = v;
-    if (ADR) r.gold[i] = gold;
-  };
-  const bool start0 = ADR && *r.first != 0;
   if (kKeep) load_state(r.disp);
   if (lead && a.dirty[s]) {  // bonds broken by a check between calls
     bond_sum_row<DIM>(a, t);
@@ -271,36 +255,10 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
       f[1] = fma(ti, S.y, f[1]);
       if (DIM == 3) f[2] = fma(ti, S.z, f[2]);
     }
-    double2 c = make_double2(0.0, 0.0);
-    if (ADR) {  // g = f + b, and this slice's part of the Rayleigh quotient
-      if (lead) {
-        f[0] += bb.x;
-        f[1] += bb.y;
-        f[2] += bb.z;
-        const double2 sums = adr_terms(fl == 0 && lam.x > 0.0, u, v, make_double4(f[0], f[1], f[2], 0.0), gold, lam.x);
-        if (t.lane == 0) r.part[s] = sums;
-      }
-      if (!grid_barrier(a, r.grid, target)) return;
-      c = adr_damping(r.part, a.n_pad >> 5);
-    }
-    // ---- update (as update() and k_adr_update)
+    // ---- update (as update())
     if (lead) {
       if (fl == 0) {
-        if (ADR) {
-          if (lam.x > 0.0) {
-            const bool start = start0 && step == 0;
-            v.x = adr_velocity(v.x, f[0], lam.y, c.x, c.y, start);
-            v.y = adr_velocity(v.y, f[1], lam.y, c.x, c.y, start);
-            v.z = adr_velocity(v.z, f[2], lam.y, c.x, c.y, start);
-            u.x = u.x + v.x;
-            u.y = u.y + v.y;
-            u.z = u.z + v.z;
-          } else {
-            v = make_double4(0.0, 0.0, 0.0, 0.0);
-          }
-        } else {
-          explicit_move<DIM>(bp, f, a.bacc ? &bb : nullptr, u, v);
-        }
+        explicit_move<DIM>(bp, f, a.bacc ? &bb : nullptr, u, v);
       } else if (fl == 1) {
         u = make_double4(0.0, 0.0, 0.0, u.w);
         v = make_double4(0.0, 0.0, 0.0, 0.0);
@@ -312,10 +270,9 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
         v = make_double4(bp.rate * g.x, bp.rate * g.y, bp.rate * g.z, 0.0);
       }
       disp_out[i] = u;  // .w carries V_i unchanged
-      if (ADR) gold = make_double4(f[0], f[1], f[2], 0.0);
     }
     const bool last = step + 1 == r.nsteps;
-    if (!kKeep || last) store_state();
+    if (lead && (!kKeep || last)) a.vel[i] = v;
     if (last) break;
     slots(t.sub, true);
     if (!grid_barrier(a, r.grid, target)) return;
@@ -323,7 +280,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   if (lead && (!isfinite(u.x) || !isfinite(u.y) || !isfinite(u.z))) atomicExch(&a.counters[5], 1ull);
   if (blockIdx.x == 0 && threadIdx.x == 0) {
     *a.d_step = r.step0 + r.nsteps - 1;
-    if (ADR) *r.first = 0;  // every block read it before its first barrier
   }
 }
 
@@ -331,8 +287,7 @@ template <int DIM, int SPLIT, bool PAIR, int MAXT>
 cudaError_t launch(pd_ctx* c, StepArgs a, ResidentArgs r, unsigned grid, int block) {
   void* args[] = {&a, &r};
   const size_t sm = SPLIT > 1 ? (size_t)block * 3 * sizeof(double) : 0;
-  const void* k = a.adr ? (const void*)k_resident<DIM, SPLIT, PAIR, true, MAXT>
-                        : (const void*)k_resident<DIM, SPLIT, PAIR, false, MAXT>;
+  const void* k = (const void*)k_resident<DIM, SPLIT, PAIR, MAXT>;
   return cudaLaunchCooperativeKernel(k, dim3(grid), dim3((unsigned)block), args, sm, c->stream);
 }
 
@@ -356,7 +311,7 @@ cudaError_t launch_split(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, un
 ResidentPlan resident_plan(const pd_ctx* c) {
   ResidentPlan p;
   if (!c->auto_map || c->precision != PD_FP64 || c->kin != PD_LINEARIZED || !c->bond_cache || !c->pairs || !c->pairs_ok ||
-      c->profile || c->sms <= 0)
+      c->solver != PD_SOLVER_EXPLICIT || c->profile || c->sms <= 0)
     return p;
   // Warps per slice: four while that leaves an SM at most 16 warps (128 registers each), two up to 20, in 2D
   // one up to 24 (80 registers).  Beyond, the pass kernels are the faster ones (us per step, resident against
@@ -389,10 +344,6 @@ pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int6
   r.step0 = c->steps;
   r.grid = GridBar{c->bar, c->bar_base};
   r.uv = c->vol_uniform ? 1 : 0;
-  r.gold = c->gold;
-  r.lam = c->lam;
-  r.part = c->adr_part;
-  r.first = c->adr_first;
   const cudaError_t e = c->dim == 3 ? launch_split<3>(c, a, r, p.grid, p.block, p.split, p.pair)
                                     : launch_split<2>(c, a, r, p.grid, p.block, p.split, p.pair);
   if (e == cudaErrorCooperativeLaunchTooLarge || e == cudaErrorNotSupported) {
@@ -402,7 +353,7 @@ pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int6
   }
   if (e != cudaSuccess) return cuda_fail(e, "cudaLaunchCooperativeKernel");
   const bool pair = p.pair || p.block > 512;
-  const unsigned per_step = 2u + (pair ? 1u : 0u) + (a.adr ? 1u : 0u);
+  const unsigned per_step = pair ? 3u : 2u;
   c->bar_base += p.grid * (per_step * (unsigned)nsteps - 1u);
   if (nsteps & 1) c->cur ^= 1;
   *done = true;

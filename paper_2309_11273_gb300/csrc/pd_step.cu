@@ -681,13 +681,13 @@ __global__ void k_bond_sums(StepArgs a) {
 
 // THETA = false: the failure check alone (applied to the current state before it is read), with no
 // theta sum and no xi.du store: 6 FP64 instructions per bond.
-template <int DIM, int SPLIT, bool THETA>
+template <int DIM, int SPLIT, bool THETA, bool SERIAL>
 __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* __restrict__ disp,
                                                      int write_theta) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (write_theta && blockIdx.x == 0 && threadIdx.x == 0) *a.d_step += 1;
   double acc[2] = {0.0, 0.0};  // theta sum, and 1 if a bond of this warp's slots broke (warp-uniform)
-  constexpr int U = kU64, P = 4 / SPLIT, H = P > U ? P / U : 1;  // H half batches of U slots: the sum's parts
+  constexpr int U = kU64, P = SERIAL ? 1 : 4 / SPLIT, H = P > U ? P / U : 1;  // H half batches of U slots: the sum's parts
   double part[1][P] = {};
   int b = 0;
   if (t.active) {
@@ -738,7 +738,7 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
   }
   if (SPLIT == 1) __syncwarp();  // lane 0's status words, for the bS recomputation below
   double th1[1];
-  parts_sum<SPLIT, 1>(part, th1);
+  parts_sum<SPLIT, 1, P>(part, th1);
   acc[0] = th1[0];
   parts_across<SPLIT, 2>(acc);  // (SPLIT > 1: its block barrier orders the other warps' words)
   if (t.active && t.sub == 0) {
@@ -821,11 +821,12 @@ __global__ void __launch_bounds__(512) k_pass1a_f64p(StepArgs a, const double4* 
 // UV: every body has one particle volume, so V_j = V_i for every bond (same body) and the sum takes
 // the lane's own V_i: the same FMAs on the same values, without the neighbour index stream and the
 // gather of V_j.
-template <int DIM, int SPLIT, bool UV>
+template <int DIM, int SPLIT, bool UV, bool SERIAL>
 __global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* __restrict__ disp, int write_theta) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (write_theta && blockIdx.x == 0 && threadIdx.x == 0) *a.d_step += 1;
-  double acc[1], part[1][4 / SPLIT] = {};
+  constexpr int P = SERIAL ? 1 : 4 / SPLIT;
+  double acc[1], part[1][P] = {};
   int b = 0;
   if (t.active) {
     b = a.body ? a.body[t.i] : 0;
@@ -870,10 +871,10 @@ __global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* 
       for (int u = 0; u < U; ++u) dn[u] = td[(int64_t)min(k0 + (U + u) * SPLIT, t.W - 1) << 5];
 #pragma unroll
       for (int u = 0; u < U; ++u)
-        if ((wd[u] >> t.lane) & 1u) part[0][u % (4 / SPLIT)] = fma(v[u], d[u], part[0][u % (4 / SPLIT)]);
+        if ((wd[u] >> t.lane) & 1u) part[0][u % P] = fma(v[u], d[u], part[0][u % P]);
     }
   }
-  parts_sum<SPLIT, 1>(part, acc);
+  parts_sum<SPLIT, 1, P>(part, acc);
   parts_across<SPLIT, 1>(acc);
   if (t.active && t.sub == 0) {
     if (write_theta) {
@@ -1071,11 +1072,12 @@ __global__ void k_check_u32(int64_t n_pad, const double4* __restrict__ disp, flo
   cu[i] = make_float4(__double2float_rn(u.x), __double2float_rn(u.y), __double2float_rn(u.z), 0.0f);
 }
 
-template <int DIM, int SPLIT>
+template <int DIM, int SPLIT, bool SERIAL>
 __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* __restrict__ disp,
                                                      double4* __restrict__ disp_out) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
-  double f[3], part[3][4 / SPLIT] = {};
+  constexpr int P = SERIAL ? 1 : 4 / SPLIT;
+  double f[3], part[3][P] = {};
   int b = 0;
   if (t.active) {
     b = a.body ? a.body[t.i] : 0;
@@ -1083,7 +1085,7 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
     const int32_t* __restrict__ cl = a.col + t.base + t.lane;
     const double* __restrict__ td = a.bd + t.base + t.lane;
     // two slots in flight per warp and half batch: with four the parts of the sums need 77 registers
-    constexpr int U = 2, P = 4 / SPLIT, H = P > U ? P / U : 1;
+    constexpr int U = SERIAL ? 4 : 2, H = P > U ? P / U : 1;
     int32_t jn[U];
     uint32_t wn[U];
     load_slots<U, SPLIT>(t, cl, bw, t.sub, jn, wn);
@@ -1118,7 +1120,7 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
       }
     }
   }
-  parts_sum<SPLIT, 3>(part, f);
+  parts_sum<SPLIT, 3, P>(part, f);
   parts_across<SPLIT, 3>(f);
   if (t.active && t.sub == 0) {
     const double ti = a.thm[t.i].x;
@@ -2231,23 +2233,79 @@ __global__ void k_adr_lambda(StepArgs a, const double* __restrict__ alpha, doubl
 
 constexpr int kAdrBlock = 256;
 
-// Per slice: sum over its free particles' components of u (k u) and u u, k = -(g - g_prev) / (lambda v).
+// Sum of a 256-thread block's values in the order of a shared-memory tree (thread t adds t + 128, t + 64, ..., t +
+// 1), the last five levels by shuffles; the result in thread 0.  The order is part of the solver: where the
+// velocities change sign its damping amplifies a change of rounding by 1e8 within a hundred iterations.
+__device__ __forceinline__ double2 block_tree(double num, double den) {
+  __shared__ double sn[kAdrBlock], sd[kAdrBlock];
+  const int t = threadIdx.x;
+  sn[t] = num;
+  sd[t] = den;
+  __syncthreads();
+  for (int w = kAdrBlock / 2; w >= 32; w >>= 1) {
+    if (t < w) {
+      sn[t] += sn[t + w];
+      sd[t] += sd[t + w];
+    }
+    __syncthreads();
+  }
+  if (t >= 32) return make_double2(0.0, 0.0);
+  num = sn[t];
+  den = sd[t];
+#pragma unroll
+  for (int w = 16; w > 0; w >>= 1) {
+    num += __shfl_down_sync(kFull, num, w);
+    den += __shfl_down_sync(kFull, den, w);
+  }
+  return make_double2(num, den);
+}
+
+// Per block: sum over its free particles' components of u (k u) and u u, k = -(g - g_prev) / (lambda v).
 __global__ void __launch_bounds__(kAdrBlock) k_adr_sums(StepArgs a, const double4* __restrict__ disp,
                                                          const double4* __restrict__ gold,
                                                          const double2* __restrict__ lam,
                                                          double2* __restrict__ part) {
   const int64_t i = blockIdx.x * (int64_t)kAdrBlock + threadIdx.x;
-  if (i >= a.n_pad) return;  // whole warps: n_pad is a multiple of 32
-  const double2 s = adr_terms((!a.flag || a.flag[i] == 0) && lam[i].x > 0.0, disp[i], a.vel[i], a.gnew[i], gold[i], lam[i].x);
-  if ((threadIdx.x & 31) == 0) part[i >> 5] = s;
+  double num = 0.0, den = 0.0;
+  if (i < a.n_pad && (!a.flag || a.flag[i] == 0) && lam[i].x > 0.0) {
+    const double4 u = disp[i], v = a.vel[i], g = a.gnew[i], go = gold[i];
+    const double li = lam[i].x;
+    const double uu[3] = {u.x, u.y, u.z}, vv[3] = {v.x, v.y, v.z}, gg[3] = {g.x, g.y, g.z},
+                 gp[3] = {go.x, go.y, go.z};
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const double kk = vv[k] != 0.0 ? -(gg[k] - gp[k]) / (li * vv[k]) : 0.0;
+      num += uu[k] * kk * uu[k];
+      den += uu[k] * uu[k];
+    }
+  }
+  const double2 s = block_tree(num, den);
+  if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// One block: the damping and the start flag of this iteration.
-__global__ void __launch_bounds__(1024) k_adr_coef(const double2* __restrict__ part, int64_t nslices, int* first,
+// One block: c = 2 sqrt(num / den) (0 unless both are positive), the start flag of this iteration and
+// 1 / (2 + c).
+__global__ void __launch_bounds__(1024) k_adr_coef(const double2* __restrict__ part, int nblk, int* first,
                                                    double4* st) {
-  const double2 c = adr_damping(part, nslices);
+  __shared__ double sn[1024], sd[1024];
+  double num = 0.0, den = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += 1024) {
+    num += part[b].x;
+    den += part[b].y;
+  }
+  sn[threadIdx.x] = num;
+  sd[threadIdx.x] = den;
+  __syncthreads();
+  for (int w = 512; w > 0; w >>= 1) {
+    if (threadIdx.x < w) {
+      sn[threadIdx.x] += sn[threadIdx.x + w];
+      sd[threadIdx.x] += sd[threadIdx.x + w];
+    }
+    __syncthreads();
+  }
   if (threadIdx.x == 0) {
-    *st = make_double4(c.x, (double)*first, c.y, 0.0);
+    const double c = (sd[0] > 0.0 && sn[0] > 0.0) ? 2.0 * sqrt(sn[0] / sd[0]) : 0.0;
+    *st = make_double4(c, (double)*first, 1.0 / (2.0 + c), 0.0);
     *first = 0;
   }
 }
@@ -2272,10 +2330,15 @@ __global__ void __launch_bounds__(kAdrBlock) k_adr_update(StepArgs a, const doub
     const double2 li = lam[i];  // (lambda, 1 / lambda)
     if (li.x > 0.0) {
       const double4 s = *st;
-      const bool start = s.y != 0.0;
-      v.x = adr_velocity(v.x, g.x, li.y, s.x, s.z, start);
-      v.y = adr_velocity(v.y, g.y, li.y, s.x, s.z, start);
-      v.z = adr_velocity(v.z, g.z, li.y, s.x, s.z, start);
+      if (s.y != 0.0) {
+        const double h = 0.5 * li.y;
+        v = make_double4(g.x * h, g.y * h, g.z * h, 0.0);
+      } else {
+        const double cm = 2.0 - s.x, r2 = 2.0 * li.y;
+        v.x = (cm * v.x + g.x * r2) * s.z;
+        v.y = (cm * v.y + g.y * r2) * s.z;
+        v.z = (cm * v.z + g.z * r2) * s.z;
+      }
       u.x = u.x + v.x;
       u.y = u.y + v.y;
       u.z = u.z + v.z;
@@ -2659,6 +2722,7 @@ void launch_pass1a_nlp(pd_ctx* c, const StepArgs& a, unsigned grid, int block) {
 
 template <int DIM, int SPLIT>
 void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, int block, size_t sm) {
+  const bool serial = SPLIT == 1 && a.adr;  // the relaxation solver's sums: parts_sum
   if (c->kin == PD_NONLINEAR && a.bA && a.own0 && !write_theta) {
     if (a.check) k_check_nlp<DIM, SPLIT><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
   } else if (c->kin == PD_NONLINEAR && a.bA && a.own0) {
@@ -2695,15 +2759,21 @@ void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, 
       c->times.mid = take_event(c);
       cudaEventRecord(c->times.mid, c->stream);
     }
-    if (c->vol_uniform)
-      k_pass1b_f64p<DIM, SPLIT, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    if (serial && c->vol_uniform)
+      k_pass1b_f64p<DIM, 1, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    else if (serial)
+      k_pass1b_f64p<DIM, 1, false, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    else if (c->vol_uniform)
+      k_pass1b_f64p<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else
-      k_pass1b_f64p<DIM, SPLIT, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1b_f64p<DIM, SPLIT, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
   } else if (c->precision == PD_FP64 && a.bA) {
-    if (write_theta)
-      k_pass1_f64t<DIM, SPLIT, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    if (write_theta && serial)
+      k_pass1_f64t<DIM, 1, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    else if (write_theta)
+      k_pass1_f64t<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else
-      k_pass1_f64t<DIM, SPLIT, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1_f64t<DIM, SPLIT, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
   }
   else if (c->precision == PD_FP64)
     k_pass1_f64<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
@@ -2719,8 +2789,10 @@ void launch_pass2(pd_ctx* c, const StepArgs& a, unsigned grid, int block, size_t
     k_pass2_nlt<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->kin == PD_NONLINEAR)
     k_pass2_nl<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
+  else if (c->precision == PD_FP64 && a.bA && SPLIT == 1 && a.adr)
+    k_pass2_f64t<DIM, 1, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64 && a.bA)
-    k_pass2_f64t<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
+    k_pass2_f64t<DIM, SPLIT, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64)
     k_pass2_f64<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else
@@ -2847,7 +2919,7 @@ namespace {
 
 template <int DIM>
 void dispatch_pass(pd_ctx* c, const StepArgs& a, int pass, int write_theta) {
-  const int split = c->auto_map && c->precision == PD_FP64 && c->kin == PD_LINEARIZED && a.bA ? auto_split64(c) : c->split;
+  const int split = c->auto_map && c->precision == PD_FP64 && c->kin == PD_LINEARIZED && a.bA && !a.adr ? auto_split64(c) : c->split;
   int block = c->block;
   if (c->auto_map && c->precision == PD_FP64) block = split == 4 ? 2 * kAutoBlock64 : kAutoBlock64;
   else if (c->auto_map && c->lattice) block = kAutoBlockLat;
@@ -2977,10 +3049,11 @@ pd_status ensure_adr(pd_ctx* c) {
   pd_status st;
   if (!c->lam) {
     const int64_t np = c->n_pad;
+    const size_t nblk = (size_t)((np + kAdrBlock - 1) / kAdrBlock);
     if ((st = alloc(c, &c->lam, np)) != PD_OK) return st;
     if ((st = alloc(c, &c->gnew, np)) != PD_OK) return st;
     if ((st = alloc(c, &c->gold, np)) != PD_OK) return st;
-    if ((st = alloc(c, &c->adr_part, (size_t)c->nslices)) != PD_OK) return st;
+    if ((st = alloc(c, &c->adr_part, nblk)) != PD_OK) return st;
     if ((st = alloc(c, &c->adr_st, 1)) != PD_OK) return st;
     if ((st = alloc(c, &c->adr_first, 1)) != PD_OK) return st;
     PD_CUDA(cudaMemsetAsync(c->gnew, 0, sizeof(double4) * np, c->stream));
@@ -3074,7 +3147,7 @@ pd_status launch_step(pd_ctx* c, bool check) {
   if (a.adr) {
     const unsigned nblk = (unsigned)((c->n_pad + kAdrBlock - 1) / kAdrBlock);
     k_adr_sums<<<nblk, kAdrBlock, 0, c->stream>>>(a, c->disp[c->cur], c->gold, c->lam, c->adr_part);
-    k_adr_coef<<<1, 1024, 0, c->stream>>>(c->adr_part, c->nslices, c->adr_first, c->adr_st);
+    k_adr_coef<<<1, 1024, 0, c->stream>>>(c->adr_part, (int)nblk, c->adr_first, c->adr_st);
     k_adr_update<<<nblk, kAdrBlock, 0, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1], c->gold, c->lam,
                                                     c->adr_st,
                                                     c->precision == PD_MIXED ? c->u32[c->cur ^ 1] : nullptr,
@@ -3260,7 +3333,7 @@ pd_status check_device_error(pd_ctx* c) {
       c->bar_base = 0;
     }
     return fail(PD_ERR_TIMEOUT, "a staged neighbour-index copy or a grid barrier did not complete within the wait "
-                                "limit; the step's results were not written");
+                                "limit; the steps' results were not written");
   }
   if (nonfinite) {
     PD_CUDA(cudaMemsetAsync(c->counters + 5, 0, sizeof(nonfinite), c->stream));

@@ -110,6 +110,33 @@ def test_mixed_impact_and_batch():
     _same(lambda: BatchSimulation(W.plate_batch(nplates=9, side_hi=90), precision=PD_MIXED), [60, 40])
 
 
+def test_contexts_on_their_own_streams_and_threads():
+    """Two FP64 and one mixed context, each with its own stream, step from three threads at once (every grid
+    wants the whole chip): all end with the state of a run alone."""
+    import threading
+    makes = [lambda: Simulation(_plate(200, 120)), lambda: Simulation(_plate(90, 60)),
+             lambda: Simulation(_plate(230, 160), precision=PD_MIXED)]
+    alone = []
+    for mk in makes:
+        sim = mk()
+        sim.step(400)
+        alone.append(sim.state()[0])
+        sim.close()
+    sims, got = [mk() for mk in makes], [None] * 3
+
+    def work(k):
+        for _ in range(8):
+            sims[k].step(50)
+        got[k] = sims[k].state()[0]
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(3)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    for a, g in zip(alone, got):
+        assert g is not None and np.array_equal(a, g)
+
+
 def test_switching_between_the_kernels_keeps_the_run():
     ref = Simulation(_plate(90, 60))
     ref.step(120)
