@@ -57,7 +57,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   // batch waited for its indices and then its rows from memory (a 45,000-particle block 134.8 -> 124.4 us per
   // iteration with 2, 129.9 with 4, 139.4 with 8, which push each other out).
   constexpr int kAhead = PAIR && DIM == 3 ? 2 : 0;
-  if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
+  // an earlier launch gave up and its error is not yet reported (one answer for the whole block)
+  if (__syncthreads_or(ld_relaxed(r.grid.bar + 1) != 0u)) return;
   unsigned target = r.grid.base;
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   const bool lead = t.active && t.sub == 0;

@@ -40,7 +40,8 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident_lat(StepArgs a, LatRun r) 
   constexpr bool kKeep = MAXT <= 512;  // the FP64 state in registers
   constexpr int NB = MAXT <= 256 ? 4 : (LO ? 1 : 2);
   constexpr int U = 4;
-  if (ld_relaxed(r.grid.bar + 1) != 0u) return;  // an earlier launch gave up: its error is not yet reported
+  // an earlier launch gave up and its error is not yet reported (one answer for the whole block)
+  if (__syncthreads_or(ld_relaxed(r.grid.bar + 1) != 0u)) return;
   unsigned target = r.grid.base;
   const SliceIdx t = slice_index<1>(a.n_pad, a.slice_ptr);
   const int lane = t.lane;
