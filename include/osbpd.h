@@ -137,9 +137,9 @@ typedef struct {
 /* Options for pd_set_option / pd_get_option. */
 typedef enum {
   PD_OPT_GRAPH_CHUNK = 1,  /* steps captured per CUDA graph launch (0: no graphs). Default 100.  Bodies
-                              with linearized bonds that fit the GPU in one wave (explicit solver; PD_FP64
-                              up to about 115,000 particles in 2D and 48,000 in 3D, PD_MIXED on the
-                              lattice layout up to 117,000) take all steps of a call in one cooperative
+                              that fit the GPU in one wave (explicit solver; PD_FP64 with linearized
+                              bonds up to about 115,000 particles in 2D and 48,000 in 3D, PD_MIXED on
+                              the lattice layout up to 117,000) take all steps of a call in one cooperative
                               launch instead, while no launch mapping was chosen (PD_OPT_BLOCK,
                               PD_OPT_SPLIT, PD_OPT_LAT_STAGE); results are bitwise the same */
   PD_OPT_PROFILE = 2,      /* 1: time every kernel launch with CUDA events (forces eager launches) */

@@ -209,5 +209,58 @@ __device__ __forceinline__ void update(const StepArgs& a, int64_t i, int b, cons
   a.vel[i] = v;
 }
 
+// A bond of the geometrically nonlinear model in FP64 (the comment above k_pass1_nl), and the FP64
+// re-decision of the mixed kernels with the same arithmetic.
+template <int DIM>
+struct BondNL {
+  double yx, yy, yz;  // Y
+  double p;           // |Y|^2 - |xi|^2
+  double q;           // |xi|^2
+};
+
+template <int DIM>
+__device__ __forceinline__ BondNL<DIM> bond_nl(const double4& pi, const double4& pj, const double4& ui,
+                                              const double4& uj) {
+  BondNL<DIM> r;
+  const double ex = pj.x - pi.x, ey = pj.y - pi.y, ez = DIM == 3 ? pj.z - pi.z : 0.0;
+  const double hx = uj.x - ui.x, hy = uj.y - ui.y, hz = DIM == 3 ? uj.z - ui.z : 0.0;
+  r.yx = ex + hx;
+  r.yy = ey + hy;
+  r.yz = ez + hz;
+  r.p = hx * (ex + r.yx) + hy * (ey + r.yy);
+  r.q = ex * ex + ey * ey;
+  if (DIM == 3) {
+    r.p = fma(hz, ez + r.yz, r.p);
+    r.q = fma(ez, ez, r.q);
+  }
+  return r;
+}
+
+template <int DIM>
+__device__ __noinline__ bool fp64_breaks_nl(const StepArgs& a, int64_t i, int32_t j,
+                                            const double4* __restrict__ disp) {
+  const int b = a.body ? a.body[i] : 0;
+  const BondNL<DIM> r = bond_nl<DIM>(a.pos[i], a.pos[j], disp[i], disp[j]);
+  return r.p >= a.bp[b].s0nl * r.q;
+}
+
+// The hardware approximations of 1 / sqrt(x) and 1 / x with a subnormal x read as zero (PTX
+// rsqrt.approx.ftz.f32, rcp.approx.ftz.f32), for the FP32 nonlinear kernels: without .ftz each call
+// carries a test and rescaling for subnormal inputs.  Their arguments are squared bond lengths and
+// sums of bond lengths: |Y|^2 and |Y| + |xi| in units of the coordinate quantum (|xi| >= 1), and
+// |Y'|^2 = |n|^2 + p and |Y'| + |n| >= 1 in lattice units, normal numbers for every bond not
+// compressed to within 2^-63 of its length, where the results equal those of rsqrtf and __fdividef
+// bit for bit.
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 }  // namespace
 }  // namespace pd

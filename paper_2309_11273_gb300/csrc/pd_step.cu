@@ -36,12 +36,6 @@ __device__ __noinline__ bool fp64_breaks(const StepArgs& a, int64_t i, int32_t j
   return fp64_breaks_inl<DIM>(a, i, j, disp, s0);
 }
 
-// Nonlinear FP64 re-decision for the mixed path: |Y|^2 - |xi|^2 >= s0 (2 + s0) |xi|^2 with the
-// arithmetic of the FP64 nonlinear kernels (defined with them below).
-template <int DIM>
-__device__ __noinline__ bool fp64_breaks_nl(const StepArgs& a, int64_t i, int32_t j,
-                                            const double4* __restrict__ disp);
-
 // Slot batches: each thread handles U slots per iteration; the neighbour indices and status words
 // of the next batch are loaded while the current batch's gathers are in flight, so that several
 // dependent index -> gather chains overlap.
@@ -171,39 +165,6 @@ __global__ void __launch_bounds__(512) k_pass2_f64(StepArgs a, const double4* __
 // as eta . (xi + Y) = 2 xi.eta + eta.eta, so e = (|Y|^2 - |xi|^2) / (|Y| + |xi|) carries no
 // cancellation, and the break test e / |xi| >= s0 (Eq 1.30) is taken without square roots as
 // |Y|^2 - |xi|^2 >= s0 (2 + s0) |xi|^2.
-template <int DIM>
-struct BondNL {
-  double yx, yy, yz;  // Y
-  double p;           // |Y|^2 - |xi|^2
-  double q;           // |xi|^2
-};
-
-template <int DIM>
-__device__ __forceinline__ BondNL<DIM> bond_nl(const double4& pi, const double4& pj, const double4& ui,
-                                              const double4& uj) {
-  BondNL<DIM> r;
-  const double ex = pj.x - pi.x, ey = pj.y - pi.y, ez = DIM == 3 ? pj.z - pi.z : 0.0;
-  const double hx = uj.x - ui.x, hy = uj.y - ui.y, hz = DIM == 3 ? uj.z - ui.z : 0.0;
-  r.yx = ex + hx;
-  r.yy = ey + hy;
-  r.yz = ez + hz;
-  r.p = hx * (ex + r.yx) + hy * (ey + r.yy);
-  r.q = ex * ex + ey * ey;
-  if (DIM == 3) {
-    r.p = fma(hz, ez + r.yz, r.p);
-    r.q = fma(ez, ez, r.q);
-  }
-  return r;
-}
-
-template <int DIM>
-__device__ __noinline__ bool fp64_breaks_nl(const StepArgs& a, int64_t i, int32_t j,
-                                            const double4* __restrict__ disp) {
-  const int b = a.body ? a.body[i] : 0;
-  const BondNL<DIM> r = bond_nl<DIM>(a.pos[i], a.pos[j], disp[i], disp[j]);
-  return r.p >= a.bp[b].s0nl * r.q;
-}
-
 template <int DIM, int SPLIT>
 __global__ void __launch_bounds__(512) k_pass1_nl(StepArgs a, const double4* __restrict__ disp,
                                                    int write_theta) {
@@ -1161,24 +1122,6 @@ __global__ void k_bond_tables(StepArgs a, double4* __restrict__ bA, double4* __r
 }
 
 // ----------------------------------------------------------------------------------- mixed path
-// The hardware approximations of 1 / sqrt(x) and 1 / x with a subnormal x read as zero (PTX
-// rsqrt.approx.ftz.f32, rcp.approx.ftz.f32), for the FP32 nonlinear kernels: without .ftz each call
-// carries a test and rescaling for subnormal inputs.  Their arguments are squared bond lengths and
-// sums of bond lengths: |Y|^2 and |Y| + |xi| in units of the coordinate quantum (|xi| >= 1), and
-// |Y'|^2 = |n|^2 + p and |Y'| + |n| >= 1 in lattice units, normal numbers for every bond not
-// compressed to within 2^-63 of its length, where the results equal those of rsqrtf and __fdividef
-// bit for bit.
-__device__ __forceinline__ float rsqrt_ftz(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float rcp_ftz(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
 // FP32 bond arithmetic on fixed-point coordinates (xi exact as an integer multiple of the quantum Q,
 // then rounded once to FP32) and an FP32 shadow copy of u.  The band half-width B bounds
 // |g32 - g| for g = xi.du - s0 |xi|^2 (in Q units) from the FP32 representation of u, the rounding

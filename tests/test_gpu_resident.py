@@ -5,7 +5,7 @@ barrier wait (GPU only)."""
 import numpy as np
 import pytest
 
-from paper_2309_11273_gb300 import PD_MIXED, PD_W_INV, BatchSimulation, PDError, Simulation
+from paper_2309_11273_gb300 import PD_MIXED, PD_NONLINEAR, PD_W_INV, BatchSimulation, PDError, Simulation
 from paper_2309_11273_gb300 import _binding as B
 from paper_2309_11273_gb300 import workloads as W
 
@@ -102,6 +102,16 @@ def test_mixed_blocks_are_bitwise_the_pass_kernels(shape, influence):
     def make():
         w = W.notched_block(*shape, nsteps=300, seed=5, amp=2e-8, dt=2.5e-7)
         return Simulation(w, precision=PD_MIXED, influence=influence)
+    _same(make, [1, 25, 24])
+
+
+@pytest.mark.parametrize("lo", [0, 1])
+@pytest.mark.parametrize("shape", [(7, 5), (40, 40), (279, 278), (341, 340), (350, 340), (9, 7, 5), (33, 12, 10), (61, 30, 35),
+                                   (64, 45, 40)])
+def test_mixed_nonlinear_bodies_are_bitwise_the_pass_kernels(shape, lo):
+    def make():
+        w = _plate(*shape) if len(shape) == 2 else W.notched_block(*shape, nsteps=300, seed=5, amp=2e-8)
+        return Simulation(w, precision=PD_MIXED, kinematics=PD_NONLINEAR, shadow_lo=lo)
     _same(make, [1, 25, 24])
 
 
