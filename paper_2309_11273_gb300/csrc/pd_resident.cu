@@ -82,11 +82,6 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
     if (a.bacc) bb = a.bacc[i];
   };
   if (kKeep) load_state(r.disp);
-  if (lead && a.dirty[s]) {  // bonds broken by a check between calls
-    bond_sum_row<DIM>(a, t);
-    __syncwarp();
-    if (t.lane == 0) a.dirty[s] = 0;
-  }
   const double vi = t.active ? a.pos[i].w : 0.0;
   // the neighbours of a batch of slots (past the row: its last one), loaded in place or ahead
   int32_t jn[U];
@@ -200,10 +195,13 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
       ti = bp.Kp * (th * mu);
       a.thm[i].x = ti;
       if (step + 1 == r.nsteps) a.theta[i] = th;
-      if (PAIR ? a.dirty[s] != 0 : sum[1] != 0.0) {  // uniform over the warp
+      // The marks are consumed here alone: in the pair form every store to them and to the bits they stand for
+      // lies before the barrier above, and without it only a check between calls sets them, before the launch.
+      const bool marked = (PAIR || step == 0) && a.dirty[s] != 0;  // uniform over the warp
+      if (marked || sum[1] != 0.0) {
         bond_sum_row<DIM>(a, t);
         __syncwarp();
-        if (PAIR && t.lane == 0) a.dirty[s] = 0;
+        if (marked && t.lane == 0) a.dirty[s] = 0;
       }
     }
     if (!grid_barrier(a, r.grid, target)) return;

@@ -175,3 +175,38 @@ def test_expired_barrier_reports_timeout_and_the_context_recovers():
     ref = Simulation(w)
     ref.step(50)
     assert np.array_equal(sim.state()[0], ref.state()[0])
+
+
+def _run_unread(sim, calls):
+    for k in calls:
+        sim.step(k)
+    out = list(sim.state()) + [sim.damage(), sim.neighbors()[2]]
+    sim.close()
+    return out
+
+
+def _same_unread(make, calls):
+    res, ref = _run_unread(make(), calls), _run_unread(_pass_kernels(make()), calls)
+    assert (ref[-1] == 0).any()  # bonds broke
+    for x, y in zip(res, ref):
+        assert np.array_equal(x, y)
+
+
+# The first step of a call that follows an unread one checks its bonds, and so does each launch of a call longer
+# than one launch (1000 steps): the intact sums a call starts from and the marks of its first check must not mix.
+# (40, 40): without the pair form; the others with it, at four, two and one warps per slice
+@pytest.mark.parametrize("nx,ny,ratio", [(40, 40, 3.015), (138, 140, 4.015), (200, 200, 3.015), (341, 340, 3.015)])
+@pytest.mark.parametrize("calls", [[1, 1, 1, 2, 3, 12], [1, 1100]])
+def test_unread_calls_on_breaking_plates(nx, ny, ratio, calls):
+    _same_unread(lambda: Simulation(_plate(nx, ny, ratio)), calls)
+
+
+@pytest.mark.parametrize("shape", [(9, 7, 5), (30, 25, 24), (40, 38, 32)])
+def test_unread_calls_on_breaking_blocks(shape):
+    _same_unread(lambda: Simulation(W.notched_block(*shape, nsteps=100, seed=5, amp=2e-8)), [1, 1, 2, 1, 40, 55])
+
+
+@pytest.mark.parametrize("kinematics", [0, PD_NONLINEAR])
+@pytest.mark.parametrize("nx,ny", [(40, 40), (341, 340)])
+def test_unread_calls_on_breaking_mixed_plates(nx, ny, kinematics):
+    _same_unread(lambda: Simulation(_plate(nx, ny), precision=PD_MIXED, kinematics=kinematics), [1, 1, 1, 2, 3, 12, 30])
