@@ -62,20 +62,25 @@ __device__ __forceinline__ void split_reduce(T (&v)[NC]) {
 // The sums of the tabled FP64 kernels run in four parts, slot k in part k mod 4, combined as (0 + 2) +
 // (1 + 3) whatever the number of warps that share a slice: a warp holds 4 / SPLIT of them, so the result
 // is bitwise the same for every split (and four independent chains of FP64 additions are shorter).
-// P = 1 with one warp per slice: the plain sum in slot order, which the relaxation solver keeps (block_tree).
+// P = 1: each warp's plain sum in slot order, which the relaxation solver keeps (block_tree).
 template <int SPLIT, int NC, int P = 4 / SPLIT>
 __device__ __forceinline__ void parts_sum(const double (&p)[NC][P], double (&v)[NC]) {
 #pragma unroll
   for (int c = 0; c < NC; ++c) {
-    if constexpr (P == 1) v[c] = p[c][0];
+    if constexpr (P == 1) v[c] = p[c][0];  // (split 4: one part per warp)
     else if constexpr (SPLIT == 1) v[c] = (p[c][0] + p[c][2]) + (p[c][1] + p[c][3]);
     else v[c] = p[c][0] + p[c][1];
   }
 }
-// ... and across the warps of the slice (their parts combined by the first warp).
-template <int SPLIT, int NC>
+// ... and across the warps of the slice (their parts combined by the first warp; SERIAL, the relaxation solver:
+// the warps' sums added one after the other).
+template <int SPLIT, int NC, bool SERIAL = false>
 __device__ __forceinline__ void parts_across(double (&v)[NC]) {
   if (SPLIT == 1) return;
+  if constexpr (SERIAL) {
+    split_reduce<SPLIT, NC>(v);
+    return;
+  }
   extern __shared__ unsigned char smem_raw[];
   double* red = reinterpret_cast<double*>(smem_raw);
 #pragma unroll

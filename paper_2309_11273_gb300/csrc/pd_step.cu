@@ -701,7 +701,7 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
   double th1[1];
   parts_sum<SPLIT, 1, P>(part, th1);
   acc[0] = th1[0];
-  parts_across<SPLIT, 2>(acc);  // (SPLIT > 1: its block barrier orders the other warps' words)
+  parts_across<SPLIT, 2, SERIAL>(acc);  // (SPLIT > 1: its block barrier orders the other warps' words)
   if (t.active && t.sub == 0) {
     if (THETA && write_theta) {
       const double th = a.aA[t.i] * acc[0];
@@ -836,7 +836,7 @@ __global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* 
     }
   }
   parts_sum<SPLIT, 1, P>(part, acc);
-  parts_across<SPLIT, 1>(acc);
+  parts_across<SPLIT, 1, SERIAL>(acc);
   if (t.active && t.sub == 0) {
     if (write_theta) {
       const double th = a.aA[t.i] * acc[0];
@@ -1082,7 +1082,7 @@ __global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* _
     }
   }
   parts_sum<SPLIT, 3, P>(part, f);
-  parts_across<SPLIT, 3>(f);
+  parts_across<SPLIT, 3, SERIAL>(f);
   if (t.active && t.sub == 0) {
     const double ti = a.thm[t.i].x;
     const double4 S = a.bS[t.i];
@@ -2665,7 +2665,7 @@ void launch_pass1a_nlp(pd_ctx* c, const StepArgs& a, unsigned grid, int block) {
 
 template <int DIM, int SPLIT>
 void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, int block, size_t sm) {
-  const bool serial = SPLIT == 1 && a.adr;  // the relaxation solver's sums: parts_sum
+  const bool serial = a.adr != 0;  // the relaxation solver's sums: parts_sum
   if (c->kin == PD_NONLINEAR && a.bA && a.own0 && !write_theta) {
     if (a.check) k_check_nlp<DIM, SPLIT><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
   } else if (c->kin == PD_NONLINEAR && a.bA && a.own0) {
@@ -2703,16 +2703,16 @@ void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, 
       cudaEventRecord(c->times.mid, c->stream);
     }
     if (serial && c->vol_uniform)
-      k_pass1b_f64p<DIM, 1, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1b_f64p<DIM, SPLIT, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else if (serial)
-      k_pass1b_f64p<DIM, 1, false, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1b_f64p<DIM, SPLIT, false, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else if (c->vol_uniform)
       k_pass1b_f64p<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else
       k_pass1b_f64p<DIM, SPLIT, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
   } else if (c->precision == PD_FP64 && a.bA) {
     if (write_theta && serial)
-      k_pass1_f64t<DIM, 1, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1_f64t<DIM, SPLIT, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else if (write_theta)
       k_pass1_f64t<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else
@@ -2732,8 +2732,8 @@ void launch_pass2(pd_ctx* c, const StepArgs& a, unsigned grid, int block, size_t
     k_pass2_nlt<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->kin == PD_NONLINEAR)
     k_pass2_nl<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
-  else if (c->precision == PD_FP64 && a.bA && SPLIT == 1 && a.adr)
-    k_pass2_f64t<DIM, 1, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
+  else if (c->precision == PD_FP64 && a.bA && a.adr)
+    k_pass2_f64t<DIM, SPLIT, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64 && a.bA)
     k_pass2_f64t<DIM, SPLIT, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64)
