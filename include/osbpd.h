@@ -190,7 +190,7 @@ typedef enum {
                               stream, 0 (default) = 3 chunks of 16 slots, 1 = 2 x 16, 2 = 3 x 8,
                               3 = 2 x 8 (smaller rings leave more of the SM's combined L1 / shared
                               memory to the displacement gathers); pd_autotune chooses it */
-  PD_OPT_SHADOW_LO = 13    /* lattice kernels: 1 = carry each particle's FP32 displacement copy
+  PD_OPT_SHADOW_LO = 13,   /* lattice kernels: 1 = carry each particle's FP32 displacement copy
                               (u / h) as two FP32 words hi + lo (lo the rounding remainder of hi,
                               16 more bytes per particle and per step gathered per bond in both
                               passes; linearized and nonlinear bonds), so that a bond's
@@ -200,6 +200,9 @@ typedef enum {
                               0 (default) = one word.  Decisions stay exact either way (the same
                               rounding band covers both).  May be set at any time; pd_get_option
                               reports 1 only while the built layout is the lattice one. */
+  PD_OPT_DEVICE_LIMIT = 14 /* testing the failure path: device bytes (pd_get_info) above which the
+                              context's allocations fail as if the device had no memory left.
+                              Default 0: no limit of its own. */
 } pd_option;
 
 /* Solvers (PD_OPT_SOLVER).

@@ -628,6 +628,10 @@ pd_status pd_set_option(pd_ctx* c, int32_t option, int64_t value) {
         if (st != PD_OK) return st;
       }
       break;
+    case PD_OPT_DEVICE_LIMIT:
+      if (value < 0) return fail(PD_ERR_ARG, "PD_OPT_DEVICE_LIMIT must be >= 0");
+      c->device_limit = value;
+      break;
     case PD_OPT_PAIRS:
       // A failure check of the pair form marks slices whose bS its next pass 1b recomputes; the
       // other form never reads those marks, so a switch recomputes every bS before the next step.
@@ -666,6 +670,7 @@ pd_status pd_get_option(pd_ctx* c, int32_t option, int64_t* value) {
     case PD_OPT_LATTICE: *value = c->built ? (c->lattice ? 1 : 0) : c->lattice_opt; break;
     case PD_OPT_LAT_STAGE: *value = c->lat_stage; break;
     case PD_OPT_SHADOW_LO: *value = c->built ? (c->shadow_lo ? 1 : 0) : c->shadow_lo_opt; break;
+    case PD_OPT_DEVICE_LIMIT: *value = c->device_limit; break;
     default: return fail(PD_ERR_ARG, "unknown option");
   }
   return PD_OK;

@@ -272,6 +272,7 @@ struct pd_ctx {
   cudaGraphExec_t graph[2] = {nullptr, nullptr};
   pd::KernelTimes times;
   int64_t device_bytes = 0;
+  int64_t device_limit = 0;    // testing (PD_OPT_DEVICE_LIMIT): alloc fails beyond it; 0: no limit
   std::vector<void*> allocs;
   std::vector<size_t> alloc_bytes;
   size_t n_create_allocs = 0;  // allocations made at creation; later ones belong to the build
@@ -287,6 +288,11 @@ template <class T>
 pd_status alloc(pd_ctx* c, T** p, size_t count);
 void free_all(pd_ctx* c);
 void release(pd_ctx* c, void* p);  // frees one allocation of the context (nullptr: nothing)
+template <class T>
+void drop(pd_ctx* c, T** p) {  // ... and forgets it
+  release(c, *p);
+  *p = nullptr;
+}
 void free_build(pd_ctx* c);
 void material_constants(int model, double E, double nu, double* A, double* K, double* G);
 pd_status upload_body_params(pd_ctx* c);
@@ -344,7 +350,8 @@ pd_status pd::alloc(pd_ctx* c, T** p, size_t count) {
   *p = nullptr;
   if (count == 0) count = 1;
   void* q = nullptr;
-  cudaError_t e = cudaMalloc(&q, count * sizeof(T));
+  const bool over = c->device_limit > 0 && c->device_bytes + (int64_t)(count * sizeof(T)) > c->device_limit;
+  cudaError_t e = over ? cudaErrorMemoryAllocation : cudaMalloc(&q, count * sizeof(T));
   if (e != cudaSuccess) {
     cudaGetLastError();
     return pd::fail(PD_ERR_OOM, "cudaMalloc of " + std::to_string(count * sizeof(T)) + " bytes failed");

@@ -2921,27 +2921,63 @@ pd_status init_disp_w(pd_ctx* c) {
   return PD_OK;
 }
 
+// The per-slot tables of the tabled FP64 path, all of them or none: a step after a failed allocation must
+// not find some of them.
+static pd_status alloc_bond_tables(pd_ctx* c, size_t ne) {
+  pd_status st;
+  if (c->kin == PD_NONLINEAR) {
+    if ((st = alloc(c, &c->bA, ne)) != PD_OK) return st;
+    if ((st = alloc(c, &c->bE, ne)) != PD_OK) return st;
+    if (!c->pairs_ok) return PD_OK;
+    if ((st = alloc(c, &c->bt, ne)) != PD_OK) return st;
+    if ((st = alloc(c, &c->bY, ne)) != PD_OK) return st;
+    if ((st = alloc(c, &c->bC, ne)) != PD_OK) return st;
+    if ((st = alloc(c, &c->bX2, ne)) != PD_OK) return st;
+    return alloc(c, &c->bX, ne);
+  }
+  const size_t nt = c->dim == 3 ? ne : (3 * ne + 3) / 4;  // 2D rows: 24 bytes (slot_row)
+  if ((st = alloc(c, &c->bA, nt)) != PD_OK) return st;
+  if ((st = alloc(c, &c->bB, nt)) != PD_OK) return st;
+  if ((st = alloc(c, &c->bd, ne)) != PD_OK) return st;
+  if ((st = alloc(c, &c->bS, (size_t)c->n_pad)) != PD_OK) return st;
+  return c->pairs_ok ? alloc(c, &c->dirty, (size_t)c->nslices) : PD_OK;
+}
+
+static void drop_bond_tables(pd_ctx* c) {
+  drop(c, &c->bA);
+  drop(c, &c->bE);
+  drop(c, &c->bt);
+  drop(c, &c->bY);
+  drop(c, &c->bC);
+  drop(c, &c->bX2);
+  drop(c, &c->bX);
+  drop(c, &c->bB);
+  drop(c, &c->bd);
+  drop(c, &c->bS);
+  drop(c, &c->dirty);
+}
+
 // Allocates and fills the per-slot tables of the tabled FP64 path (once per build), and brings the
 // per-particle intact sums up to date with the status bits.
 pd_status ensure_bond_cache(pd_ctx* c) {
   if (!c->bond_cache || c->precision != PD_FP64) return PD_OK;
-  pd_status st;
   const size_t ne = (size_t)std::max<int64_t>(c->nentries, 32);
   const int tb = 256;
   const unsigned grid = (unsigned)((c->n_pad + tb - 1) / tb);
+  const bool fresh = !c->bA;
+  if (fresh) {
+    const pd_status st = alloc_bond_tables(c, ne);
+    if (st != PD_OK) {
+      drop_bond_tables(c);
+      return st;
+    }
+  }
   if (c->kin == PD_NONLINEAR) {
-    if (c->bA) return PD_OK;
-    if ((st = alloc(c, &c->bA, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bE, ne)) != PD_OK) return st;
+    if (!fresh) return PD_OK;
     PD_CUDA(cudaMemsetAsync(c->bE, 0, sizeof(double2) * ne, c->stream));
     if (c->pairs_ok) {
-      if ((st = alloc(c, &c->bt, ne)) != PD_OK) return st;
       PD_CUDA(cudaMemsetAsync(c->bt, 0, sizeof(double) * ne, c->stream));
-      if ((st = alloc(c, &c->bY, ne)) != PD_OK) return st;
       PD_CUDA(cudaMemsetAsync(c->bY, 0, sizeof(double4) * ne, c->stream));
-      if ((st = alloc(c, &c->bC, ne)) != PD_OK) return st;
-      if ((st = alloc(c, &c->bX2, ne)) != PD_OK) return st;
-      if ((st = alloc(c, &c->bX, ne)) != PD_OK) return st;
       StepArgs ax = make_args(c);
       if (c->dim == 3)
         k_bond_tables_nlp<3><<<grid, tb, 0, c->stream>>>(ax, c->bC, c->bX, c->bX2);
@@ -2957,17 +2993,9 @@ pd_status ensure_bond_cache(pd_ctx* c) {
     PD_CUDA(cudaGetLastError());
     return PD_OK;
   }
-  if (!c->bA) {
-    const size_t nt = c->dim == 3 ? ne : (3 * ne + 3) / 4;  // 2D rows: 24 bytes (slot_row)
-    if ((st = alloc(c, &c->bA, nt)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bB, nt)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bd, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bS, (size_t)c->n_pad)) != PD_OK) return st;
+  if (fresh) {
     PD_CUDA(cudaMemsetAsync(c->bd, 0, sizeof(double) * ne, c->stream));  // padding slots stay 0
-    if (c->pairs_ok) {
-      if ((st = alloc(c, &c->dirty, (size_t)c->nslices)) != PD_OK) return st;
-      PD_CUDA(cudaMemsetAsync(c->dirty, 0, (size_t)c->nslices, c->stream));
-    }
+    if (c->pairs_ok) PD_CUDA(cudaMemsetAsync(c->dirty, 0, (size_t)c->nslices, c->stream));
     StepArgs a = make_args(c);
     if (c->dim == 3)
       k_bond_tables<3><<<grid, tb, 0, c->stream>>>(a, c->bA, c->bB);
@@ -2993,19 +3021,25 @@ pd_status ensure_adr(pd_ctx* c) {
   if (!c->lam) {
     const int64_t np = c->n_pad;
     const size_t nblk = (size_t)((np + kAdrBlock - 1) / kAdrBlock);
-    if ((st = alloc(c, &c->lam, np)) != PD_OK) return st;
-    if ((st = alloc(c, &c->gnew, np)) != PD_OK) return st;
-    if ((st = alloc(c, &c->gold, np)) != PD_OK) return st;
-    if ((st = alloc(c, &c->adr_part, nblk)) != PD_OK) return st;
-    if ((st = alloc(c, &c->adr_st, 1)) != PD_OK) return st;
-    if ((st = alloc(c, &c->adr_first, 1)) != PD_OK) return st;
+    double* alpha = nullptr;
+    st = alloc(c, &c->lam, np);
+    if (st == PD_OK) st = alloc(c, &c->gnew, np);
+    if (st == PD_OK) st = alloc(c, &c->gold, np);
+    if (st == PD_OK) st = alloc(c, &c->adr_part, nblk);
+    if (st == PD_OK) st = alloc(c, &c->adr_st, 1);
+    if (st == PD_OK) st = alloc(c, &c->adr_first, 1);
+    if (st == PD_OK) st = alloc(c, &alpha, np);
+    if (st != PD_OK) {  // all of them or none, as alloc_bond_tables
+      drop(c, &c->lam);
+      drop(c, &c->gnew);
+      drop(c, &c->gold);
+      drop(c, &c->adr_part);
+      drop(c, &c->adr_st);
+      drop(c, &c->adr_first);
+      return st;
+    }
     PD_CUDA(cudaMemsetAsync(c->gnew, 0, sizeof(double4) * np, c->stream));
     PD_CUDA(cudaMemsetAsync(c->gold, 0, sizeof(double4) * np, c->stream));
-    double* alpha = nullptr;
-    if (cudaMalloc(&alpha, sizeof(double) * np) != cudaSuccess) {
-      cudaGetLastError();
-      return fail(PD_ERR_OOM, "cudaMalloc of the ADR temporary failed");
-    }
     StepArgs a = make_args(c);
     const int tb = 256;
     const unsigned grid = (unsigned)((np + tb - 1) / tb);
@@ -3018,7 +3052,7 @@ pd_status ensure_adr(pd_ctx* c) {
     }
     cudaError_t e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    cudaFree(alpha);
+    release(c, alpha);
     if (e != cudaSuccess) return cuda_fail(e, "ADR density");
   }
   if (c->adr_restart) {
@@ -3150,6 +3184,7 @@ static void ensure_check_tables(pd_ctx* c) {
   float4* cA = nullptr;
   float4* cu = nullptr;
   if (alloc(c, &cA, (size_t)c->nentries) != PD_OK || alloc(c, &cu, (size_t)c->n_pad) != PD_OK) {
+    release(c, cA);
     clear_error();
     return;
   }

@@ -1,0 +1,66 @@
+"""A step whose device allocations fail (PD_OPT_DEVICE_LIMIT stands for a full device): it reports PD_ERR_OOM, so
+does the next one, the state stays as it was, and once there is room the run is bitwise that of a context that
+always had it (GPU only)."""
+import numpy as np
+import pytest
+
+from paper_2309_11273_gb300 import PD_LINEARIZED, PD_NONLINEAR, PDError, Simulation
+from paper_2309_11273_gb300 import _binding as B
+from paper_2309_11273_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+
+def _sim(dim, kinematics, solver):
+    if dim == 3:
+        w = W.notched_block(12, 8, 7, nsteps=100, seed=5, amp=2e-8)
+        w.flag = w.axis_point = w.axis_dir = None
+    else:
+        w = W.cracked_plate(nx=40, ny=30, crack_cells=20.125)
+        w.u0 = np.random.default_rng(3).normal(0.0, 2e-9, (2, w.n))
+    sim = Simulation(w, kinematics=kinematics, s0=0.0 if solver else None)
+    sim.set_option(B.PD_OPT_SOLVER, solver)
+    return sim
+
+
+def _bytes(sim):
+    return B.pd_get_info(sim.h)[2]
+
+
+def _full_run(make):
+    """(device bytes before the first step, after six steps and a read, the state)."""
+    ref = make()
+    b0 = _bytes(ref)
+    ref.step(6)
+    want = ref.state()
+    b1 = _bytes(ref)
+    ref.close()
+    return b0, b1, want
+
+
+@pytest.mark.parametrize("solver", [B.PD_SOLVER_EXPLICIT, B.PD_SOLVER_ADR])
+@pytest.mark.parametrize("dim,kinematics", [(2, PD_LINEARIZED), (3, PD_LINEARIZED), (2, PD_NONLINEAR), (3, PD_NONLINEAR)])
+def test_a_failed_allocation_leaves_nothing_half_built(dim, kinematics, solver):
+    def make():
+        return _sim(dim, kinematics, solver)
+    b0, b1, want = _full_run(make)
+    refused = 0
+    for part in np.linspace(0.0, 1.0, 13)[:-1]:
+        sim = make()
+        u0 = sim.state()[0]
+        sim.set_option(B.PD_OPT_DEVICE_LIMIT, int(b0 + part * (b1 - b0)))
+        try:
+            sim.step(6)
+        except PDError as e:
+            assert e.status == B.PD_ERR_OOM
+            refused += 1
+            with pytest.raises(PDError) as again:
+                sim.step(6)
+            assert again.value.status == B.PD_ERR_OOM
+            assert np.array_equal(sim.state()[0], u0)
+            sim.set_option(B.PD_OPT_DEVICE_LIMIT, 0)
+            sim.step(6)
+            for x, y in zip(sim.state(), want):
+                assert np.array_equal(x, y)
+        sim.close()
+    assert refused > 0
