@@ -175,7 +175,10 @@ typedef enum {
                               Linearized results are bitwise the same, also when the option is
                               switched between steps; nonlinear theta sums differ in rounding
                               order only.  Has no effect when the build could not pair
-                              every entry (pd_get_option then reports 0). */
+                              every entry, or, with nonlinear bonds, when the device has no room
+                              for the pair form's tables (120 bytes per bond slot against 48; the
+                              single pass then runs until the next build); pd_get_option reports
+                              0 in both cases. */
   PD_OPT_LATTICE = 11,     /* PD_MIXED (linearized or nonlinear bonds): 1 (default) = when every
                               body's particles lie on a regular lattice (bond vectors h n with
                               integer n to within 2^-30 h, uniform volumes, a family |n|^2 <= m^2 for

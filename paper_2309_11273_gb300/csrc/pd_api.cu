@@ -72,6 +72,7 @@ void free_build(pd_ctx* c) {
   c->bY = nullptr;
   c->bC = nullptr;
   c->bX = c->bX2 = nullptr;
+  c->nl_single = false;
   c->lam = nullptr;
   c->gnew = c->gold = nullptr;
   c->adr_part = nullptr;
@@ -666,7 +667,7 @@ pd_status pd_get_option(pd_ctx* c, int32_t option, int64_t* value) {
     case PD_OPT_STAGE: *value = c->stage; break;
     case PD_OPT_EXPIRE_WAITS: *value = c->expire_waits; break;
     case PD_OPT_SOLVER: *value = c->solver; break;
-    case PD_OPT_PAIRS: *value = (c->pairs && c->pairs_ok && c->precision == PD_FP64) ? 1 : 0; break;
+    case PD_OPT_PAIRS: *value = (c->pairs && c->pairs_ok && !c->nl_single && c->precision == PD_FP64) ? 1 : 0; break;
     case PD_OPT_LATTICE: *value = c->built ? (c->lattice ? 1 : 0) : c->lattice_opt; break;
     case PD_OPT_LAT_STAGE: *value = c->lat_stage; break;
     case PD_OPT_SHADOW_LO: *value = c->built ? (c->shadow_lo ? 1 : 0) : c->shadow_lo_opt; break;

@@ -221,6 +221,7 @@ struct pd_ctx {
   double4* bC = nullptr;          // nonlinear FP64 pair form: per-slot constants of pass 1a (see StepArgs)
   double* bX = nullptr;           // nonlinear FP64 pair form: per-slot |xi| V_j
   double* bX2 = nullptr;          // nonlinear FP64 pair form: per-slot |xi|^2 V_j
+  bool nl_single = false;         // nonlinear FP64: the pair form's tables did not fit, the single pass runs
   int bond_cache = 1;             // use the table in the FP64 path
   int pairs = 1;                  // FP64 tabled path: evaluate each bond once per pair (needs pairs_ok)
   int stage = 1;                  // mixed path: TMA-staged index streams (split 1)

@@ -2921,40 +2921,94 @@ pd_status init_disp_w(pd_ctx* c) {
   return PD_OK;
 }
 
-// The per-slot tables of the tabled FP64 path, all of them or none: a step after a failed allocation must
+// The per-slot tables of the linearized FP64 forms, all of them or none: a step after a failed allocation must
 // not find some of them.
 static pd_status alloc_bond_tables(pd_ctx* c, size_t ne) {
-  pd_status st;
-  if (c->kin == PD_NONLINEAR) {
-    if ((st = alloc(c, &c->bA, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bE, ne)) != PD_OK) return st;
-    if (!c->pairs_ok) return PD_OK;
-    if ((st = alloc(c, &c->bt, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bY, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bC, ne)) != PD_OK) return st;
-    if ((st = alloc(c, &c->bX2, ne)) != PD_OK) return st;
-    return alloc(c, &c->bX, ne);
-  }
   const size_t nt = c->dim == 3 ? ne : (3 * ne + 3) / 4;  // 2D rows: 24 bytes (slot_row)
-  if ((st = alloc(c, &c->bA, nt)) != PD_OK) return st;
-  if ((st = alloc(c, &c->bB, nt)) != PD_OK) return st;
-  if ((st = alloc(c, &c->bd, ne)) != PD_OK) return st;
-  if ((st = alloc(c, &c->bS, (size_t)c->n_pad)) != PD_OK) return st;
-  return c->pairs_ok ? alloc(c, &c->dirty, (size_t)c->nslices) : PD_OK;
+  pd_status st = alloc(c, &c->bA, nt);
+  if (st == PD_OK) st = alloc(c, &c->bB, nt);
+  if (st == PD_OK) st = alloc(c, &c->bd, ne);
+  if (st == PD_OK) st = alloc(c, &c->bS, (size_t)c->n_pad);
+  if (st == PD_OK && c->pairs_ok) st = alloc(c, &c->dirty, (size_t)c->nslices);
+  if (st == PD_OK) return PD_OK;
+  drop(c, &c->bA);
+  drop(c, &c->bB);
+  drop(c, &c->bd);
+  drop(c, &c->bS);
+  drop(c, &c->dirty);
+  return st;
 }
 
-static void drop_bond_tables(pd_ctx* c) {
-  drop(c, &c->bA);
-  drop(c, &c->bE);
+// ... and those of the nonlinear pair form beside bA.
+static void drop_nl_pair_tables(pd_ctx* c) {
   drop(c, &c->bt);
   drop(c, &c->bY);
   drop(c, &c->bC);
   drop(c, &c->bX2);
   drop(c, &c->bX);
-  drop(c, &c->bB);
-  drop(c, &c->bd);
-  drop(c, &c->bS);
-  drop(c, &c->dirty);
+}
+static pd_status alloc_nl_pair_tables(pd_ctx* c, size_t ne) {
+  pd_status st = alloc(c, &c->bt, ne);
+  if (st == PD_OK) st = alloc(c, &c->bY, ne);
+  if (st == PD_OK) st = alloc(c, &c->bC, ne);
+  if (st == PD_OK) st = alloc(c, &c->bX2, ne);
+  if (st == PD_OK) st = alloc(c, &c->bX, ne);
+  if (st != PD_OK) drop_nl_pair_tables(c);
+  return st;
+}
+
+// The nonlinear FP64 tables of the form that steps next: bA (32 bytes per slot) with the pair form's (88) or the
+// single pass's bE (16).  The other form's are given back when memory is short, and where the pair form's do not
+// fit even so, the body runs the single pass for the rest of the build (nl_single), whose 48 bytes per slot are
+// fewer than either form took before the pair form tabled its constants.
+static pd_status ensure_nl_tables(pd_ctx* c, size_t ne) {
+  const int tb = 256;
+  const unsigned grid = (unsigned)((c->n_pad + tb - 1) / tb);
+  pd_status st;
+  if (!c->bA) {
+    if ((st = alloc(c, &c->bA, ne)) != PD_OK) return st;
+    const StepArgs a = make_args(c);
+    if (c->dim == 3)
+      k_bond_tables_nl<3><<<grid, tb, 0, c->stream>>>(a, c->bA);
+    else
+      k_bond_tables_nl<2><<<grid, tb, 0, c->stream>>>(a, c->bA);
+    PD_CUDA(cudaGetLastError());
+  }
+  if (c->pairs && c->pairs_ok && !c->nl_single && !c->bX) {
+    st = alloc_nl_pair_tables(c, ne);
+    if (st != PD_OK && c->bE) {
+      drop(c, &c->bE);
+      st = alloc_nl_pair_tables(c, ne);
+    }
+    if (st == PD_OK) {
+      PD_CUDA(cudaMemsetAsync(c->bt, 0, sizeof(double) * ne, c->stream));
+      PD_CUDA(cudaMemsetAsync(c->bY, 0, sizeof(double4) * ne, c->stream));
+      const StepArgs a = make_args(c);
+      if (c->dim == 3)
+        k_bond_tables_nlp<3><<<grid, tb, 0, c->stream>>>(a, c->bC, c->bX, c->bX2);
+      else
+        k_bond_tables_nlp<2><<<grid, tb, 0, c->stream>>>(a, c->bC, c->bX, c->bX2);
+      PD_CUDA(cudaGetLastError());
+    } else {
+      clear_error();
+      c->nl_single = true;
+    }
+  }
+  if (c->pairs && c->bX) return PD_OK;
+  if (!c->bE) {
+    st = alloc(c, &c->bE, ne);
+    if (st != PD_OK && c->bX) {
+      drop_nl_pair_tables(c);
+      st = alloc(c, &c->bE, ne);
+    }
+    if (st != PD_OK) {
+      drop(c, &c->bA);
+      c->nl_single = false;
+      return st;
+    }
+    PD_CUDA(cudaMemsetAsync(c->bE, 0, sizeof(double2) * ne, c->stream));
+  }
+  return PD_OK;
 }
 
 // Allocates and fills the per-slot tables of the tabled FP64 path (once per build), and brings the
@@ -2962,38 +3016,12 @@ static void drop_bond_tables(pd_ctx* c) {
 pd_status ensure_bond_cache(pd_ctx* c) {
   if (!c->bond_cache || c->precision != PD_FP64) return PD_OK;
   const size_t ne = (size_t)std::max<int64_t>(c->nentries, 32);
+  if (c->kin == PD_NONLINEAR) return ensure_nl_tables(c, ne);
   const int tb = 256;
   const unsigned grid = (unsigned)((c->n_pad + tb - 1) / tb);
-  const bool fresh = !c->bA;
-  if (fresh) {
+  if (!c->bA) {
     const pd_status st = alloc_bond_tables(c, ne);
-    if (st != PD_OK) {
-      drop_bond_tables(c);
-      return st;
-    }
-  }
-  if (c->kin == PD_NONLINEAR) {
-    if (!fresh) return PD_OK;
-    PD_CUDA(cudaMemsetAsync(c->bE, 0, sizeof(double2) * ne, c->stream));
-    if (c->pairs_ok) {
-      PD_CUDA(cudaMemsetAsync(c->bt, 0, sizeof(double) * ne, c->stream));
-      PD_CUDA(cudaMemsetAsync(c->bY, 0, sizeof(double4) * ne, c->stream));
-      StepArgs ax = make_args(c);
-      if (c->dim == 3)
-        k_bond_tables_nlp<3><<<grid, tb, 0, c->stream>>>(ax, c->bC, c->bX, c->bX2);
-      else
-        k_bond_tables_nlp<2><<<grid, tb, 0, c->stream>>>(ax, c->bC, c->bX, c->bX2);
-      PD_CUDA(cudaGetLastError());
-    }
-    StepArgs a = make_args(c);
-    if (c->dim == 3)
-      k_bond_tables_nl<3><<<grid, tb, 0, c->stream>>>(a, c->bA);
-    else
-      k_bond_tables_nl<2><<<grid, tb, 0, c->stream>>>(a, c->bA);
-    PD_CUDA(cudaGetLastError());
-    return PD_OK;
-  }
-  if (fresh) {
+    if (st != PD_OK) return st;
     PD_CUDA(cudaMemsetAsync(c->bd, 0, sizeof(double) * ne, c->stream));  // padding slots stay 0
     if (c->pairs_ok) PD_CUDA(cudaMemsetAsync(c->dirty, 0, (size_t)c->nslices, c->stream));
     StepArgs a = make_args(c);
@@ -3200,6 +3228,8 @@ static void ensure_check_tables(pd_ctx* c) {
 
 pd_status launch_refresh_check(pd_ctx* c) {
   if (!c->check_pending) return PD_OK;
+  if (c->kin == PD_NONLINEAR && c->bA)  // after a switch of PD_OPT_PAIRS: the other form's
+    if (const pd_status st = ensure_bond_cache(c); st != PD_OK) return st;
   ensure_check_tables(c);
   StepArgs a = make_args(c);
   a.check = 1;
@@ -3357,7 +3387,10 @@ pd_status run_steps(pd_ctx* c, int64_t nsteps) {
   pd_status st = ensure_bond_cache(c);
   if (st != PD_OK) return st;
   if (c->precision == PD_FP64 && !c->bond_cache) c->bs_stale = true;  // untabled kernels break bonds
-  if ((st = ensure_adr(c)) != PD_OK) return st;
+  if ((st = ensure_adr(c)) != PD_OK) {
+    c->nl_single = false;  // no step was taken: the next call chooses the form again
+    return st;
+  }
   int64_t left = nsteps;
   const bool mixed = c->precision == PD_MIXED;
   const ResidentPlan plan = mixed ? resident_lat_plan(c) : resident_plan(c);

@@ -64,3 +64,44 @@ def test_a_failed_allocation_leaves_nothing_half_built(dim, kinematics, solver):
                 assert np.array_equal(x, y)
         sim.close()
     assert refused > 0
+
+
+@pytest.mark.parametrize("dim", [2, 3])
+def test_nonlinear_bodies_take_the_single_pass_where_the_pair_tables_do_not_fit(dim):
+    b0, b_pair, _ = _full_run(lambda: _sim(dim, PD_NONLINEAR, B.PD_SOLVER_EXPLICIT))
+
+    def single():
+        sim = _sim(dim, PD_NONLINEAR, B.PD_SOLVER_EXPLICIT)
+        sim.set_option(B.PD_OPT_PAIRS, 0)
+        return sim
+    _, b_single, want = _full_run(single)
+    # 120 and 48 bytes per slot: neither form holds the other's tables
+    assert 2.4 * (b_single - b0) < b_pair - b0 < 2.6 * (b_single - b0)
+    for limit in (b_single, (b_single + b_pair) // 2, b_pair - 1):
+        sim = _sim(dim, PD_NONLINEAR, B.PD_SOLVER_EXPLICIT)
+        sim.set_option(B.PD_OPT_DEVICE_LIMIT, limit)
+        sim.step(6)
+        for x, y in zip(sim.state(), want):
+            assert np.array_equal(x, y)
+        assert sim.get_option(B.PD_OPT_PAIRS) == 0
+        sim.close()
+
+
+@pytest.mark.parametrize("read", [False, True])
+def test_switching_the_nonlinear_form_when_only_one_fits(read):
+    _, b_pair, _ = _full_run(lambda: _sim(3, PD_NONLINEAR, B.PD_SOLVER_EXPLICIT))
+    out = []
+    for limit in (0, b_pair):
+        sim = _sim(3, PD_NONLINEAR, B.PD_SOLVER_EXPLICIT)
+        sim.set_option(B.PD_OPT_DEVICE_LIMIT, limit)
+        for pairs in (1, 0, 1, 0):
+            sim.step(3)
+            sim.set_option(B.PD_OPT_PAIRS, pairs)
+            if read:
+                sim.damage()  # the pending check, in the form just chosen
+            sim.step(2)
+            assert sim.get_option(B.PD_OPT_PAIRS) == pairs
+        out.append(list(sim.state()) + [sim.damage()])
+        sim.close()
+    for x, y in zip(*out):
+        assert np.array_equal(x, y)
