@@ -334,7 +334,11 @@ ResidentPlan resident_plan(const pd_ctx* c) {
 
 pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done) {
   *done = false;
-  if (pd_status st = ensure_grid_bar(c); st != PD_OK) return st;
+  if (const pd_status st = ensure_grid_bar(c); st != PD_OK) {
+    if (st != PD_ERR_OOM) return st;
+    clear_error();
+    return PD_OK;  // no room for the barrier's words: the pass kernels take the steps
+  }
   ResidentArgs r{};
   r.disp = c->disp[c->cur];
   r.disp_out = c->disp[c->cur ^ 1];

@@ -571,7 +571,11 @@ ResidentPlan resident_lat_plan(const pd_ctx* c) {
 
 pd_status run_resident_lat(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done) {
   *done = false;
-  if (pd_status st = ensure_grid_bar(c); st != PD_OK) return st;
+  if (const pd_status st = ensure_grid_bar(c); st != PD_OK) {
+    if (st != PD_ERR_OOM) return st;
+    clear_error();
+    return PD_OK;  // no room for the barrier's words: the pass kernels take the steps
+  }
   LatRun r{};
   for (int k = 0; k < 2; ++k) {
     const int s = c->cur ^ k;

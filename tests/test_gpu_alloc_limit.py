@@ -4,7 +4,7 @@ always had it (GPU only)."""
 import numpy as np
 import pytest
 
-from paper_2309_11273_gb300 import PD_LINEARIZED, PD_NONLINEAR, PDError, Simulation
+from paper_2309_11273_gb300 import PD_FP64, PD_LINEARIZED, PD_MIXED, PD_NONLINEAR, PDError, Simulation
 from paper_2309_11273_gb300 import _binding as B
 from paper_2309_11273_gb300 import workloads as W
 
@@ -104,4 +104,22 @@ def test_switching_the_nonlinear_form_when_only_one_fits(read):
         out.append(list(sim.state()) + [sim.damage()])
         sim.close()
     for x, y in zip(*out):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("precision", [PD_FP64, PD_MIXED])
+def test_no_room_for_the_resident_kernels_barrier(precision):
+    def make():
+        w = W.cracked_plate(nx=40, ny=30, crack_cells=20.125)
+        return Simulation(w, precision=precision)
+    ref = make()
+    ref.step(6)
+    want = ref.state()
+    sim = make()
+    sim.set_option(B.PD_OPT_PROFILE, 1)  # the pass kernels: every table, no barrier yet
+    sim.step(1)
+    sim.set_option(B.PD_OPT_PROFILE, 0)
+    sim.set_option(B.PD_OPT_DEVICE_LIMIT, _bytes(sim))
+    sim.step(5)
+    for x, y in zip(sim.state(), want):
         assert np.array_equal(x, y)
