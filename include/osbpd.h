@@ -46,7 +46,7 @@ typedef enum {
   PD_ERR_OOM = -3,      /* a device or host allocation failed */
   PD_ERR_CUDA = -4,     /* a CUDA runtime call failed */
   PD_ERR_NUMERIC = -5,  /* the state became non-finite or exceeded the divergence guard */
-  PD_ERR_TIMEOUT = -6   /* reserved for bounded device waits */
+  PD_ERR_TIMEOUT = -6   /* a bounded wait on the device expired */
 } pd_status;
 
 /* Eq 1.8 / 1.15 / 1.16 rows. */
@@ -166,7 +166,8 @@ typedef enum {
                               of the GPU's global timer) expires; the warps skip their outputs
                               and the next pd_sync / pd_get_* returns PD_ERR_TIMEOUT.  In the
                               resident kernels (PD_OPT_GRAPH_CHUNK) a block does not arrive at the grid
-                              barrier, with the same end after 4 s.  Default 0. */
+                              barrier, whose wait expires after 4 s: PD_ERR_TIMEOUT as well, and the
+                              state is lost half way through the call (see pd_step).  Default 0. */
   PD_OPT_SOLVER = 9,       /* pd_solver: PD_SOLVER_EXPLICIT (0, default) or PD_SOLVER_ADR (1) */
   PD_OPT_PAIRS = 10,       /* PD_FP64 with the bond cache on: 1 (default) = form each bond's
                               extension (linearized: xi.(u_j - u_i); nonlinear: e and 1/|Y|) and
@@ -293,7 +294,13 @@ pd_status pd_set_state(pd_ctx* c, const double* u, const double* v);
  * update with boundary conditions at t_{n+1}.  Runs as CUDA-graph chunks of PD_OPT_GRAPH_CHUNK
  * steps when graphs are enabled.  Enqueue only: returns before the GPU finishes.  A state that
  * became non-finite is reported by the next pd_sync / pd_get_* as PD_ERR_NUMERIC (a one-pass check
- * over the particles is enqueued after the steps). */
+ * over the particles is enqueued after the steps).
+ * When the bounded wait (4 s) of a resident launch's grid barrier expires, the next pd_sync / pd_get_*
+ * returns PD_ERR_TIMEOUT and the state is lost: displacements, velocities and bond status belong to no
+ * common step, and the step count is the one enqueued.  pd_step, pd_autotune, pd_check_state,
+ * pd_save_state and pd_get_* (but not pd_get_info, pd_get_option, pd_get_profile) then return
+ * PD_ERR_STATE until pd_set_state (which leaves the bond status as it is), pd_load_state or
+ * pd_build_neighbors. */
 pd_status pd_step(pd_ctx* c, int64_t nsteps);
 
 /* Waits for all work of the context. */

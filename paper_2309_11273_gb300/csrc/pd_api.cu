@@ -80,6 +80,7 @@ void free_build(pd_ctx* c) {
   c->adr_first = nullptr;
   c->bar = nullptr;
   c->bar_base = 0;
+  c->lost = false;
   c->adr_restart = true;
   c->diag_theta = nullptr;
   c->diag_part = nullptr;
@@ -433,6 +434,8 @@ pd_status pd_set_state(pd_ctx* c, const double* u, const double* v) {
   c->check_pending = false;
   c->skip_next_check = true;
   c->adr_restart = true;
+  c->lost = false;
+  if ((st = reset_grid_bar(c)) != PD_OK) return st;  // a launch that gave up unread: the new state steps all the same
   PD_CUDA(cudaStreamSynchronize(c->stream));
   return PD_OK;
 }
@@ -455,6 +458,7 @@ pd_status pd_get_damage(pd_ctx* c, double* phi) {
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
   if (!phi) return fail(PD_ERR_ARG, "phi is NULL");
+  if (c->lost) return check_lost(c);
   if ((st = launch_refresh_check(c)) != PD_OK) return st;
   if ((st = check_device_error(c)) != PD_OK) return st;
   if ((st = launch_damage(c, c->scratch)) != PD_OK) return st;
@@ -466,6 +470,7 @@ pd_status pd_get_damage(pd_ctx* c, double* phi) {
 pd_status pd_get_state(pd_ctx* c, double* u, double* v, double* theta) {
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
+  if (c->lost) return check_lost(c);
   if (cudaStreamQuery(c->stream) == cudaErrorNotReady) {  // the GPU still steps
     cudaGetLastError();
     populate(u, sizeof(double) * c->dim * c->n);
@@ -501,6 +506,7 @@ pd_status pd_get_neighbors(pd_ctx* c, int64_t* row_ptr, int32_t* col, uint8_t* i
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
   if (!row_ptr || !col) return fail(PD_ERR_ARG, "row_ptr and col are required");
+  if ((st = check_lost(c)) != PD_OK) return st;
   if ((st = launch_refresh_check(c)) != PD_OK) return st;
   std::vector<int64_t> sptr(c->nslices + 1);
   std::vector<int32_t> hcol(c->nentries);
@@ -542,6 +548,7 @@ pd_status pd_get_stats(pd_ctx* c, pd_stats* s) {
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
   if (!s) return fail(PD_ERR_ARG, "stats is NULL");
+  if ((st = check_lost(c)) != PD_OK) return st;
   if ((st = launch_refresh_check(c)) != PD_OK) return st;
   std::vector<uint32_t> hbits(c->nentries / 32);
   unsigned long long cnt[2];
@@ -569,6 +576,7 @@ pd_status pd_check_state(pd_ctx* c, double max_abs) {
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
   if (!(max_abs > 0)) return fail(PD_ERR_ARG, "max_abs_u must be > 0");
+  if ((st = check_lost(c)) != PD_OK) return st;
   int nonfinite = 0;
   double m = 0.0;
   if ((st = max_abs_u(c, &m, &nonfinite)) != PD_OK) return st;
@@ -756,6 +764,7 @@ pd_status pd_save_state(pd_ctx* c, const char* path) {
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
   if (!path) return fail(PD_ERR_ARG, "path is NULL");
+  if (c->lost) return check_lost(c);
   if ((st = check_device_error(c)) != PD_OK) return st;
   CheckpointHeader hd{};
   std::memcpy(hd.magic, kCkptMagic, 8);
@@ -837,6 +846,7 @@ pd_status pd_load_state(pd_ctx* c, const char* path) {
   c->check_pending = (hd.flags & 1) != 0;
   c->skip_next_check = (hd.flags & 2) != 0;
   c->bs_stale = true;  // the loaded status bits
+  c->lost = false;
   c->adr_restart = true;
   drop_graphs(c);
   return PD_OK;
@@ -912,6 +922,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
   pd_status st = check_ctx(c, true);
   if (st != PD_OK) return st;
   if (trial_steps < 1) return fail(PD_ERR_ARG, "trial_steps must be >= 1");
+  if ((st = check_lost(c)) != PD_OK) return st;
   cudaDeviceProp prop;
   PD_CUDA(cudaGetDeviceProperties(&prop, c->device));
   char key[512];

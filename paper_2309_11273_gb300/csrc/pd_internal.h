@@ -264,6 +264,7 @@ struct pd_ctx {
   int sms = 0;                  // SMs of the device; 0: no cooperative launch (the resident step kernel is off)
   unsigned* bar = nullptr;      // resident step kernel: grid barrier (arrivals, abort)
   unsigned bar_base = 0;        // ... arrivals enqueued so far
+  bool lost = false;            // a resident launch gave up half way and was reported: there is no state to read or step
   int graph_chunk = 100;
   int profile = 0;
   int validate = 0;
@@ -323,6 +324,8 @@ pd_status apply_bc_now(pd_ctx* c);
 pd_status sync_shadow(pd_ctx* c);
 pd_status max_abs_u(pd_ctx* c, double* out, int* nonfinite);
 pd_status check_device_error(pd_ctx* c);
+pd_status check_lost(pd_ctx* c);       // PD_OK unless a resident launch lost the state (reported or not)
+pd_status reset_grid_bar(pd_ctx* c);   // after the work enqueued so far, the resident kernels may run again
 pd_status run_steps(pd_ctx* c, int64_t nsteps);
 pd_status read_profile(pd_ctx* c);
 // The resident step kernel (pd_resident.cu): all steps of a call in one cooperative launch, for bodies

@@ -3336,18 +3336,45 @@ pd_status check_device_error(pd_ctx* c) {
   PD_CUDA(cudaStreamSynchronize(c->stream));
   if (flag) {
     PD_CUDA(cudaMemsetAsync(c->counters + 4, 0, sizeof(flag), c->stream));
-    if (c->bar) {  // the resident step kernel's barrier starts over
-      PD_CUDA(cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
-      c->bar_base = 0;
+    unsigned gave_up = 0;
+    if (c->bar) {
+      PD_CUDA(cudaMemcpyAsync(&gave_up, c->bar + 1, sizeof(gave_up), cudaMemcpyDeviceToHost, c->stream));
+      PD_CUDA(cudaStreamSynchronize(c->stream));
+      if (pd_status st = reset_grid_bar(c); st != PD_OK) return st;
     }
-    return fail(PD_ERR_TIMEOUT, "a staged neighbour-index copy or a grid barrier did not complete within the wait "
-                                "limit; the steps' results were not written");
+    if (gave_up) {
+      c->lost = true;
+      return fail(PD_ERR_TIMEOUT, "a grid barrier of the resident step kernel did not complete within the wait limit: "
+                                  "the state is lost (pd_set_state, pd_load_state or pd_build_neighbors gives a new one)");
+    }
+    return fail(PD_ERR_TIMEOUT, "a staged neighbour-index copy did not complete within the wait limit; "
+                                "the step's results were not written");
   }
   if (nonfinite) {
     PD_CUDA(cudaMemsetAsync(c->counters + 5, 0, sizeof(nonfinite), c->stream));
     return fail(PD_ERR_NUMERIC, "the displacement became non-finite (the run diverged)");
   }
   return PD_OK;
+}
+
+pd_status reset_grid_bar(pd_ctx* c) {
+  if (!c->bar) return PD_OK;
+  PD_CUDA(cudaMemsetAsync(c->bar, 0, 2 * sizeof(unsigned), c->stream));
+  c->bar_base = 0;
+  return PD_OK;
+}
+
+// A resident launch that gives up has moved some blocks' particles and broken some of their bonds up to the step
+// where the wait ran out, and keeps the velocities of its start: neither the old state nor a new one.
+pd_status check_lost(pd_ctx* c) {
+  if (c->lost)
+    return fail(PD_ERR_STATE, "the state was lost when a grid barrier ran out of time (PD_ERR_TIMEOUT): set a new one "
+                              "with pd_set_state, pd_load_state or pd_build_neighbors");
+  if (!c->bar) return PD_OK;
+  unsigned gave_up = 0;
+  PD_CUDA(cudaMemcpyAsync(&gave_up, c->bar + 1, sizeof(gave_up), cudaMemcpyDeviceToHost, c->stream));
+  PD_CUDA(cudaStreamSynchronize(c->stream));
+  return gave_up ? check_device_error(c) : PD_OK;
 }
 
 pd_status max_abs_u(pd_ctx* c, double* out, int* nonfinite) {
@@ -3374,6 +3401,7 @@ constexpr int64_t kResidentSteps = 1000;
 // chunks of graph_chunk steps, then single steps.
 pd_status run_steps(pd_ctx* c, int64_t nsteps) {
   if (nsteps <= 0) return PD_OK;
+  if (c->lost) return check_lost(c);
   if (c->prm[0].influence == PD_W_INV) {
     // w = delta / |xi| lives in the FP64 per-slot tables and in the lattice kernels' direction table
     if (c->solver == PD_SOLVER_ADR)

@@ -210,3 +210,53 @@ def test_unread_calls_on_breaking_blocks(shape):
 @pytest.mark.parametrize("nx,ny", [(40, 40), (341, 340)])
 def test_unread_calls_on_breaking_mixed_plates(nx, ny, kinematics):
     _same_unread(lambda: Simulation(_plate(nx, ny), precision=PD_MIXED, kinematics=kinematics), [1, 1, 1, 2, 3, 12, 30])
+
+
+@pytest.mark.parametrize("first", ["sync", "state", "damage", "stats", "neighbors", "check_state", "autotune", "save"])
+def test_an_expired_barrier_loses_the_state(first, tmp_path):
+    """The first call that meets it reports the timeout; then nothing reads or steps the state until there is a new
+    one (a checkpoint brings back the bond status too)."""
+    w = _plate(60, 40)
+    ckpt = str(tmp_path / "before")
+    ref = Simulation(w, precision=PD_MIXED if first == "state" else 0)
+    ref.step(30)
+    ref.save_state(ckpt)
+    ref.step(20)
+    sim = Simulation(w, precision=PD_MIXED if first == "state" else 0)
+    sim.set_option(B.PD_OPT_EXPIRE_WAITS, 1)
+    sim.step(3)
+    calls = {"sync": sim.sync, "state": sim.state, "damage": sim.damage, "stats": sim.stats, "neighbors": sim.neighbors,
+             "check_state": lambda: B._check(B.pd_check_state(sim.h, 1.0)), "autotune": lambda: B.pd_autotune(sim.h, 1),
+             "save": lambda: sim.save_state(str(tmp_path / "lost")), "step": lambda: sim.step(1)}
+    with pytest.raises(PDError) as e:
+        calls[first]()
+    assert e.value.status == B.PD_ERR_TIMEOUT
+    sim.set_option(B.PD_OPT_EXPIRE_WAITS, 0)
+    for name, call in calls.items():
+        if name == "sync":
+            call()
+            continue
+        with pytest.raises(PDError) as e:
+            call()
+        assert e.value.status == B.PD_ERR_STATE, name
+    sim.load_state(ckpt)
+    sim.step(20)
+    for x, y in zip(list(sim.state()) + [sim.damage()], list(ref.state()) + [ref.damage()]):
+        assert np.array_equal(x, y)
+
+
+def test_a_state_set_before_the_timeout_is_read_steps_all_the_same():
+    w = W.plate_vibration(nx=40, ny=20, nsteps=20)
+    sim = Simulation(w, s0=0.0)
+    sim.set_option(B.PD_OPT_EXPIRE_WAITS, 1)
+    sim.step(3)
+    sim.set_option(B.PD_OPT_EXPIRE_WAITS, 0)
+    sim.set_state(w.initial_u())
+    sim.step(20)
+    with pytest.raises(PDError) as e:
+        sim.sync()
+    assert e.value.status == B.PD_ERR_TIMEOUT
+    ref = Simulation(w, s0=0.0)
+    ref.step(20)
+    for x, y in zip(sim.state(), ref.state()):
+        assert np.array_equal(x, y)
