@@ -337,7 +337,9 @@ pd_status pd_check_state(pd_ctx* c, double max_abs_u);
  * restores the state, bond status and step count afterwards.  PD_FP64 contexts with the bond cache
  * also try both settings of PD_OPT_PAIRS for every mapping and keep the faster (read it back with
  * pd_get_option).  If the environment variable PD_AUTOTUNE_CACHE names a file, results are looked
- * up / appended there under a key made of the problem sizes, precision and device name.
+ * up / appended there under a key made of the problem sizes, the form of the step (precision, kinematics,
+ * solver, influence function, layout, options that choose kernels) and the device name.  Lines of another
+ * format are passed over.
  * *block / *split (may be NULL) receive the choice. */
 pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block, int32_t* split);
 

@@ -12,6 +12,7 @@
 #include <string>
 
 #include "pd_internal.h"
+#include "pd_tune.h"
 
 namespace pd {
 
@@ -925,34 +926,33 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
   if ((st = check_lost(c)) != PD_OK) return st;
   cudaDeviceProp prop;
   PD_CUDA(cudaGetDeviceProperties(&prop, c->device));
-  char key[512];
-  std::snprintf(key, sizeof(key), "osbpd n=%lld bonds=%lld entries=%lld dim=%d prec=%d bodies=%d lattice=%d dev=%s",
-                (long long)c->n, (long long)c->nbonds, (long long)c->nentries, c->dim, c->precision,
-                c->nbodies, c->lattice ? 1 : 0, prop.name);
-  for (char* p = key; *p; ++p)
-    if (*p == '\n' || *p == '|') *p = ' ';
+  TuneProblem problem;
+  problem.n = c->n;
+  problem.bonds = c->nbonds;
+  problem.entries = c->nentries;
+  problem.dim = c->dim;
+  problem.precision = c->precision;
+  problem.bodies = c->nbodies;
+  problem.kinematics = c->kin;
+  problem.solver = c->solver;
+  problem.influence = c->prm[0].influence;
+  problem.lattice = c->lattice ? 1 : 0;
+  problem.shadow_lo = c->shadow_lo ? 1 : 0;
+  problem.bond_cache = c->bond_cache;
+  problem.stage = c->stage;
+  problem.validate = c->validate;
+  problem.device = prop.name;
+  const std::string key = tune_key(problem);
   const char* cache = std::getenv("PD_AUTOTUNE_CACHE");
-  int best_block = -1, best_split = -1, best_pairs = -1, best_lat = -1, best_auto = 0;
+  TuneChoice best;
   if (cache) {
     if (FILE* f = std::fopen(cache, "r")) {
       char line[700];
-      while (std::fgets(line, sizeof(line), f)) {
-        char* bar = std::strchr(line, '|');
-        if (!bar) continue;
-        *bar = 0;
-        int b = 0, s = 0, pr = -1, rg = -1, am = 0;
-        if (std::strcmp(line, key) == 0 && std::sscanf(bar + 1, "%d %d %d %d %d", &b, &s, &pr, &rg, &am) >= 2) {
-          best_block = b;
-          best_split = s;
-          best_pairs = pr;
-          best_lat = rg;
-          best_auto = am;
-        }
-      }
+      while (std::fgets(line, sizeof(line), f)) tune_parse(line, key, &best);
       std::fclose(f);
     }
   }
-  if (best_block < 0) {
+  if (best.block < 0) {
     // snapshot of everything a step modifies
     const int64_t np = c->n_pad;
     double4 *su = nullptr, *sv = nullptr, *sg = nullptr;
@@ -1016,12 +1016,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     const int stage0 = c->lat_stage;
-    int best_ring = stage0;
-    struct Candidate {
-      int block, split, pairs, ring;
-      bool automatic;
-    };
-    std::vector<Candidate> cands;
+    std::vector<TuneChoice> cands;
     c->auto_map = true;
     c->pairs = pairs0;
     // the automatic choice, where it is more than launch shapes: the resident step kernel
@@ -1036,7 +1031,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
           for (int po = 0; po < (try_pairs ? 2 : 1); ++po)
             cands.push_back({bl, sp, try_pairs ? pair_opts[po] : pairs0, stage0, false});
       }
-    for (const Candidate& cd : cands) {
+    for (const TuneChoice& cd : cands) {
       c->auto_map = cd.automatic;
       c->block = cd.block;
       c->split = cd.split;
@@ -1056,11 +1051,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
       cudaEventElapsedTime(&ms, e0, e1);
       if (ms < best_ms) {
         best_ms = ms;
-        best_block = cd.block;
-        best_split = cd.split;
-        best_pairs = cd.pairs;
-        best_ring = cd.ring;
-        best_auto = cd.automatic ? 1 : 0;
+        best = cd;
       }
     }
     c->pairs = pairs0;
@@ -1080,25 +1071,24 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     c->auto_map = auto0;
     if (st != PD_OK) return st;
     if (st2 != PD_OK) return st2;
-    best_lat = best_ring;
-    if (cache && best_block > 0) {
+    if (cache && best.block > 0) {
       if (FILE* f = std::fopen(cache, "a")) {
-        std::fprintf(f, "%s|%d %d %d %d %d\n", key, best_block, best_split, best_pairs, best_ring, best_auto);
+        std::fputs(tune_line(key, best).c_str(), f);
         std::fclose(f);
       }
     }
   }
-  c->block = best_block;
-  c->split = best_split;
-  c->auto_map = best_auto != 0;
-  if (best_lat >= 0) c->lat_stage = best_lat;
-  if (best_pairs >= 0) {
-    if ((best_pairs != 0) != (c->pairs != 0)) c->bs_stale = true;  // as a PD_OPT_PAIRS switch
-    c->pairs = best_pairs;
+  c->block = best.block;
+  c->split = best.split;
+  c->auto_map = best.automatic;
+  if (best.ring >= 0) c->lat_stage = best.ring;
+  if (best.pairs >= 0) {
+    if ((best.pairs != 0) != (c->pairs != 0)) c->bs_stale = true;  // as a PD_OPT_PAIRS switch
+    c->pairs = best.pairs;
   }
   drop_graphs(c);
-  if (block_out) *block_out = best_block;
-  if (split_out) *split_out = best_split;
+  if (block_out) *block_out = best.block;
+  if (split_out) *split_out = best.split;
   return PD_OK;
 }
 
