@@ -332,15 +332,17 @@ pd_status pd_get_stats(pd_ctx* c, pd_stats* s);
 pd_status pd_check_state(pd_ctx* c, double max_abs_u);
 
 /* Picks the launch mapping (threads per block, warps per 32-particle slice) of the step kernels by
- * timing trial_steps steps of every candidate on the context's own data (the automatic choice with its
- * resident kernel among them, where it applies), keeps the fastest, and
+ * timing trial_steps steps of every candidate on the context's own data, keeps the fastest, and
  * restores the state, bond status and step count afterwards.  PD_FP64 contexts with the bond cache
  * also try both settings of PD_OPT_PAIRS for every mapping and keep the faster (read it back with
  * pd_get_option).  If the environment variable PD_AUTOTUNE_CACHE names a file, results are looked
  * up / appended there under a key made of the problem sizes, the form of the step (precision, kinematics,
  * solver, influence function, layout, options that choose kernels) and the device name.  Lines of another
  * format are passed over.
- * *block / *split (may be NULL) receive the choice. */
+ * In PD_FP64 and on the lattice layout the automatic shapes of a context without a mapping are among the
+ * candidates (with the resident kernels where they apply), also in a context whose mapping was set: where
+ * they are the fastest, they are what the context runs from then on.
+ * *block / *split (may be NULL) receive the choice; 256 / 1 for the automatic shapes. */
 pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block, int32_t* split);
 
 pd_status pd_set_option(pd_ctx* c, int32_t option, int64_t value);

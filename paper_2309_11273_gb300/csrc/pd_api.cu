@@ -1005,32 +1005,15 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
     c->profile = 0;
     c->graph_chunk = 0;
     double best_ms = 1e300;
-    const int blocks[] = {64, 128, 256, 512};
-    const int splits[] = {1, 2, 4};
     // FP64 with the pair tables: the pair form (one more launch per step, fewer FP64 instructions)
     // against the single pass, which wins on small bodies where launches dominate
     const int pairs0 = c->pairs;
     const bool try_pairs = c->precision == PD_FP64 && c->pairs_ok && c->bond_cache;
-    const int pair_opts[2] = {1, 0};
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     const int stage0 = c->lat_stage;
-    std::vector<TuneChoice> cands;
-    c->auto_map = true;
-    c->pairs = pairs0;
-    // the automatic choice, where it is more than launch shapes: the resident step kernel
-    if (resident_plan(c).split || resident_lat_plan(c).split) cands.push_back({block0, split0, pairs0, stage0, true});
-    for (int bl : blocks)
-      for (int sp : splits) {
-        if ((bl / 32) % sp) continue;
-        if (c->lattice && sp != 1) continue;  // the lattice kernels run one warp per slice
-        if (c->lattice)
-          for (int ring = 0; ring < 4; ++ring) cands.push_back({bl, sp, pairs0, ring, false});
-        else
-          for (int po = 0; po < (try_pairs ? 2 : 1); ++po)
-            cands.push_back({bl, sp, try_pairs ? pair_opts[po] : pairs0, stage0, false});
-      }
+    const std::vector<TuneChoice> cands = tune_candidates(c->precision == PD_FP64, c->lattice, try_pairs, pairs0, stage0);
     for (const TuneChoice& cd : cands) {
       c->auto_map = cd.automatic;
       c->block = cd.block;

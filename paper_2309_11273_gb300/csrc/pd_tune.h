@@ -1,9 +1,11 @@
-// The cache lines of pd_autotune: "key|block split pairs ring automatic".  No CUDA here: a host test compiles it.
+// The candidates of pd_autotune and its cache lines, "key|block split pairs ring automatic".  No CUDA here: a host
+// test compiles it.
 #pragma once
 
 #include <cstdio>
 #include <cstring>
 #include <string>
+#include <vector>
 
 namespace pd {
 
@@ -12,6 +14,32 @@ struct TuneChoice {
   int block = -1, split = -1, pairs = -1, ring = -1;
   bool automatic = false;
 };
+
+// The mappings that are timed.  The automatic one comes first wherever it is more than one (block, split): the FP64
+// forms give pass 1a a shape of its own and small bodies the resident kernel, and the lattice kernels a ring beside
+// their block, so that no explicit mapping stands for what an untuned context runs.
+inline std::vector<TuneChoice> tune_candidates(bool fp64, bool lattice, bool try_pairs, int pairs, int ring) {
+  std::vector<TuneChoice> r;
+  const int npairs = try_pairs ? 2 : 1;
+  auto add = [&](int block, int split, int k, int rg, bool automatic) {
+    TuneChoice t;
+    t.block = block;
+    t.split = split;
+    t.pairs = try_pairs ? 1 - k : pairs;
+    t.ring = rg;
+    t.automatic = automatic;
+    r.push_back(t);
+  };
+  if (fp64 || lattice)
+    for (int k = 0; k < npairs; ++k) add(256, 1, k, ring, true);  // (the options as a new context has them)
+  for (int block : {64, 128, 256, 512})
+    for (int split : {1, 2, 4}) {
+      if ((block / 32) % split) continue;
+      if (lattice && split != 1) continue;  // the lattice kernels run one warp per slice
+      for (int k = 0; k < (lattice ? 4 : npairs); ++k) add(block, split, lattice ? 0 : k, lattice ? k : ring, false);
+    }
+  return r;
+}
 
 // What the fastest mapping depends on.  Everything that decides which kernels a step runs belongs to it: a choice
 // made for one form (nonlinear bonds, say, which have no resident kernel in FP64) must not be taken for another.

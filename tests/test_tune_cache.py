@@ -83,3 +83,36 @@ def test_other_devices_and_formats_are_passed_over(so):
     assert _parse(so, old, BASE) is None
     for bad in (b"", b"no bar\n", b"|64 1 1 0 0\n", full.replace(b"|64", b"|x")):
         assert _parse(so, bad, BASE) is None
+
+
+CAND = r"""
+#include "pd_tune.h"
+extern "C" int candidates(int fp64, int lattice, int try_pairs, int pairs, int ring, int* out) {
+  int n = 0;
+  for (const pd::TuneChoice& t : pd::tune_candidates(fp64, lattice, try_pairs, pairs, ring)) {
+    int* o = out + 5 * n++;
+    o[0] = t.block; o[1] = t.split; o[2] = t.pairs; o[3] = t.ring; o[4] = t.automatic;
+  }
+  return n;
+}
+"""
+
+
+@pytest.mark.parametrize("fp64,lattice,try_pairs", [(1, 0, 1), (1, 0, 0), (0, 1, 0), (0, 0, 0)])
+def test_what_an_untuned_context_runs_is_timed_too(tmp_path, fp64, lattice, try_pairs):
+    cxx = shutil.which("g++") or shutil.which("c++")
+    if not cxx:
+        pytest.skip("no host C++ compiler")
+    (tmp_path / "c.cc").write_text(CAND)
+    subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I" + HDR, str(tmp_path / "c.cc"), "-o",
+                    str(tmp_path / "c.so")], check=True)
+    out = (ctypes.c_int * 500)()
+    n = ctypes.CDLL(str(tmp_path / "c.so")).candidates(fp64, lattice, try_pairs, 1, 0, out)
+    got = [tuple(out[5 * k:5 * k + 5]) for k in range(n)]
+    assert len(set(got)) == n
+    pairs = [1, 0] if try_pairs else [1]
+    assert [t for t in got if t[4]] == ([(256, 1, p, 0, 1) for p in pairs] if fp64 or lattice else [])
+    splits = [1] if lattice else [1, 2, 4]
+    rings = [0, 1, 2, 3] if lattice else [0]
+    assert {t[:4] for t in got if not t[4]} == {(b, s, p, r) for b in (64, 128, 256, 512) for s in splits
+                                                if (b // 32) % s == 0 for p in pairs for r in rings}
