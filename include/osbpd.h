@@ -204,9 +204,17 @@ typedef enum {
                               0 (default) = one word.  Decisions stay exact either way (the same
                               rounding band covers both).  May be set at any time; pd_get_option
                               reports 1 only while the built layout is the lattice one. */
-  PD_OPT_DEVICE_LIMIT = 14 /* testing the failure path: device bytes (pd_get_info) above which the
+  PD_OPT_DEVICE_LIMIT = 14, /* testing the failure path: device bytes (pd_get_info) above which the
                               context's allocations fail as if the device had no memory left.
                               Default 0: no limit of its own. */
+  PD_OPT_RESIDENT = 15     /* 1 (default) = the steps of small bodies in one cooperative launch per call
+                              (PD_OPT_GRAPH_CHUNK); 0 = the pass kernels, in their automatic shapes.
+                              Results are bitwise the same.  A resident launch wants the whole GPU, so
+                              contexts that step at the same time on streams of their own take turns:
+                              up to three are faster with it, from four bodies of about 100 x 100
+                              particles or more 0 is (up to 1.7 times).  pd_get_option reports whether the last
+                              pd_step ran in a resident launch (before the first one of a build:
+                              the setting). */
 } pd_option;
 
 /* Solvers (PD_OPT_SOLVER).

@@ -29,6 +29,7 @@ PD_OPT_LATTICE = 11
 PD_OPT_LAT_STAGE = 12
 PD_OPT_SHADOW_LO = 13
 PD_OPT_DEVICE_LIMIT = 14
+PD_OPT_RESIDENT = 15
 PD_W_ONE, PD_W_INV = 0, 1
 PD_SOLVER_EXPLICIT, PD_SOLVER_ADR = 0, 1
 PD_K_PASS1, PD_K_PASS2, PD_K_PASS1B = 0, 1, 2

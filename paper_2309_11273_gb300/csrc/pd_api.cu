@@ -81,6 +81,7 @@ void free_build(pd_ctx* c) {
   c->adr_first = nullptr;
   c->bar = nullptr;
   c->bar_base = 0;
+  c->last_resident = -1;
   c->lost = false;
   c->adr_restart = true;
   c->diag_theta = nullptr;
@@ -642,6 +643,9 @@ pd_status pd_set_option(pd_ctx* c, int32_t option, int64_t value) {
       if (value < 0) return fail(PD_ERR_ARG, "PD_OPT_DEVICE_LIMIT must be >= 0");
       c->device_limit = value;
       break;
+    case PD_OPT_RESIDENT:
+      c->resident = value != 0;
+      break;
     case PD_OPT_PAIRS:
       // A failure check of the pair form marks slices whose bS its next pass 1b recomputes; the
       // other form never reads those marks, so a switch recomputes every bS before the next step.
@@ -681,6 +685,7 @@ pd_status pd_get_option(pd_ctx* c, int32_t option, int64_t* value) {
     case PD_OPT_LAT_STAGE: *value = c->lat_stage; break;
     case PD_OPT_SHADOW_LO: *value = c->built ? (c->shadow_lo ? 1 : 0) : c->shadow_lo_opt; break;
     case PD_OPT_DEVICE_LIMIT: *value = c->device_limit; break;
+    case PD_OPT_RESIDENT: *value = c->last_resident >= 0 ? c->last_resident : c->resident; break;
     default: return fail(PD_ERR_ARG, "unknown option");
   }
   return PD_OK;
@@ -941,6 +946,7 @@ pd_status pd_autotune(pd_ctx* c, int32_t trial_steps, int32_t* block_out, int32_
   problem.bond_cache = c->bond_cache;
   problem.stage = c->stage;
   problem.validate = c->validate;
+  problem.resident = c->resident;
   problem.device = prop.name;
   const std::string key = tune_key(problem);
   const char* cache = std::getenv("PD_AUTOTUNE_CACHE");

@@ -264,6 +264,8 @@ struct pd_ctx {
   int sms = 0;                  // SMs of the device; 0: no cooperative launch (the resident step kernel is off)
   unsigned* bar = nullptr;      // resident step kernel: grid barrier (arrivals, abort)
   unsigned bar_base = 0;        // ... arrivals enqueued so far
+  int resident = 1;             // PD_OPT_RESIDENT
+  int last_resident = -1;       // the last pd_step of the build ran in a resident launch (-1: none yet)
   bool lost = false;            // a resident launch gave up half way and was reported: there is no state to read or step
   int graph_chunk = 100;
   int profile = 0;

@@ -309,7 +309,7 @@ cudaError_t launch_split(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, un
 
 ResidentPlan resident_plan(const pd_ctx* c) {
   ResidentPlan p;
-  if (!c->auto_map || c->precision != PD_FP64 || c->kin != PD_LINEARIZED || !c->bond_cache || !c->pairs || !c->pairs_ok ||
+  if (!c->resident || !c->auto_map || c->precision != PD_FP64 || c->kin != PD_LINEARIZED || !c->bond_cache || !c->pairs || !c->pairs_ok ||
       c->solver != PD_SOLVER_EXPLICIT || c->profile || c->sms <= 0)
     return p;
   // Warps per slice: four while that leaves an SM at most 16 warps (128 registers each), two up to 20, in 2D

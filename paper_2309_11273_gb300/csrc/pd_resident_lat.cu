@@ -558,7 +558,7 @@ pd_status upload_resident_tables(int device) { return upload_lattice_constants(d
 
 ResidentPlan resident_lat_plan(const pd_ctx* c) {
   ResidentPlan p;
-  if (!c->auto_map || c->precision != PD_MIXED || !c->lattice || c->validate || c->profile ||
+  if (!c->resident || !c->auto_map || c->precision != PD_MIXED || !c->lattice || c->validate || c->profile ||
       c->solver != PD_SOLVER_EXPLICIT || c->sms <= 0)
     return p;
   const int64_t warps = (c->nslices + c->sms - 1) / c->sms;  // per block, one block per SM

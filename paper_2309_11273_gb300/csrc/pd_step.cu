@@ -3437,10 +3437,12 @@ pd_status run_steps(pd_ctx* c, int64_t nsteps) {
       c->steps += n;
     }
     if (left == 0) {
+      c->last_resident = 1;
       c->check_pending = true;
       return PD_OK;  // the kernel has marked a non-finite state
     }
   }
+  c->last_resident = 0;
   st = launch_set_step(c, c->steps - 1);
   if (st != PD_OK) return st;
   if (c->skip_next_check) {

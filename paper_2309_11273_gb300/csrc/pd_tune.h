@@ -46,7 +46,7 @@ inline std::vector<TuneChoice> tune_candidates(bool fp64, bool lattice, bool try
 struct TuneProblem {
   long long n = 0, bonds = 0, entries = 0;
   int dim = 0, precision = 0, bodies = 0, kinematics = 0, solver = 0, influence = 0;
-  int lattice = 0, shadow_lo = 0, bond_cache = 0, stage = 0, validate = 0;
+  int lattice = 0, shadow_lo = 0, bond_cache = 0, stage = 0, validate = 0, resident = 0;
   std::string device;
 };
 
@@ -54,9 +54,9 @@ inline std::string tune_key(const TuneProblem& p) {
   char s[384];
   std::snprintf(s, sizeof(s),
                 "osbpd-2 n=%lld bonds=%lld entries=%lld dim=%d prec=%d bodies=%d kin=%d solver=%d infl=%d lattice=%d lo=%d "
-                "cache=%d stage=%d validate=%d dev=",
+                "cache=%d stage=%d validate=%d resident=%d dev=",
                 p.n, p.bonds, p.entries, p.dim, p.precision, p.bodies, p.kinematics, p.solver, p.influence, p.lattice,
-                p.shadow_lo, p.bond_cache, p.stage, p.validate);
+                p.shadow_lo, p.bond_cache, p.stage, p.validate, p.resident);
   std::string key = std::string(s) + p.device;
   for (char& c : key)
     if (c == '\n' || c == '|') c = ' ';

@@ -260,3 +260,84 @@ def test_a_state_set_before_the_timeout_is_read_steps_all_the_same():
     ref.step(20)
     for x, y in zip(sim.state(), ref.state()):
         assert np.array_equal(x, y)
+
+
+def _last_path(sim, steps=2):
+    sim.step(steps)
+    return sim.get_option(B.PD_OPT_RESIDENT)
+
+
+# which bodies run resident on the 152 SMs of a GB300: both sides of every limit of the plans (24, 20 and 16 warps per SM)
+@pytest.mark.parametrize("nx,ny,want", [(5, 4, 1), (139, 140, 1), (221, 220, 1), (341, 340, 1), (350, 340, 0)])
+def test_plates_take_the_kernel_that_the_plan_names(nx, ny, want):
+    for kw in ({}, {"precision": PD_MIXED}, {"precision": PD_MIXED, "kinematics": PD_NONLINEAR}):
+        sim = Simulation(_plate(nx, ny), **kw)
+        assert sim.get_option(B.PD_OPT_RESIDENT) == 1  # the setting, before the first step
+        assert _last_path(sim) == want, kw
+        assert _last_path(_pass_kernels(sim)) == 0
+        sim.close()
+
+
+@pytest.mark.parametrize("shape,fp64,mixed", [((9, 7, 5), 1, 1), ((40, 38, 32), 1, 1), ((40, 38, 33), 0, 1), ((64, 45, 40), 0, 1),
+                                              ((64, 48, 40), 0, 0)])
+def test_blocks_take_the_kernel_that_the_plan_names(shape, fp64, mixed):
+    for kw, want in (({}, fp64), ({"precision": PD_MIXED}, mixed), ({"kinematics": PD_NONLINEAR}, 0),
+                     ({"precision": PD_MIXED, "kinematics": PD_NONLINEAR}, mixed)):
+        sim = Simulation(W.notched_block(*shape), **kw)
+        assert _last_path(sim) == want, kw
+        sim.close()
+
+
+@pytest.mark.parametrize("precision", [0, PD_MIXED])
+def test_the_resident_option(precision):
+    ref = Simulation(_plate(90, 60), precision=precision)
+    assert _last_path(ref, 40) == 1
+    sim = Simulation(_plate(90, 60), precision=precision)
+    sim.set_option(B.PD_OPT_RESIDENT, 0)
+    assert sim.get_option(B.PD_OPT_RESIDENT) == 0
+    assert _last_path(sim, 20) == 0
+    sim.set_option(B.PD_OPT_RESIDENT, 1)
+    assert _last_path(sim, 20) == 1
+    for x, y in zip(list(sim.state()) + [sim.damage()], list(ref.state()) + [ref.damage()]):
+        assert np.array_equal(x, y)
+    for opt in (B.PD_OPT_PROFILE, B.PD_OPT_SOLVER):
+        sim.set_option(opt, 1)
+        assert _last_path(sim) == 0
+        sim.set_option(opt, 0)
+        assert _last_path(sim) == 1
+
+
+@pytest.mark.parametrize("precision", [0, PD_MIXED])
+def test_a_callers_capture_takes_the_pass_kernels(precision):
+    import torch
+    stream = torch.cuda.Stream()
+    ref = Simulation(_plate(90, 60), precision=precision)
+    ref.step(10)
+    sim = Simulation(_plate(90, 60), precision=precision, stream=stream.cuda_stream)
+    assert _last_path(sim, 2) == 1
+    sim.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+        sim.step(8)
+    assert sim.get_option(B.PD_OPT_RESIDENT) == 0
+    with torch.cuda.stream(stream):
+        g.replay()
+    for x, y in zip(list(sim.state()) + [sim.damage()], list(ref.state()) + [ref.damage()]):
+        assert np.array_equal(x, y)
+
+
+@pytest.mark.parametrize("offset", [1, 511])
+def test_a_read_into_arrays_that_share_their_pages(offset):
+    """pd_get_state brings the pages of large output arrays in while the GPU still steps: what else lies on the first
+    and last page stays as it was."""
+    w = W.notched_block(60, 60, 60)
+    ref = Simulation(w, precision=PD_MIXED)
+    ref.step(40)
+    want = ref.state()[0]
+    sim = Simulation(w, precision=PD_MIXED)
+    buf = np.full(3 * w.n + 1024, -7.5)
+    u = buf[offset:offset + 3 * w.n].reshape(3, w.n)
+    sim.step(40)
+    B.pd_get_state(sim.h, 3, w.n, u=u, v=False, theta=False)
+    assert np.array_equal(u, want)
+    assert (buf[:offset] == -7.5).all() and (buf[offset + 3 * w.n:] == -7.5).all()

@@ -11,7 +11,7 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 HDR = os.path.join(ROOT, "paper_2309_11273_gb300", "csrc")
 FIELDS = ["n", "bonds", "entries", "dim", "precision", "bodies", "kinematics", "solver", "influence", "lattice", "shadow_lo",
-          "bond_cache", "stage", "validate"]
+          "bond_cache", "stage", "validate", "resident"]
 
 SRC = r"""
 #include "pd_tune.h"
@@ -19,7 +19,7 @@ static pd::TuneProblem problem(const long long* v, const char* dev) {
   pd::TuneProblem p;
   p.n = v[0]; p.bonds = v[1]; p.entries = v[2]; p.dim = v[3]; p.precision = v[4]; p.bodies = v[5]; p.kinematics = v[6];
   p.solver = v[7]; p.influence = v[8]; p.lattice = v[9]; p.shadow_lo = v[10]; p.bond_cache = v[11]; p.stage = v[12];
-  p.validate = v[13]; p.device = dev;
+  p.validate = v[13]; p.resident = v[14]; p.device = dev;
   return p;
 }
 extern "C" void line_of(const long long* v, const char* dev, const int* t, char* out) {
@@ -47,18 +47,18 @@ def so(tmp_path_factory):
     return ctypes.CDLL(str(d / "t.so"))
 
 
-BASE = [1600, 41000, 45000, 2, 0, 1, 0, 0, 0, 0, 0, 1, 1, 0]
+BASE = [1600, 41000, 45000, 2, 0, 1, 0, 0, 0, 0, 0, 1, 1, 0, 1]
 
 
 def _line(so, v, t, dev=b"NVIDIA GB300"):
     out = ctypes.create_string_buffer(1024)
-    so.line_of((ctypes.c_longlong * 14)(*v), dev, (ctypes.c_int * 5)(*t), out)
+    so.line_of((ctypes.c_longlong * 15)(*v), dev, (ctypes.c_int * 5)(*t), out)
     return out.value
 
 
 def _parse(so, line, v, dev=b"NVIDIA GB300"):
     t = (ctypes.c_int * 5)(*([-9] * 5))
-    return list(t) if so.parse(line, (ctypes.c_longlong * 14)(*v), dev, t) else None
+    return list(t) if so.parse(line, (ctypes.c_longlong * 15)(*v), dev, t) else None
 
 
 @pytest.mark.parametrize("choice", [[256, 1, 1, 0, 1], [64, 2, 0, 3, 0]])
