@@ -459,7 +459,7 @@ __global__ void __launch_bounds__(512) k_pass1a_nlp(StepArgs a, const double4* _
     const int k = own + m;
     const bool mine = k < cnt;
     const int64_t e = t.base + t.lane + ((int64_t)k << 5);
-    double p = 0.0, yx = 0.0, yy = 0.0, yz = 0.0, xv = 0.0;
+    double p = 0.0, yx = 0.0, yy = 0.0, yz = 0.0, xv = 0.0, xl = 0.0;
     double4 c = make_double4(0.0, 0.0, 0.0, 0.0);
     int32_t te = 0;
     if (mine) {
@@ -467,6 +467,7 @@ __global__ void __launch_bounds__(512) k_pass1a_nlp(StepArgs a, const double4* _
       const double4 g = ta[(int64_t)k << 5];
       c = tc[(int64_t)k << 5];
       xv = tx[(int64_t)k << 5];
+      xl = g.w;
       const double4 uj = disp[j];
       te = tw[(int64_t)k << 5];
       const double hx = uj.x - ui.x, hy = uj.y - ui.y, hz = DIM == 3 ? uj.z - ui.z : 0.0;
@@ -492,7 +493,10 @@ __global__ void __launch_bounds__(512) k_pass1a_nlp(StepArgs a, const double4* _
         double yl2 = yx * yx + yy * yy;
         if (DIM == 3) yl2 = fma(yz, yz, yl2);
         ry = rsqrt(yl2);
-        z = tt / fma(yl2 * ry, c.y, 1.0);
+        // (two particles at one place, tabled with 1/|xi| = 0: z is e itself, and so it is in the stored factors;
+        // selected on the integer pipe)
+        const bool apart = __double2hiint(c.y) != 0;
+        z = (apart ? tt : p) / fma(yl2 * ry, apart ? c.y : 1.0, apart ? 1.0 : xl);
       }
       const double mx = ry * yx, my = ry * yy, mz = ry * yz;  // M = Y / |Y| (Eq 1.13), -M at j
       const double ev = c.w * z, tij = xv * z;                // Eq 1.14's and Eq 1.6's terms of entry (i, j)
@@ -579,7 +583,9 @@ __global__ void __launch_bounds__(512) k_pass2_nlp(StepArgs a, const double4* __
 
 // Per-slot tables of the nonlinear pair form, |xi| and |xi|^2 as in k_bond_tables_nl and the threshold
 // with the rounding of the single pass (s0 (2 + s0) times |xi| |xi|): bC = (1 / |xi|^2, 1 / |xi|,
-// s0 (2 + s0) |xi|^2, G (1/m_i + 1/m_j) V_j |xi|), bX = |xi| V_j, bX2 = |xi|^2 V_j.
+// s0 (2 + s0) |xi|^2, G (1/m_i + 1/m_j) V_j |xi|), bX = |xi| V_j, bX2 = |xi|^2 V_j.  Where 1 / |xi|^2 is no finite
+// number (two particles at one place) the bond takes the root whatever its length (t = inf or NaN) and the tables
+// are those of e instead of e / |xi|: bC = (inf, 0, s0 (2 + s0) |xi|^2, G (1/m_i + 1/m_j) V_j), bX2 = |xi| V_j.
 template <int DIM>
 __global__ void k_bond_tables_nlp(StepArgs a, double4* __restrict__ bC, double* __restrict__ bX,
                                   double* __restrict__ bX2) {
@@ -596,10 +602,11 @@ __global__ void k_bond_tables_nlp(StepArgs a, double4* __restrict__ bC, double* 
     double ex, ey, ez, d, q;
     bond_f64<DIM>(pi, pj, zero, zero, ex, ey, ez, d, q);
     const double xl = sqrt(q);
-    const bool bond = q > 0.0;
-    bC[e] = make_double4(bond ? 1.0 / q : 0.0, bond ? 1.0 / xl : 0.0, s0nl * (xl * xl), G * (mi + a.mu[j]) * pj.w * xl);
+    const bool apart = isfinite(1.0 / q);
+    const double g = G * (mi + a.mu[j]) * pj.w;
+    bC[e] = make_double4(1.0 / q, apart ? 1.0 / xl : 0.0, s0nl * (xl * xl), apart ? g * xl : g);
     bX[e] = xl * pj.w;
-    bX2[e] = q * pj.w;
+    bX2[e] = (apart ? q : xl) * pj.w;
   }
 }
 

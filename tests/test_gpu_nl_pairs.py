@@ -8,7 +8,8 @@ import numpy as np
 import pytest
 
 import oracle as O
-from paper_2309_11273_gb300 import PD_NONLINEAR, Simulation
+from paper_2309_11273_gb300 import PD_NONLINEAR, PDError, Simulation
+from paper_2309_11273_gb300._binding import PD_ERR_NUMERIC
 from paper_2309_11273_gb300 import workloads as W
 
 pytestmark = pytest.mark.gpu
@@ -48,3 +49,31 @@ def test_extension_series_and_its_range(dim, uniform, stretch):
     assert np.abs(v - ref.v).max() <= 1e-12 * np.abs(ref.v).max()
     assert np.abs(u - ref.u).max() <= 1e-12 * np.abs(ref.u).max()
     assert np.abs(theta - ref.theta).max() <= 1e-12 * np.abs(ref.theta).max()
+
+
+@pytest.mark.parametrize("uniform", [True, False])
+@pytest.mark.parametrize("dim", [2, 3])
+def test_two_particles_at_one_place(dim, uniform):
+    """A bond of no length: once its ends have moved apart its extension is |Y| and it pulls along Y, as the single
+    pass (PD_OPT_PAIRS 0), which tables no 1/|xi|, has it; at rest the state has no direction for it and the run is
+    reported as non-finite in both forms.  The same bars as above."""
+    rng = np.random.default_rng(5)
+    w = _body(dim, uniform, rng)
+    for k, j in ((3, 4), (40, 39), (100, 137)):  # in one slice and across two
+        w.x[k], w.y[k] = w.x[j], w.y[j]
+        if dim == 3:
+            w.z[k] = w.z[j]
+    w.u0 = rng.normal(0.0, 1e-6, (dim, w.n))
+    got = []
+    for pairs in (1, 0):
+        sim = Simulation(w, s0=0.0, kinematics=PD_NONLINEAR, pairs=pairs)
+        sim.step(1)
+        got.append(sim.state())
+        sim.set_state(np.zeros((dim, w.n)))
+        sim.step(1)
+        with pytest.raises(PDError) as e:
+            sim.sync()
+        assert e.value.status == PD_ERR_NUMERIC
+        sim.close()
+    for x, y in zip(*got):
+        assert np.abs(x - y).max() <= 1e-12 * np.abs(y).max()
