@@ -97,19 +97,21 @@ __device__ __forceinline__ void parts_across(double (&v)[NC]) {
 }
 
 // Eq 2.11 for a free particle with the force density f and the body force b (nullptr: none): v += (dt / rho)
-// (f + b), u += dt v, two or three FMAs per component (an FP64 instruction occupies its pipe for 64 cycles
-// per warp); the z components stay as they are in 2D.
+// (f + b), u += dt v, two FMAs per component and an addition for b (an FP64 instruction occupies its pipe for 64
+// cycles per warp); f + b is formed first, so that a particle in balance gets no rounding of dt f / rho.  The z
+// components stay as they are in 2D.
 template <int DIM>
 __device__ __forceinline__ void explicit_move(const BodyDev& bp, const double f[3], const double4* b, double4& u,
                                               double4& v) {
-  v.x = fma(bp.dt_rho, f[0], v.x);
-  v.y = fma(bp.dt_rho, f[1], v.y);
-  if (DIM == 3) v.z = fma(bp.dt_rho, f[2], v.z);
+  double g[3] = {f[0], f[1], f[2]};
   if (b) {
-    v.x = fma(bp.dt_rho, b->x, v.x);
-    v.y = fma(bp.dt_rho, b->y, v.y);
-    if (DIM == 3) v.z = fma(bp.dt_rho, b->z, v.z);
+    g[0] += b->x;
+    g[1] += b->y;
+    if (DIM == 3) g[2] += b->z;
   }
+  v.x = fma(bp.dt_rho, g[0], v.x);
+  v.y = fma(bp.dt_rho, g[1], v.y);
+  if (DIM == 3) v.z = fma(bp.dt_rho, g[2], v.z);
   u.x = fma(bp.dt, v.x, u.x);
   u.y = fma(bp.dt, v.y, u.y);
   if (DIM == 3) u.z = fma(bp.dt, v.z, u.z);
