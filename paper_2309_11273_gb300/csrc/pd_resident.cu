@@ -53,10 +53,11 @@ __global__ void __launch_bounds__(MAXT, 1) k_resident(StepArgs a, ResidentArgs r
   constexpr bool kKeep = MAXT <= 512;  // the particles' state in registers
   constexpr int U = MAXT <= 256 && !PAIR ? 8 : (kKeep ? 4 : 2);
   constexpr int H = P > U ? P / U : 1;
-  // Batches of the static streams fetched to L2 ahead: in 3D they do not stay there from step to step, and each
-  // batch waited for its indices and then its rows from memory (a 45,000-particle block 134.8 -> 124.4 us per
-  // iteration with 2, 129.9 with 4, 139.4 with 8, which push each other out).
-  constexpr int kAhead = PAIR && DIM == 3 ? 2 : 0;
+  // Batches of the static streams fetched to L2 ahead: the tables of a larger 3D body do not stay there from step to
+  // step, and each batch waited for its indices and then its rows from memory.  With four warps per slice the body
+  // (up to 19,456 particles) is small enough to stay.  us per step with 0 / 2 / 4 batches: two warps per slice, 28^3
+  // 74 / 70 / 73, 32^3 90 / 87 / 92, 36^3 120 / 107 / 114; four, 20^3 32.4 / 36.0 / 36.1, 24^3 43.9 / 46.9 / 47.4.
+  constexpr int kAhead = PAIR && DIM == 3 && SPLIT < 4 ? 2 : 0;
   // an earlier launch gave up and its error is not yet reported (one answer for the whole block)
   if (__syncthreads_or(ld_relaxed(r.grid.bar + 1) != 0u)) return;
   unsigned target = r.grid.base;
@@ -328,6 +329,9 @@ ResidentPlan resident_plan(const pd_ctx* c) {
   p.split = split;
   p.block = (int)warps * 32;
   p.grid = (unsigned)((ns * split + warps - 1) / warps);
+  // The pair form has fewer FP64 instructions and one barrier more (us per step without / with it: plates of 140^2,
+  // 536,000 bonds, 16.8 / 17.0, 160^2, 702,000, 19.2 / 18.7; blocks of 16^3, 394,000, 23.6 / 26.9, 18^3, 576,000,
+  // 33.5 / 31.8, 24^3, 1.44M, 48.3 / 42.6).
   p.pair = c->nbonds > 600000;
   return p;
 }
