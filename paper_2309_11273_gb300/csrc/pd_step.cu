@@ -2649,11 +2649,13 @@ cudaEvent_t take_event(pd_ctx* c) {
 // kSplit1a warps per slice in the pair forms' pass 1a, which sums nothing, so that its results do not
 // depend on the split (nonlinear: 1.405 -> 1.34 ms).
 constexpr int kAutoBlock64 = 64;
-// Split of the linearized tabled kernels (any split gives the same sums): two warps per slice, and in 3D
-// four, in 128-thread blocks, where two would end in a partial second wave (48^3 particles 272 -> 243 us
-// per step; one wave at 40^3 155 against 163, many at 1M particles 1766 against 1777).
+// Split of the linearized tabled kernels (any split gives the same sums): two warps per slice, and in 3D four, in
+// 128-thread blocks, between the sizes where two end in a partial second wave and those of many waves.  us per step
+// with 1 / 2 / 4: blocks of 42^3 (2,316 slices) 204 / 162 / 167, 44^3 233 / 223 / 213, 48^3 261 / 270 / 252, 56^3 442 /
+// 388 / 376, 60^3 (6,750) 495 / 444 / 444, 68^3 (9,826) 657 / 612 / 614, 80^3 1005 / 957 / 967, 100^3 1838 / 1787 / 1820;
+// plates of 400^2 98.5 / 89.9 / 94.7, 1000^2 406 / 414 / 470, 64 uneven plates 411 / 409 / 445.
 inline int auto_split64(const pd_ctx* c) {
-  return c->dim == 3 && c->nslices * 2 > (int64_t)c->sms * 32 && c->nslices <= 16000 ? 4 : 2;
+  return c->dim == 3 && c->nslices * 2 > (int64_t)c->sms * 32 && c->nslices <= 9000 ? 4 : 2;
 }
 constexpr int kSplit1aL = 2, kBlock1aL = 64;    // linearized
 constexpr int kSplit1aNL = 4, kBlock1aNL = 128;  // nonlinear
