@@ -291,11 +291,18 @@ cudaError_t launch(pd_ctx* c, StepArgs a, ResidentArgs r, unsigned grid, int blo
   return cudaLaunchCooperativeKernel(k, dim3(grid), dim3((unsigned)block), args, sm, c->stream);
 }
 
+// (Only the forms that resident_plan names: four warps per slice up to 512 threads, two and one from 288 on, one in
+// 2D only.)
 template <int DIM, int SPLIT>
 cudaError_t launch_form(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, unsigned grid, int block, bool pair) {
-  if (block > 512) return launch<DIM, SPLIT, true, 768>(c, a, r, grid, block);
+  if (block > 512) {
+    if constexpr (SPLIT < 4) return launch<DIM, SPLIT, true, 768>(c, a, r, grid, block);
+    return cudaErrorInvalidConfiguration;
+  }
   if (pair) return launch<DIM, SPLIT, true, 512>(c, a, r, grid, block);
-  return block > 256 ? launch<DIM, SPLIT, false, 512>(c, a, r, grid, block) : launch<DIM, SPLIT, false, 256>(c, a, r, grid, block);
+  if constexpr (SPLIT == 4)
+    if (block <= 256) return launch<DIM, SPLIT, false, 256>(c, a, r, grid, block);
+  return launch<DIM, SPLIT, false, 512>(c, a, r, grid, block);
 }
 
 template <int DIM>
@@ -303,7 +310,8 @@ cudaError_t launch_split(pd_ctx* c, const StepArgs& a, const ResidentArgs& r, un
                          bool pair) {
   if (split == 4) return launch_form<DIM, 4>(c, a, r, grid, block, pair);
   if (split == 2) return launch_form<DIM, 2>(c, a, r, grid, block, pair);
-  return launch_form<DIM, 1>(c, a, r, grid, block, pair);
+  if constexpr (DIM == 2) return launch_form<DIM, 1>(c, a, r, grid, block, pair);
+  return cudaErrorInvalidConfiguration;
 }
 
 }  // namespace
