@@ -322,14 +322,15 @@ ResidentPlan resident_plan(const pd_ctx* c) {
       c->solver != PD_SOLVER_EXPLICIT || c->profile || c->sms <= 0)
     return p;
   // Warps per slice: four while that leaves an SM at most 16 warps (128 registers each), two up to 20, in 2D
-  // one up to 24 (80 registers).  Beyond, the pass kernels are the faster ones (us per step, resident against
-  // pass kernels: plates of 250^2 32 / 41, 340^2 59 / 70; blocks of 34^3 112 / 115, with one warp per slice
-  // 40^3 163 / 155).
+  // one up to 24 (80 registers beyond 16), but not where two warps per slice of the pass kernels fill just one wave
+  // (tight_wave).  Elsewhere the pass kernels are the faster ones.  us per step, resident against pass kernels: plates
+  // of 262^2 33.8 / 37.1, 278^2 (2,416 slices) 37.1 / 40.8, 279^2 (2,433) 50.0 / 40.2, 295^2 (2,720) 52.5 / 43.9, 297^2
+  // 52.8 / 53.2, 340^2 59 / 65; blocks of 34^3 97 / 115, with one warp per slice 40^3 163 / 155.
   const int64_t ns = c->nslices, sms = c->sms;
   int split = 0;
   if (ns * 4 <= sms * 16) split = 4;
   else if (ns * 2 <= sms * 20) split = 2;
-  else if (ns <= sms * 24 && c->dim == 2) split = 1;
+  else if (ns <= sms * 24 && c->dim == 2 && !tight_wave(c)) split = 1;
   if (!split) return p;
   // One block per SM; a slice's warps share a block (parts_across).
   int64_t warps = (ns * split + sms - 1) / sms;

@@ -53,6 +53,7 @@ __device__ __forceinline__ void load_slots(const SliceIdx& t, const int32_t* __r
 }
 
 // ------------------------------------------------------------------------------------ FP64 path
+constexpr int kTightBlock = 128;  // largest block of the 56-register instances (tight)
 constexpr int kU64 = 2;  // (the recompute and single-pass nonlinear kernels)
 constexpr int kU32 = 4;
 
@@ -730,8 +731,8 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
 // which recomputes its bS.  Each lane walks its own owned entries: a common slot for the warp runs over
 // the union of the lanes' ranges, 1.08 times as many on the 200 x 100 x 50 block and 1.4 times on 60 x 30
 // x 25 (1.87 -> 1.81 ms and 225 -> 207 us per step).
-template <int DIM, int SPLIT>
-__global__ void __launch_bounds__(512) k_pass1a_f64p(StepArgs a, const double4* __restrict__ disp) {
+template <int DIM, int SPLIT, bool TIGHT>
+__global__ void __launch_bounds__(TIGHT ? kTightBlock : 512, TIGHT ? 9 : 0) k_pass1a_f64p(StepArgs a, const double4* __restrict__ disp) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (!t.active) return;  // whole warps; no block-wide barrier below
   const int b = a.body ? a.body[t.i] : 0;
@@ -789,8 +790,8 @@ __global__ void __launch_bounds__(512) k_pass1a_f64p(StepArgs a, const double4* 
 // UV: every body has one particle volume, so V_j = V_i for every bond (same body) and the sum takes
 // the lane's own V_i: the same FMAs on the same values, without the neighbour index stream and the
 // gather of V_j.
-template <int DIM, int SPLIT, bool UV, bool SERIAL>
-__global__ void __launch_bounds__(512) k_pass1b_f64p(StepArgs a, const double4* __restrict__ disp, int write_theta) {
+template <int DIM, int SPLIT, bool UV, bool SERIAL, bool TIGHT>
+__global__ void __launch_bounds__(TIGHT ? kTightBlock : 512, TIGHT ? 9 : 0) k_pass1b_f64p(StepArgs a, const double4* __restrict__ disp, int write_theta) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   if (write_theta && blockIdx.x == 0 && threadIdx.x == 0) *a.d_step += 1;
   constexpr int P = SERIAL ? 1 : 4 / SPLIT;
@@ -1040,8 +1041,8 @@ __global__ void k_check_u32(int64_t n_pad, const double4* __restrict__ disp, flo
   cu[i] = make_float4(__double2float_rn(u.x), __double2float_rn(u.y), __double2float_rn(u.z), 0.0f);
 }
 
-template <int DIM, int SPLIT, bool SERIAL>
-__global__ void __launch_bounds__(512) k_pass2_f64t(StepArgs a, const double4* __restrict__ disp,
+template <int DIM, int SPLIT, bool SERIAL, bool TIGHT>
+__global__ void __launch_bounds__(TIGHT ? kTightBlock : 512, TIGHT ? 9 : 0) k_pass2_f64t(StepArgs a, const double4* __restrict__ disp,
                                                      double4* __restrict__ disp_out) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
   constexpr int P = SERIAL ? 1 : 4 / SPLIT;
@@ -2664,6 +2665,15 @@ inline unsigned slice_grid(const pd_ctx* c, int split, int block) {
   return (unsigned)((c->nslices * 32 * (int64_t)split + block - 1) / block);
 }
 
+// The linearized tabled kernels take up to 64 registers, 32 warps per SM.  Two warps per slice of a plate of 32 to 36
+// warps per SM would then leave a last wave nearly empty; TIGHT holds the kernels to 56 registers (9 blocks of 4
+// warps, or 18 of 2), one wave: 80,802 particles 49.3 -> 42.0 us per step, 290^2 52.5 -> 44.9.  Elsewhere the 64
+// registers are the faster choice.
+template <int DIM, int SPLIT>
+inline bool tight(const pd_ctx* c, int block) {
+  return DIM == 2 && SPLIT == 2 && block <= kTightBlock && kTightBlock % block == 0 && tight_wave(c);
+}
+
 template <int DIM, int SPLIT>
 void launch_pass1a_nlp(pd_ctx* c, const StepArgs& a, unsigned grid, int block) {
   if (c->vol_uniform)
@@ -2675,6 +2685,7 @@ void launch_pass1a_nlp(pd_ctx* c, const StepArgs& a, unsigned grid, int block) {
 template <int DIM, int SPLIT>
 void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, int block, size_t sm) {
   const bool serial = a.adr != 0;  // the relaxation solver's sums: parts_sum
+  const bool one_wave = !serial && tight<DIM, SPLIT>(c, block);
   if (c->kin == PD_NONLINEAR && a.bA && a.own0 && !write_theta) {
     if (a.check) k_check_nlp<DIM, SPLIT><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
   } else if (c->kin == PD_NONLINEAR && a.bA && a.own0) {
@@ -2702,23 +2713,31 @@ void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, 
       k_check_f64p<DIM, SPLIT, false><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur], nullptr, nullptr);
     }
   } else if (c->precision == PD_FP64 && a.bA && a.own0) {
-    if (c->auto_map)
-      k_pass1a_f64p<DIM, kSplit1aL>
+    if (c->auto_map && tight<DIM, kSplit1aL>(c, kBlock1aL))
+      k_pass1a_f64p<DIM, kSplit1aL, DIM == 2>
           <<<slice_grid(c, kSplit1aL, kBlock1aL), kBlock1aL, 0, c->stream>>>(a, c->disp[c->cur]);
+    else if (c->auto_map)
+      k_pass1a_f64p<DIM, kSplit1aL, false>
+          <<<slice_grid(c, kSplit1aL, kBlock1aL), kBlock1aL, 0, c->stream>>>(a, c->disp[c->cur]);
+    else if (one_wave)
+      k_pass1a_f64p<DIM, SPLIT, DIM == 2 && SPLIT == 2><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
     else
-      k_pass1a_f64p<DIM, SPLIT><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
+      k_pass1a_f64p<DIM, SPLIT, false><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
     if (c->profile) {
       c->times.mid = take_event(c);
       cudaEventRecord(c->times.mid, c->stream);
     }
     if (serial && c->vol_uniform)
-      k_pass1b_f64p<DIM, SPLIT, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1b_f64p<DIM, SPLIT, true, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else if (serial)
-      k_pass1b_f64p<DIM, SPLIT, false, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
-    else if (c->vol_uniform)
-      k_pass1b_f64p<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1b_f64p<DIM, SPLIT, false, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    else if (c->vol_uniform)  // (within the tight wave's registers as it is)
+      k_pass1b_f64p<DIM, SPLIT, true, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+    else if (one_wave)
+      k_pass1b_f64p<DIM, SPLIT, false, false, DIM == 2 && SPLIT == 2>
+          <<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else
-      k_pass1b_f64p<DIM, SPLIT, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
+      k_pass1b_f64p<DIM, SPLIT, false, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
   } else if (c->precision == PD_FP64 && a.bA) {
     if (write_theta && serial)
       k_pass1_f64t<DIM, SPLIT, true, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
@@ -2742,9 +2761,12 @@ void launch_pass2(pd_ctx* c, const StepArgs& a, unsigned grid, int block, size_t
   else if (c->kin == PD_NONLINEAR)
     k_pass2_nl<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64 && a.bA && a.adr)
-    k_pass2_f64t<DIM, SPLIT, true><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
+    k_pass2_f64t<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
+  else if (c->precision == PD_FP64 && a.bA && tight<DIM, SPLIT>(c, block))
+    k_pass2_f64t<DIM, SPLIT, false, DIM == 2 && SPLIT == 2>
+        <<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64 && a.bA)
-    k_pass2_f64t<DIM, SPLIT, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
+    k_pass2_f64t<DIM, SPLIT, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64)
     k_pass2_f64<DIM, SPLIT><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else
