@@ -439,7 +439,9 @@ __device__ __forceinline__ void nl_series(double t, double& ext, double& inv) {
 // that does not depend on the displacement tabled (bC, bX2: 80 bytes read and 80 written per pair, 0.4
 // of the pipe's time at the HBM rate) and the failure threshold compared on the integer pipe.  Each lane
 // walks its own owned entries (own0 up to its family size): a common slot for the warp would run over
-// the union of the lanes' ranges, 1.16 times as many on a 101 x 50 x 49 block and 1.4 times on 60 x 30 x 25.
+// the union of the lanes' ranges, 1.16 times as many on a 101 x 50 x 49 block and 1.4 times on 60 x 30 x 25
+// (1574 against 1347 us per step on the former; on scattered points too, 64^3 1828 against 1503: unlike the
+// linearized form's, this pass is bound by its arithmetic).
 // UV: every body has one particle volume, so both entries' terms are the same products, formed once.
 template <int DIM, int SPLIT, bool UV>
 __global__ void __launch_bounds__(512) k_pass1a_nlp(StepArgs a, const double4* __restrict__ disp) {
@@ -721,6 +723,23 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
   }
 }
 
+// How a warp's lanes walk their owned entries (slots own .. cnt - 1 of each) in k_pass1a_f64p: each lane its own
+// first, second, ... entry, or all of them the same slot, over the union of their ranges (false).  The former takes
+// fewer turns: the union has 1.08 times as many on the 200 x 100 x 50 block, 1.4 times on 60 x 30 x 25.  But a turn
+// reads up to one line per different first slot, one on most of a lattice, a dozen or more on scattered points,
+// whose streams fall apart into single sectors.  So the union is taken where it costs fewer than 1/48 more turns per
+// different first slot.  us per step, each lane for itself / by this rule (factors of 20 to 90 tried): scattered
+// cubes of 40^3 182 / 165, 44^3 283 / 247, 64^3 701 / 610, 80^3 1285 / 1099; blocks of 40^3 146 / 146 (a factor of 40:
+// 151, 20: 158), 64^3 527 / 527, the 1M-particle block 1763 / 1762, 64 uneven plates 410 / 410.
+constexpr int kOwnTurns = 48;
+__device__ __forceinline__ bool own_each(int own, int cnt) {
+  const unsigned same = __match_any_sync(kFull, own);
+  const int starts = __popc(__ballot_sync(kFull, (int)(threadIdx.x & 31) == __ffs(same) - 1));
+  const int turns = __reduce_max_sync(kFull, (unsigned)(cnt - own));
+  const int all = (int)__reduce_max_sync(kFull, (unsigned)cnt) - (int)__reduce_min_sync(kFull, (unsigned)own);
+  return kOwnTurns * all >= (kOwnTurns + starts) * turns;
+}
+
 // Pair form of the tabled FP64 pass 1, used when the build paired the two entries of every bond.
 // ξ·(u_j − u_i) is the same number at both ends (ξ and u_j − u_i both change sign, exactly), so
 // pass 1a forms it once, at the owned entry, applies the failure check to the pair (clearing both
@@ -728,9 +747,7 @@ __global__ void __launch_bounds__(512) k_pass1_f64t(StepArgs a, const double4* _
 // intact entries in slot order.  Per directed bond that is 3 FP64 instructions in 1a and 1 in 1b
 // against 7 in the single pass, with the same values: d, the decisions, bd and theta are bitwise
 // those of k_pass1_f64t.  A slice in which a bond broke (at either end) is marked for pass 1b,
-// which recomputes its bS.  Each lane walks its own owned entries: a common slot for the warp runs over
-// the union of the lanes' ranges, 1.08 times as many on the 200 x 100 x 50 block and 1.4 times on 60 x 30
-// x 25 (1.87 -> 1.81 ms and 225 -> 207 us per step).
+// which recomputes its bS.
 template <int DIM, int SPLIT, bool TIGHT>
 __global__ void __launch_bounds__(TIGHT ? kTightBlock : 512, TIGHT ? 9 : 0) k_pass1a_f64p(StepArgs a, const double4* __restrict__ disp) {
   const SliceIdx t = slice_index<SPLIT>(a.n_pad, a.slice_ptr);
@@ -738,53 +755,58 @@ __global__ void __launch_bounds__(TIGHT ? kTightBlock : 512, TIGHT ? 9 : 0) k_pa
   const int b = a.body ? a.body[t.i] : 0;
   const bool can_break = a.bp[b].breaks != 0;
   const int own = a.own0[t.i], cnt = a.cnt[t.i];
-  const int nown = __reduce_max_sync(kFull, (unsigned)(cnt - own));
   const double4 ui = disp[t.i];
   uint32_t* bw = a.bits + (t.base >> 5);
   const int32_t* __restrict__ cl = a.col + t.base + t.lane;
   const int32_t* __restrict__ tw = a.twin + t.base + t.lane;
   const int64_t e0 = t.base + t.lane;
   double* td = a.bd;
-  // the owned-entry streams (index, table row, twin entry) of the next entry are loaded while the
-  // current entry's displacement gather and arithmetic run; each lane walks its own owned entries (a
-  // common slot for the warp would run over the union of the lanes' ranges)
-  bool mn = own + t.sub < cnt;
-  int32_t jn = (int32_t)t.i, ten = 0;
-  double4 gn = make_double4(0.0, 0.0, 0.0, 0.0);
-  if (mn) {
-    const int64_t kn = (int64_t)(own + t.sub) << 5;
-    jn = cl[kn];
-    gn = slot_row<DIM>(a.bA, a.ne, e0 + kn);
-    ten = tw[kn];
-  }
-  for (int m = t.sub; m < nown; m += SPLIT) {
-    const int k = own + m;
-    const bool mine = mn;
-    const int32_t j = jn, te = ten;
-    const double4 g = gn;
-    const double4 uj = disp[j];
-    mn = k + SPLIT < cnt;
+  auto walk = [&](auto each) {
+    constexpr bool EACH = decltype(each)::value;
+    const int lo = EACH ? own : (int)__reduce_min_sync(kFull, (unsigned)own);
+    const int n = __reduce_max_sync(kFull, (unsigned)(cnt - lo));
+    // the owned-entry streams (index, table row, twin entry) of the next entry are loaded while the
+    // current entry's displacement gather and arithmetic run
+    bool mn = (EACH || lo + t.sub >= own) && lo + t.sub < cnt;
+    int32_t jn = (int32_t)t.i, ten = 0;
+    double4 gn = make_double4(0.0, 0.0, 0.0, 0.0);
     if (mn) {
-      const int64_t kn = (int64_t)(k + SPLIT) << 5;
+      const int64_t kn = (int64_t)(lo + t.sub) << 5;
       jn = cl[kn];
       gn = slot_row<DIM>(a.bA, a.ne, e0 + kn);
       ten = tw[kn];
     }
-    const int64_t e = t.base + t.lane + ((int64_t)k << 5);
-    double d = g.x * (uj.x - ui.x) + g.y * (uj.y - ui.y);
-    if (DIM == 3) d = fma(g.z, uj.z - ui.z, d);
-    if (mine) {
-      td[e] = d;
-      td[te] = d;
-      // an owned bit changes only here
-      if (a.check && can_break && ((bw[k] >> t.lane) & 1u) && pd_ge_threshold(d, g.w)) {  // d >= s0 |xi|^2
-        atomicAnd(&bw[k], ~(1u << t.lane));
-        atomicAnd(a.bits + (te >> 5), ~(1u << (te & 31)));
-        a.dirty[t.i >> 5] = 1;
-        a.dirty[j >> 5] = 1;
+    for (int m = t.sub; m < n; m += SPLIT) {
+      const int k = lo + m;
+      const bool mine = mn;
+      const int32_t j = jn, te = ten;
+      const double4 g = gn;
+      const double4 uj = disp[j];
+      mn = (EACH || k + SPLIT >= own) && k + SPLIT < cnt;
+      if (mn) {
+        const int64_t kn = (int64_t)(k + SPLIT) << 5;
+        jn = cl[kn];
+        gn = slot_row<DIM>(a.bA, a.ne, e0 + kn);
+        ten = tw[kn];
+      }
+      const int64_t e = t.base + t.lane + ((int64_t)k << 5);
+      double d = g.x * (uj.x - ui.x) + g.y * (uj.y - ui.y);
+      if (DIM == 3) d = fma(g.z, uj.z - ui.z, d);
+      if (mine) {
+        td[e] = d;
+        td[te] = d;
+        // an owned bit changes only here
+        if (a.check && can_break && ((bw[k] >> t.lane) & 1u) && pd_ge_threshold(d, g.w)) {  // d >= s0 |xi|^2
+          atomicAnd(&bw[k], ~(1u << t.lane));
+          atomicAnd(a.bits + (te >> 5), ~(1u << (te & 31)));
+          a.dirty[t.i >> 5] = 1;
+          a.dirty[j >> 5] = 1;
+        }
       }
     }
-  }
+  };
+  if (own_each(own, cnt)) walk(std::true_type{});
+  else walk(std::false_type{});
 }
 
 // UV: every body has one particle volume, so V_j = V_i for every bond (same body) and the sum takes
