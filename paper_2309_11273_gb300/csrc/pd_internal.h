@@ -339,9 +339,10 @@ struct ResidentPlan {
   bool pair = false;  // pass 1 in its pair form
 };
 ResidentPlan resident_plan(const pd_ctx* c);
-// Linearized FP64 plates whose slices, at two warps each, are 32 to 36 warps per SM (the 56-register pass kernels).
-inline bool tight_wave(const pd_ctx* c) {
-  return c->dim == 2 && c->nslices * 2 > (int64_t)c->sms * 32 && c->nslices * 2 <= (int64_t)c->sms * 36;
+// Linearized FP64 plates whose slices, at `split` warps each, are 32 to 36 warps per SM (the 56-register pass kernels).
+inline bool tight_wave(const pd_ctx* c, int split) {
+  const int64_t warps = c->nslices * split;
+  return c->dim == 2 && warps > (int64_t)c->sms * 32 && warps <= (int64_t)c->sms * 36;
 }
 pd_status run_resident(pd_ctx* c, const StepArgs& a, const ResidentPlan& p, int64_t nsteps, bool check0, bool* done);
 pd_status upload_resident_tables(int device);  // its copy of the direction tables, at the build

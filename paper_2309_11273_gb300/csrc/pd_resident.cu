@@ -330,7 +330,7 @@ ResidentPlan resident_plan(const pd_ctx* c) {
   int split = 0;
   if (ns * 4 <= sms * 16) split = 4;
   else if (ns * 2 <= sms * 20) split = 2;
-  else if (ns <= sms * 24 && c->dim == 2 && !tight_wave(c)) split = 1;
+  else if (ns <= sms * 24 && c->dim == 2 && !tight_wave(c, 2)) split = 1;
   if (!split) return p;
   // One block per SM; a slice's warps share a block (parts_across).
   int64_t warps = (ns * split + sms - 1) / sms;

@@ -2687,13 +2687,13 @@ inline unsigned slice_grid(const pd_ctx* c, int split, int block) {
   return (unsigned)((c->nslices * 32 * (int64_t)split + block - 1) / block);
 }
 
-// The linearized tabled kernels take up to 64 registers, 32 warps per SM.  Two warps per slice of a plate of 32 to 36
-// warps per SM would then leave a last wave nearly empty; TIGHT holds the kernels to 56 registers (9 blocks of 4
-// warps, or 18 of 2), one wave: 80,802 particles 49.3 -> 42.0 us per step, 290^2 52.5 -> 44.9.  Elsewhere the 64
-// registers are the faster choice.
+// The linearized tabled kernels take up to 64 registers, 32 warps per SM.  One or two warps per slice of a plate of 32
+// to 36 warps per SM would then leave a last wave nearly empty; TIGHT holds the kernels to 56 registers (9 blocks of 4
+// warps, or 18 of 2), one wave.  us per step with two warps: 80,802 particles 49.3 -> 42.0, 290^2 52.5 -> 44.9; with
+// one: 400^2 87.1 -> 75.7.  Elsewhere the 64 registers are the faster choice.
 template <int DIM, int SPLIT>
 inline bool tight(const pd_ctx* c, int block) {
-  return DIM == 2 && SPLIT == 2 && block <= kTightBlock && kTightBlock % block == 0 && tight_wave(c);
+  return DIM == 2 && SPLIT <= 2 && block <= kTightBlock && kTightBlock % block == 0 && tight_wave(c, SPLIT);
 }
 
 template <int DIM, int SPLIT>
@@ -2742,7 +2742,7 @@ void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, 
       k_pass1a_f64p<DIM, kSplit1aL, false>
           <<<slice_grid(c, kSplit1aL, kBlock1aL), kBlock1aL, 0, c->stream>>>(a, c->disp[c->cur]);
     else if (one_wave)
-      k_pass1a_f64p<DIM, SPLIT, DIM == 2 && SPLIT == 2><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
+      k_pass1a_f64p<DIM, SPLIT, DIM == 2 && SPLIT <= 2><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
     else
       k_pass1a_f64p<DIM, SPLIT, false><<<grid, block, 0, c->stream>>>(a, c->disp[c->cur]);
     if (c->profile) {
@@ -2756,7 +2756,7 @@ void launch_pass1(pd_ctx* c, const StepArgs& a, int write_theta, unsigned grid, 
     else if (c->vol_uniform)  // (within the tight wave's registers as it is)
       k_pass1b_f64p<DIM, SPLIT, true, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else if (one_wave)
-      k_pass1b_f64p<DIM, SPLIT, false, false, DIM == 2 && SPLIT == 2>
+      k_pass1b_f64p<DIM, SPLIT, false, false, DIM == 2 && SPLIT <= 2>
           <<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
     else
       k_pass1b_f64p<DIM, SPLIT, false, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], write_theta);
@@ -2785,7 +2785,7 @@ void launch_pass2(pd_ctx* c, const StepArgs& a, unsigned grid, int block, size_t
   else if (c->precision == PD_FP64 && a.bA && a.adr)
     k_pass2_f64t<DIM, SPLIT, true, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64 && a.bA && tight<DIM, SPLIT>(c, block))
-    k_pass2_f64t<DIM, SPLIT, false, DIM == 2 && SPLIT == 2>
+    k_pass2_f64t<DIM, SPLIT, false, DIM == 2 && SPLIT <= 2>
         <<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);
   else if (c->precision == PD_FP64 && a.bA)
     k_pass2_f64t<DIM, SPLIT, false, false><<<grid, block, sm, c->stream>>>(a, c->disp[c->cur], c->disp[c->cur ^ 1]);

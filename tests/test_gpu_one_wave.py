@@ -1,4 +1,4 @@
-"""FP64 plates of 32 to 36 warps per SM at two warps per slice, which the pass kernels take in one wave with 56 registers:
+"""FP64 plates of 32 to 36 warps per SM at one or two warps per slice, which the pass kernels take in one wave with 56 registers:
 bitwise the other mappings' states on both sides of the range, with breaking, uneven volumes, both forms of pass 1 and
 reads between steps (GPU only)."""
 import numpy as np
@@ -49,5 +49,18 @@ def test_plates_of_one_tight_wave(nx, ny, resident, uneven, pairs):
                     [(B.PD_OPT_BLOCK, 512), (B.PD_OPT_SPLIT, 2)]):
         path, got = _run(w, options, pairs=pairs)
         assert path == 0
+        for x, y in zip(got, want):
+            assert np.array_equal(x, y), options
+
+
+# the same with one warp per slice: 4,864 slices (the last with 64 registers in one wave), 4,901, 5,472 and 5,487
+@pytest.mark.parametrize("nx,ny", [(304, 512), (396, 396), (342, 512), (419, 419)])
+@pytest.mark.parametrize("uneven", [False, True])
+def test_plates_of_one_tight_wave_with_one_warp_per_slice(nx, ny, uneven):
+    w = _plate(nx, ny, uneven)
+    _, want = _run(w, [])
+    assert (want[-1] == 0).any()
+    for options in ([(B.PD_OPT_BLOCK, 64)], [(B.PD_OPT_BLOCK, 128)], [(B.PD_OPT_BLOCK, 256)]):
+        _, got = _run(w, options)
         for x, y in zip(got, want):
             assert np.array_equal(x, y), options
