@@ -156,8 +156,8 @@ pd_status ensure_xfer(pd_ctx* c) {
 
 // Brings the pages of a large output array into memory while the GPU still works on what was enqueued before
 // (their contents do not change).  A fresh allocation of that size has none yet, and the copy into it would
-// fault them in one by one after the GPU has finished (3.5M particles: 7.6 ms of a read, 50 steps and a read
-// 54.1 -> 50.6 ms; 1.2M particles of batched plates 12.3 -> 10.4 ms).  Best effort: an error changes nothing.
+// fault them in one by one after the GPU has finished (3.5M particles: 7.6 ms of a read; 50 steps and a read
+// 54.1 -> 50.6 ms).  Best effort: an error changes nothing.
 void populate(void* p, size_t bytes) {
   constexpr size_t kLeast = (size_t)4 << 20;
 #ifndef MADV_POPULATE_WRITE
@@ -651,6 +651,11 @@ pd_status pd_set_option(pd_ctx* c, int32_t option, int64_t value) {
       // other form never reads those marks, so a switch recomputes every bS before the next step.
       if ((value != 0) != (c->pairs != 0)) c->bs_stale = true;
       c->pairs = value != 0;
+      if (c->kin == PD_NONLINEAR && c->bA) {  // the other form's tables now, so that the next step may be captured
+        cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(c->stream, &cap) != cudaSuccess) cudaGetLastError();
+        else if (cap == cudaStreamCaptureStatusNone && ensure_bond_cache(c) != PD_OK) clear_error();  // the step reports it
+      }
       break;
     case PD_OPT_SOLVER:
       if (value != PD_SOLVER_EXPLICIT && value != PD_SOLVER_ADR) return fail(PD_ERR_ARG, "unknown solver");

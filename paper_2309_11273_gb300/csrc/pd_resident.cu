@@ -5,8 +5,8 @@
 // surrounds it: three launches, each with its ramp up and its last warps, and per launch the chain index ->
 // gather -> sum of a slice's row.  Here one block per SM holds its slices for the whole call; the
 // displacements and velocities of its particles stay in registers, and the passes are separated by a grid
-// barrier (about 1.3 us) instead of a launch: a 40 x 40 plate 33.7 -> 8.7 us per step (100 steps and a read), a
-// 400 x 160 plate 64 -> 36 us, bound there by the FP64 pipe (60 %) and the passes' ramps.  The arithmetic is that of
+// barrier (about 1.3 us) instead of a launch: a 40 x 40 plate 33.7 -> 8.6 us per step (100 steps and a read), a
+// 400 x 160 plate 63 -> 34 us, bound there by the FP64 pipe (60 %) and the passes' ramps.  The arithmetic is that of
 // k_pass1a_f64p / k_pass1b_f64p / k_pass2_f64t (pair form) or k_pass1_f64t / k_pass2_f64t, with the same
 // order of every sum (parts_sum), so the results are bitwise those of the pass kernels.
 #include <algorithm>

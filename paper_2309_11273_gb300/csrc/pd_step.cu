@@ -409,7 +409,9 @@ __device__ __forceinline__ double flip_sign(double x) {
 // breaks below that) both are their binomial series to degree 6, (sqrt(1 + t) - 1) / t and 1 / sqrt(1 + t)
 // cut below 2^-58 of their values: 12 FMAs, where the reciprocal square root and the division cost about
 // 25 FP64 instructions, which bound pass 1a.  A bond beyond that range takes the root and the division;
-// the choice is the bond's own, so its numbers do not depend on the warp it lands in.
+// the choice is the bond's own, so its numbers do not depend on the warp it lands in.  ms per step of a 101 x 50 x 49
+// block: every bond in the range 1.344, every one beyond (20 % stretch) 1.425, both in each warp 1.813, where the
+// root and the division alone took 2.15 throughout.
 __device__ __forceinline__ bool nl_small(double t) {
   return ((unsigned)__double2hiint(t) & 0x7fffffffu) < 0x3f700000u;  // |t| < 2^-8, false for a NaN
 }

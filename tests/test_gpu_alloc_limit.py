@@ -123,3 +123,26 @@ def test_no_room_for_the_resident_kernels_barrier(precision):
     sim.step(5)
     for x, y in zip(sim.state(), want):
         assert np.array_equal(x, y)
+
+
+def test_a_switched_nonlinear_form_may_be_captured_at_once():
+    import torch
+    stream = torch.cuda.Stream()
+
+    def make(**kw):
+        w = W.notched_block(12, 8, 7, nsteps=100, seed=5, amp=2e-8)
+        w.flag = w.axis_point = w.axis_dir = None
+        return Simulation(w, kinematics=PD_NONLINEAR, **kw)
+    ref, sim = make(), make(stream=stream.cuda_stream)
+    for s in (ref, sim):
+        s.step(2)
+        s.set_option(B.PD_OPT_PAIRS, 0)
+    ref.step(4)
+    sim.sync()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+        sim.step(4)
+    with torch.cuda.stream(stream):
+        g.replay()
+    for x, y in zip(sim.state(), ref.state()):
+        assert np.array_equal(x, y)
