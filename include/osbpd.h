@@ -138,10 +138,11 @@ typedef struct {
 typedef enum {
   PD_OPT_GRAPH_CHUNK = 1,  /* steps captured per CUDA graph launch (0: no graphs). Default 100.  Bodies
                               that fit the GPU in one wave (explicit solver; PD_FP64 with linearized
-                              bonds up to about 115,000 particles in 2D and 48,000 in 3D, PD_MIXED on
-                              the lattice layout up to 117,000) take all steps of a call in one cooperative
+                              bonds up to about 115,000 particles in 2D (but not 77,900 to 87,500) and
+                              48,000 in 3D, PD_MIXED on the lattice layout up to 117,000) take all steps of a call in one cooperative
                               launch instead, while no launch mapping was chosen (PD_OPT_BLOCK,
-                              PD_OPT_SPLIT, PD_OPT_LAT_STAGE); results are bitwise the same */
+                              PD_OPT_SPLIT, PD_OPT_LAT_STAGE) and PD_OPT_RESIDENT is 1; results are
+                              bitwise the same */
   PD_OPT_PROFILE = 2,      /* 1: time every kernel launch with CUDA events (forces eager launches) */
   PD_OPT_VALIDATE = 3,     /* PD_MIXED: 1 = also decide every bond in FP64 and count mismatches */
   PD_OPT_BLOCK = 4,        /* threads per block of the step kernels (multiple of 32, <= 512); until it or
